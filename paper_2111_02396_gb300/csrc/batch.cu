@@ -1417,11 +1417,11 @@ qt_status qt_batch_state(const qt_batch* b, uint32_t i, void* dst, size_t bytes)
   if (bytes < sb) return set_error(QT_ERR_INVALID_ARG, "qt_batch_state: %zu bytes < %zu", bytes, sb);
   // the kept state is un-normalized (deferred operators): normalize a device copy
   DevMem tmp, part;
-  if (!tmp.alloc(sb) || !part.alloc(scratch_partial_bytes() + sizeof(double) * 64))
+  if (!tmp.alloc(sb) || !part.alloc(sizeof(double) * (kPartialDoubles + kResultDoubles)))
     return set_error(QT_ERR_OUT_OF_MEMORY, "qt_batch_state: buffers");
   Scratch scr;
   scr.partial = static_cast<double*>(part.p);
-  scr.result = scr.partial + scratch_partial_bytes() / sizeof(double);
+  scr.result = scr.partial + kPartialDoubles;
   double N = 0.0;
   cudaError_t e = cudaMemcpy(tmp.p, static_cast<float2*>(b->arena.p) + T.arena_off, sb, cudaMemcpyDeviceToDevice);
   if (e == cudaSuccess) e = launch_expect(static_cast<const float2*>(tmp.p), static_cast<int>(T.n), 0, nullptr, scr, 0);

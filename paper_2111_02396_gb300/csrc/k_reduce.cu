@@ -2,51 +2,111 @@
 // Z-string expectations and bitstring sampling, plus state init / scale.
 //
 // Precision: products are formed in FP32 from the complex64 state; partial
-// sums over a short run of terms stay in FP32 and are then carried in FP64
-// (FP64 throughput on this part is low, so it is used only at that coarse
-// grain).  Every reduction has a fixed grid and a fixed combination order,
+// sums over a short run of terms stay in FP32 and are then carried in
+// double-floats (qt_dfloat.h: FP64 throughput on this part is low) and leave
+// as FP64.  Every reduction has a fixed grid and a fixed combination order,
 // so results are bitwise reproducible run to run.
 #include <cuda_runtime.h>
 
 #include <mutex>
 
 #include "kernels.h"
+#include "qt_dfloat.h"
 #include "qt_philox.h"
 
 namespace qt {
 
-size_t scratch_partial_bytes() { return sizeof(double) * kMaxRedBlocks * 64; }
+// A dependent launch: its blocks may become resident while the kernel before
+// it on the stream still runs, and wait there (cudaGridDependencySynchronize)
+// for that kernel's results.  The short kernels that follow a reduction start
+// without a launch gap this way.
+template <typename... P, typename... A>
+static cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, unsigned block, cudaStream_t st, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
 
 // ---------------------------------------------------------------------------
-// block-wide FP64 reduction of W per-thread values into partial[block][W]
+// block-wide sums of W per-thread double-floats into partial[block][W]
 // ---------------------------------------------------------------------------
 template <int W>
-__device__ __forceinline__ void block_reduce_store(double (&acc)[W], double* __restrict__ partial) {
-  __shared__ double sm[kRedThreads / 32][W];
+__device__ __forceinline__ void block_reduce_store(const float (&h)[W], const float (&l)[W],
+                                                   float2* __restrict__ partial) {
+  constexpr int P = W >= 16 ? 16 : (W >= 4 ? 4 : 2), REST = W - P;   // one transposed group and the rest
+  __shared__ float2 sm[kRedThreads / 32][W];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float2 v[P];
 #pragma unroll
-  for (int c = 0; c < W; ++c) {
-    double v = acc[c];
+  for (int c = 0; c < P; ++c) v[c] = make_float2(h[c], l[c]);
+  const float2 s = df_warp_sum<P>(v, lane);
+  constexpr int per = 32 / P;                          // lanes that hold the same sum
+  if (lane % per == 0) sm[warp][lane / per] = s;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) sm[warp][c] = v;
+  for (int c = W - REST; c < W; ++c) {
+    float2 r = make_float2(h[c], l[c]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) r = df_add(r, df_shfl_xor(r, o));
+    if (lane == 0) sm[warp][c] = r;
   }
   __syncthreads();
-  const int nw = static_cast<int>(blockDim.x >> 5);   // blocks of at most kRedThreads threads
+  const int nw = static_cast<int>(blockDim.x >> 5);    // blocks of at most kRedThreads threads
   for (int c = threadIdx.x; c < W; c += blockDim.x) {
-    double v = 0.0;
-    for (int w = 0; w < nw; ++w) v += sm[w][c];
-    partial[static_cast<size_t>(blockIdx.x) * W + c] = v;
+    float2 r = make_float2(0.f, 0.f);
+    for (int w = 0; w < nw; ++w) r = df_add(r, sm[w][c]);
+    partial[static_cast<size_t>(blockIdx.x) * W + c] = r;
   }
 }
 
-__global__ void k_finalize(const double* __restrict__ partial, int nblocks, int W,
-                           double* __restrict__ out) {
-  for (int c = threadIdx.x; c < W; c += blockDim.x) {
-    double v = 0.0;
-    for (int b = 0; b < nblocks; ++b) v += partial[static_cast<size_t>(b) * W + c];
-    out[c] = v;
+// out[c] = sum over blocks of partial[block][c].  CB columns per block of 1024
+// threads, 1024 / CB of them per column: a handful of independent loads each
+// at the largest grid.  (One thread per column chained up to 1216 FP64 adds:
+// 55 us after a 29-qubit pass, 14 after a 17-qubit one, now 4 and 3.)
+constexpr int kSumThreads = 1024;
+
+template <int CB>
+__device__ __forceinline__ float2 column_sum(const float2* partial, int nblocks, int W, int col) {
+  constexpr int SL = kSumThreads / CB;
+  __shared__ float2 sm[SL][CB];
+  const int cl = threadIdx.x % CB, sl = threadIdx.x / CB;
+  float2 r = make_float2(0.f, 0.f);
+  if (col < W) {
+#pragma unroll 4
+    for (int b = sl; b < nblocks; b += SL) r = df_add(r, partial[static_cast<size_t>(b) * W + col]);
   }
+  // lanes of a warp that hold the same column, then the warps
+  if constexpr (CB < 32) {
+#pragma unroll
+    for (int o = CB; o < 32; o <<= 1) r = df_add(r, df_shfl_xor(r, o));
+  }
+  constexpr int PER = CB < 32 ? 32 / CB : 1;             // slices of a warp
+  if (sl % PER == 0) sm[sl / PER][cl] = r;
+  __syncthreads();
+#pragma unroll
+  for (int o = SL / PER / 2; o > 0; o >>= 1) {
+    if (sl < o) sm[sl][cl] = df_add(sm[sl][cl], sm[sl + o][cl]);
+    __syncthreads();
+  }
+  return sm[0][cl];
+}
+
+template <int CB>
+__global__ void __launch_bounds__(kSumThreads) k_finalize(const float2* partial, int nblocks, int W, double* out) {
+  cudaGridDependencySynchronize();
+  const int col = blockIdx.x * CB + threadIdx.x % CB;
+  const float2 r = column_sum<CB>(partial, nblocks, W, col);
+  if (threadIdx.x < CB && col < W) out[col] = df_value(r);
+}
+
+static cudaError_t finalize(const float2* partial, int nblocks, int W, double* out, cudaStream_t st) {
+  return launch_dependent(k_finalize<4>, dim3((W + 3) / 4), kSumThreads, st, partial, nblocks, W, out);
 }
 
 template <typename Kern>
@@ -64,85 +124,294 @@ static int red_grid(Kern kern, uint64_t work_items) {
 }
 
 // ---------------------------------------------------------------------------
-// Reduced density block of qubits Q: rho[b][a] = sum_rest psi[rest,b] conj(psi[rest,a]).
-// W = 4^q reals: the 2^q diagonal entries, then (re, im) of each b < a.
+// Reduced density block of qubits Q: rho[b][a] = sum_rest psi[rest,b] conj(psi[rest,a]),
+// with basis bit j = the j-th lowest qubit (the callers reorder).
+//
+// q = 1, 2 (k_rdm): every entry in registers, W = 4^q reals: the 2^q diagonal
+// entries, then (re, im) of each b < a.  Bound by HBM: a thread keeps 8
+// 128-bit loads in flight (LOW0: qubit 0 is in Q, so members 2j and 2j + 1 of
+// a set share a load; otherwise two neighbouring sets do).  n = 29: q = 1
+// 654 -> 634 us, q = 2 834 -> 686 us (one set of 8-byte loads at a time and FP64
+// carries before); 4 GiB read at the copy rate take 634.
 // ---------------------------------------------------------------------------
 template <int Q>
 struct RdmArgs {
-  uint64_t offs[1 << Q];
-  uint32_t ins[Q];
-  uint64_t num_sets;
+  uint64_t offs[1 << Q];      // 128-bit word offset of load m within a group
+  uint32_t ins[Q + 1];        // ascending bit positions to insert zeros at
+  uint64_t num_groups;
 };
 
-constexpr int kRdmChunk = 16;   // sets summed in FP32 before the FP64 carry
+// Sets summed in FP32 before the carry: 16, and every set by itself (FINE)
+// where there are fewer than 2^20 of them.  The rounding of a run of R sets
+// leaves about R / sqrt(3 sets) * 3e-8 of an entry: 3e-10 at 2^20 sets with
+// R = 16, but it no longer averages out in small states.
+constexpr int kRdmChunk = 16;
+constexpr int kRdmFineLog = 20;
 
-template <int Q>
-__global__ void __launch_bounds__(kRedThreads) k_rdm(const float2* __restrict__ psi,
+template <int Q, bool LOW0, bool FINE>
+__global__ void __launch_bounds__(kRedThreads) k_rdm(const float4* __restrict__ psi,
                                                      const __grid_constant__ RdmArgs<Q> a,
-                                                     double* __restrict__ partial) {
+                                                     float2* __restrict__ partial) {
   constexpr int D = 1 << Q, W = D * D;
-  double acc[W];
-  float f[W];
+  constexpr int NV = LOW0 ? D / 2 : D;        // loads per group
+  constexpr int SPG = LOW0 ? 1 : 2;           // sets per group
+  constexpr int NI = LOW0 ? Q : Q + 1;        // zeros inserted into the group index
+  constexpr int U = 8 / NV;                   // groups in flight
+  cudaTriggerProgrammaticLaunchCompletion();
+  float h[W], l[W], f[W];
 #pragma unroll
-  for (int c = 0; c < W; ++c) { acc[c] = 0.0; f[c] = 0.f; }
+  for (int c = 0; c < W; ++c) { h[c] = 0.f; l[c] = 0.f; f[c] = 0.f; }
   int cnt = 0;
   const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x;
-  for (uint64_t i = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < a.num_sets;
-       i += stride) {
-    uint64_t base = i;
+  for (uint64_t i = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < a.num_groups;
+       i += U * stride) {
+    float4 v[U][NV];
 #pragma unroll
-    for (int b = 0; b < Q; ++b) {
-      const uint32_t s = a.ins[b];
-      base = ((base >> s) << (s + 1)) | (base & ((1ull << s) - 1ull));
-    }
-    float2 v[D];
+    for (int u = 0; u < U; ++u) {
+      const uint64_t g = i + u * stride;
+      uint64_t base = g;
 #pragma unroll
-    for (int m = 0; m < D; ++m) v[m] = __ldg(psi + base + a.offs[m]);
-    int c = 0;
-#pragma unroll
-    for (int b = 0; b < D; ++b) { f[c] = fmaf(v[b].x, v[b].x, fmaf(v[b].y, v[b].y, f[c])); ++c; }
-#pragma unroll
-    for (int b = 0; b < D; ++b)
-#pragma unroll
-      for (int aa = b + 1; aa < D; ++aa) {
-        // v_b conj(v_a)
-        f[c] = fmaf(v[b].x, v[aa].x, fmaf(v[b].y, v[aa].y, f[c])); ++c;
-        f[c] = fmaf(v[b].y, v[aa].x, fmaf(-v[b].x, v[aa].y, f[c])); ++c;
+      for (int b = 0; b < NI; ++b) {
+        const uint32_t s = a.ins[b];
+        base = ((base >> s) << (s + 1)) | (base & ((1ull << s) - 1ull));
       }
-    if (++cnt == kRdmChunk) {
 #pragma unroll
-      for (int k = 0; k < W; ++k) { acc[k] += static_cast<double>(f[k]); f[k] = 0.f; }
+      for (int m = 0; m < NV; ++m)
+        v[u][m] = g < a.num_groups ? __ldg(psi + (base >> 1) + a.offs[m]) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int s = 0; s < SPG; ++s) {
+        float2 x[D];
+#pragma unroll
+        for (int m = 0; m < D; ++m) {
+          const float4 w = v[u][LOW0 ? m / 2 : m];
+          const bool second = LOW0 ? (m & 1) : s == 1;
+          x[m] = second ? make_float2(w.z, w.w) : make_float2(w.x, w.y);
+        }
+        int c = 0;
+#pragma unroll
+        for (int b = 0; b < D; ++b) { f[c] = fmaf(x[b].x, x[b].x, fmaf(x[b].y, x[b].y, f[c])); ++c; }
+#pragma unroll
+        for (int b = 0; b < D; ++b)
+#pragma unroll
+          for (int aa = b + 1; aa < D; ++aa) {
+            // x_b conj(x_a)
+            f[c] = fmaf(x[b].x, x[aa].x, fmaf(x[b].y, x[aa].y, f[c])); ++c;
+            f[c] = fmaf(x[b].y, x[aa].x, fmaf(-x[b].x, x[aa].y, f[c])); ++c;
+          }
+        if constexpr (FINE) {
+#pragma unroll
+          for (int k = 0; k < W; ++k) { df_acc(h[k], l[k], f[k]); f[k] = 0.f; }
+        }
+      }
+    cnt += U * SPG;
+    if (!FINE && cnt == kRdmChunk) {
+#pragma unroll
+      for (int k = 0; k < W; ++k) { df_acc(h[k], l[k], f[k]); f[k] = 0.f; }
       cnt = 0;
     }
   }
+  if constexpr (!FINE) {
 #pragma unroll
-  for (int k = 0; k < W; ++k) acc[k] += static_cast<double>(f[k]);
-  block_reduce_store<W>(acc, partial);
+    for (int k = 0; k < W; ++k) df_acc(h[k], l[k], f[k]);
+  }
+  block_reduce_store<W>(h, l, partial);
 }
 
+// sorted copy of q qubits
 template <int Q>
-static cudaError_t rdm_q(const float2* psi, int n, const uint32_t* qubits, const Scratch& scr,
-                         cudaStream_t st) {
-  RdmArgs<Q> a;
-  uint32_t s[Q];
+static void sort_qubits(const uint32_t* qubits, uint32_t* s) {
   for (int b = 0; b < Q; ++b) s[b] = qubits[b];
   for (int i = 1; i < Q; ++i)
     for (int j = i; j > 0 && s[j - 1] > s[j]; --j) { const uint32_t t = s[j]; s[j] = s[j - 1]; s[j - 1] = t; }
-  for (int b = 0; b < Q; ++b) a.ins[b] = s[b];
+}
+
+template <int Q, bool LOW0, bool FINE>
+static cudaError_t rdm_low(const float2* psi, int n, const uint32_t* s, const Scratch& scr, cudaStream_t st) {
+  constexpr int U = 8 / (LOW0 ? (1 << Q) / 2 : (1 << Q));
+  RdmArgs<Q> a{};
+  int ni = 0;
+  if (!LOW0) a.ins[ni++] = 0;
+  for (int b = 0; b < Q; ++b) a.ins[ni++] = s[b];
   for (int m = 0; m < (1 << Q); ++m) {
     uint64_t o = 0;
+    const int mem = LOW0 ? 2 * m : m;            // the even member of load m
     for (int b = 0; b < Q; ++b)
-      if ((m >> b) & 1) o |= 1ull << qubits[b];
-    a.offs[m] = o;
+      if ((mem >> b) & 1) o |= 1ull << s[b];
+    a.offs[m] = o >> 1;
   }
-  a.num_sets = 1ull << (n - Q);
+  a.num_groups = 1ull << (n - Q - (LOW0 ? 0 : 1));
   static PerDevice grid_dev;
-  const int grid = grid_dev.get([] { return red_grid(k_rdm<Q>, ~0ull >> 1); });
-  const uint64_t need = (a.num_sets + kRedThreads - 1) / kRedThreads;
+  const int grid = grid_dev.get([] { return red_grid(k_rdm<Q, LOW0, FINE>, ~0ull >> 1); });
+  const uint64_t per = static_cast<uint64_t>(kRedThreads) * U;
+  const uint64_t need = (a.num_groups + per - 1) / per;
   const int g = static_cast<int>(need < static_cast<uint64_t>(grid) ? need : grid);
-  k_rdm<Q><<<g, kRedThreads, 0, st>>>(psi, a, scr.partial);
-  k_finalize<<<1, 64, 0, st>>>(scr.partial, g, 1 << (2 * Q), scr.result);
-  return cudaGetLastError();
+  k_rdm<Q, LOW0, FINE><<<g, kRedThreads, 0, st>>>(reinterpret_cast<const float4*>(psi), a, scr.partials());
+  return finalize(scr.partials(), g, 1 << (2 * Q), scr.result, st);
+}
+
+// ---------------------------------------------------------------------------
+// q = 3 (k_rdm3): 64 reals do not fit one thread with their carries, so a pair
+// of lanes (l, l ^ 16) shares a group: each loads the four members with its
+// value of the highest qubit, gets the other four by shuffles, and sums half
+// of the block: the triangle over its own members (16 reals) and two columns
+// of the 4 x 4 corner between the halves (16 reals).  The carries sit in
+// shared memory, which leaves the registers to loads in flight.
+// n = 29: 1856 -> 936 us (64 FP64 accumulators a thread, 8 warps an SM).
+// ---------------------------------------------------------------------------
+struct Rdm3Args {
+  uint64_t offs[4];           // 128-bit word offset of load m of the half-group
+  uint64_t half;              // 128-bit word offset of the upper half
+  uint32_t ins[4];            // ascending bit positions to insert zeros at
+  uint64_t num_groups;
+  int run;                    // sets summed in FP32 before the carry
+};
+
+constexpr int kRdm3Threads = 128;
+
+template <bool LOW0>
+__global__ void __launch_bounds__(kRdm3Threads, 4) k_rdm3(const float4* __restrict__ psi, const __grid_constant__ Rdm3Args a,
+                                                          float2* __restrict__ partial) {
+  constexpr int NV = LOW0 ? 2 : 4;            // loads per half-group
+  constexpr int SPG = LOW0 ? 1 : 2;           // sets per group
+  constexpr int NI = LOW0 ? 3 : 4;
+  constexpr int U = LOW0 ? 4 : 2;             // groups in flight
+  __shared__ float2 carry[32][kRdm3Threads];
+  cudaTriggerProgrammaticLaunchCompletion();
+  const int tid = threadIdx.x;
+  const bool upper = tid & 16;
+  float f[32];
+#pragma unroll
+  for (int k = 0; k < 32; ++k) { f[k] = 0.f; carry[k][tid] = make_float2(0.f, 0.f); }
+  int run = 0;
+  auto flush = [&] {
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+      float2 c = carry[k][tid];
+      df_acc(c.x, c.y, f[k]);
+      carry[k][tid] = c;
+      f[k] = 0.f;
+    }
+  };
+  // pairs of lanes: pair index within the grid
+  const uint64_t pair = (static_cast<uint64_t>(blockIdx.x) * kRdm3Threads + tid) >> 5 << 4 | (tid & 15);
+  const uint64_t stride = static_cast<uint64_t>(gridDim.x) * (kRdm3Threads / 2);
+  const uint64_t first = pair - (tid & 15);   // of the warp: the loop is uniform over it
+  for (uint64_t w0 = first; w0 < a.num_groups; w0 += U * stride) {
+    float4 v[U][NV];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const uint64_t g = w0 + (tid & 15) + u * stride;
+      uint64_t base = g;
+#pragma unroll
+      for (int b = 0; b < NI; ++b) {
+        const uint32_t s = a.ins[b];
+        base = ((base >> s) << (s + 1)) | (base & ((1ull << s) - 1ull));
+      }
+      base >>= 1;
+      if (upper) base += a.half;
+#pragma unroll
+      for (int m = 0; m < NV; ++m)
+        v[u][m] = g < a.num_groups ? __ldg(psi + base + a.offs[m]) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int s = 0; s < SPG; ++s) {
+        float2 own[4], x[4], y[2];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          const float4 w = v[u][LOW0 ? m / 2 : m];
+          const bool second = LOW0 ? (m & 1) : s == 1;
+          own[m] = second ? make_float2(w.z, w.w) : make_float2(w.x, w.y);
+        }
+        // corner: rows = the upper half's members, columns 0, 1 (lower lanes)
+        // or 2, 3 (upper lanes) of the lower half's
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          const float2 o = make_float2(__shfl_xor_sync(0xffffffffu, own[m].x, 16), __shfl_xor_sync(0xffffffffu, own[m].y, 16));
+          x[m] = upper ? own[m] : o;
+          if (m < 2 && !upper) y[m] = own[m];
+          if (m >= 2 && upper) y[m - 2] = o;
+        }
+        int c = 0;
+#pragma unroll
+        for (int b = 0; b < 4; ++b) { f[c] = fmaf(own[b].x, own[b].x, fmaf(own[b].y, own[b].y, f[c])); ++c; }
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+#pragma unroll
+          for (int aa = b + 1; aa < 4; ++aa) {
+            f[c] = fmaf(own[b].x, own[aa].x, fmaf(own[b].y, own[aa].y, f[c])); ++c;
+            f[c] = fmaf(own[b].y, own[aa].x, fmaf(-own[b].x, own[aa].y, f[c])); ++c;
+          }
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            // y_q conj(x_p)
+            f[c] = fmaf(y[q].x, x[p].x, fmaf(y[q].y, x[p].y, f[c])); ++c;
+            f[c] = fmaf(y[q].y, x[p].x, fmaf(-y[q].x, x[p].y, f[c])); ++c;
+          }
+        if (++run == a.run) { flush(); run = 0; }
+      }
+  }
+  flush();
+  __syncthreads();
+  // value (half, k): sum over the half's 64 threads, by two threads of 32
+  __shared__ float2 part[kRdm3Threads];
+  const int o = tid & 63, k = o & 31, hf = o >> 5, which = tid >> 6;
+  float2 sum = make_float2(0.f, 0.f);
+  for (int i = 0; i < 32; ++i) {
+    const int j = which * 32 + ((i + tid) & 31);           // rotated: neighbouring threads read other banks
+    sum = df_add(sum, carry[k][(j >> 4 << 5) | (hf << 4) | (j & 15)]);
+  }
+  part[tid] = sum;
+  __syncthreads();
+  if (tid < 64) partial[static_cast<size_t>(blockIdx.x) * 64 + tid] = df_add(part[tid], part[tid + 64]);
+}
+
+// sets summed in FP32 before the carry: the bound given at kRdmChunk
+static int carry_run(double scale, int log_sets, int cap) {
+  const double r = scale * exp2(0.5 * log_sets);
+  return r < 1.0 ? 1 : (r > cap ? cap : static_cast<int>(r));
+}
+
+template <bool LOW0>
+static cudaError_t rdm3_low(const float2* psi, int n, const uint32_t* s, const Scratch& scr, cudaStream_t st) {
+  Rdm3Args a{};
+  int ni = 0;
+  if (!LOW0) a.ins[ni++] = 0;
+  for (int b = 0; b < 3; ++b) a.ins[ni++] = s[b];
+  for (int m = 0; m < 4; ++m) {
+    const int mem = LOW0 ? (2 * m) & 3 : m;                // the even member of load m
+    a.offs[m] = ((mem & 1 ? 1ull << s[0] : 0) | (mem & 2 ? 1ull << s[1] : 0)) >> 1;
+  }
+  a.half = (1ull << s[2]) >> 1;
+  a.num_groups = 1ull << (n - 3 - (LOW0 ? 0 : 1));
+  a.run = carry_run(0.01, n - 3, kRdmChunk);
+  static PerDevice grid_dev;
+  const int grid = grid_dev.get([] {
+    int occ = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_rdm3<LOW0>, kRdm3Threads, 0);
+    return sm_count() * (occ > 0 ? occ : 1);
+  });
+  const uint64_t per = static_cast<uint64_t>(kRdm3Threads / 2) * (LOW0 ? 4 : 2);
+  uint64_t g = (a.num_groups + per - 1) / per;
+  if (g > static_cast<uint64_t>(grid)) g = grid;
+  if (g > static_cast<uint64_t>(kPartialDoubles / 64)) g = kPartialDoubles / 64;
+  k_rdm3<LOW0><<<static_cast<unsigned>(g), kRdm3Threads, 0, st>>>(reinterpret_cast<const float4*>(psi), a, scr.partials());
+  return finalize(scr.partials(), static_cast<int>(g), 64, scr.result, st);
+}
+
+template <int Q>
+static cudaError_t rdm_q(const float2* psi, int n, const uint32_t* qubits, const Scratch& scr, cudaStream_t st) {
+  uint32_t s[Q];
+  sort_qubits<Q>(qubits, s);
+  if (n - Q < kRdmFineLog)
+    return s[0] == 0 ? rdm_low<Q, true, true>(psi, n, s, scr, st) : rdm_low<Q, false, true>(psi, n, s, scr, st);
+  return s[0] == 0 ? rdm_low<Q, true, false>(psi, n, s, scr, st) : rdm_low<Q, false, false>(psi, n, s, scr, st);
 }
 
 cudaError_t launch_rdm(const float2* psi, int n, int q, const uint32_t* qubits, const Scratch& scr,
@@ -151,22 +420,62 @@ cudaError_t launch_rdm(const float2* psi, int n, int q, const uint32_t* qubits, 
   switch (q) {
     case 1: return rdm_q<1>(psi, n, qubits, scr, st);
     case 2: return rdm_q<2>(psi, n, qubits, scr, st);
-    case 3: return rdm_q<3>(psi, n, qubits, scr, st);
+    case 3: {
+      uint32_t s[3];
+      sort_qubits<3>(qubits, s);
+      return s[0] == 0 ? rdm3_low<true>(psi, n, s, scr, st) : rdm3_low<false>(psi, n, s, scr, st);
+    }
     default: return cudaErrorInvalidValue;
   }
+}
+
+void rdm_unpack(int q, const uint32_t* qubits, const double* r, double* rho) {
+  const int D = 1 << q;
+  // basis index over `qubits` of basis index x over the sorted qubits
+  auto user = [&](int x) {
+    int u = 0;
+    for (int b = 0; b < q; ++b) {
+      int pos = 0;
+      for (int k = 0; k < q; ++k) pos += qubits[k] < qubits[b];
+      u |= ((x >> pos) & 1) << b;
+    }
+    return u;
+  };
+  auto put = [&](int sb, int sa, double re, double im) {   // rho[b][a] = sum psi_b conj(psi_a), Hermitian
+    const int b = user(sb), a = user(sa);
+    rho[2 * (b * D + a)] = re;
+    rho[2 * (b * D + a) + 1] = im;
+    rho[2 * (a * D + b)] = re;
+    rho[2 * (a * D + b) + 1] = a == b ? im : -im;
+  };
+  if (q == 3) {                                            // per half: its triangle, two columns of the corner
+    for (int h = 0; h < 2; ++h, r += 32) {
+      for (int b = 0; b < 4; ++b) put(4 * h + b, 4 * h + b, r[b], 0.0);
+      int c = 4;
+      for (int b = 0; b < 4; ++b)
+        for (int a = b + 1; a < 4; ++a, c += 2) put(4 * h + b, 4 * h + a, r[c], r[c + 1]);
+      for (int p = 0; p < 4; ++p)
+        for (int k = 0; k < 2; ++k, c += 2) put(2 * h + k, 4 + p, r[c], r[c + 1]);
+    }
+    return;
+  }
+  int c = 0;
+  for (int b = 0; b < D; ++b) put(b, b, r[c++], 0.0);
+  for (int b = 0; b < D; ++b)
+    for (int a = b + 1; a < D; ++a) {
+      const double re = r[c++], im = r[c++];
+      put(b, a, re, im);
+    }
 }
 
 // ---------------------------------------------------------------------------
 // Branch probabilities of a channel on 4..6 qubits (Alg. 2 step 14): for G
 // Kraus operators at a time, P_i = <psi|K_i^dag K_i|psi> = sum over gather
-// sets of |K_i v|^2, plus N = <psi|psi> (the 4^q-entry reduced density of
-// these widths would not fit in registers).  Each thread takes whole gather
-// sets; its set is staged column-wise in shared memory (member m of thread t
-// at v[m * blockDim + t], conflict-free) and the G operators sit in shared
-// memory.  Products and row sums in FP32; runs of kKrausChunk sets in FP32,
-// carried in FP64; fixed grid and reduction order.
+// sets of |K_i v|^2, plus N = <psi|psi>.  Each thread takes whole gather sets, staged
+// column-wise in shared memory (member m of thread t at v[m * blockDim + t],
+// conflict-free), with the G operators in shared memory.  Products and row
+// sums in FP32; runs of kKrausChunk sets in FP32, carried in double-floats.
 // result[0] = N, result[1 + i] = P_i.
-// ---------------------------------------------------------------------------
 constexpr int kKrausThreads = 128;
 constexpr int kKrausChunk = 16;
 
@@ -181,17 +490,17 @@ struct KrausArgs {
 template <int Q, int G>
 __global__ void __launch_bounds__(kKrausThreads) k_kraus_norms(const float2* __restrict__ psi,
                                                                const __grid_constant__ KrausArgs<Q> a,
-                                                               double* __restrict__ partial) {
+                                                               float2* __restrict__ partial) {
   constexpr int D = 1 << Q, W = G + 1;
   extern __shared__ __align__(16) float2 s_dyn[];
   float2* sK = s_dyn;                          // G * D * D
   float2* sv = s_dyn + G * D * D;              // D * blockDim
+  cudaTriggerProgrammaticLaunchCompletion();
   for (int i = threadIdx.x; i < G * D * D; i += blockDim.x) sK[i] = a.ops[i];
   __syncthreads();
-  double acc[W];
-  float f[W];
+  float ah[W], al[W], f[W];
 #pragma unroll
-  for (int c = 0; c < W; ++c) { acc[c] = 0.0; f[c] = 0.f; }
+  for (int c = 0; c < W; ++c) { ah[c] = 0.f; al[c] = 0.f; f[c] = 0.f; }
   int cnt = 0;
   const int t = threadIdx.x, bd = blockDim.x;
   const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x;
@@ -227,13 +536,13 @@ __global__ void __launch_bounds__(kKrausThreads) k_kraus_norms(const float2* __r
     }
     if (++cnt == kKrausChunk) {
 #pragma unroll
-      for (int k = 0; k < W; ++k) { acc[k] += static_cast<double>(f[k]); f[k] = 0.f; }
+      for (int k = 0; k < W; ++k) { df_acc(ah[k], al[k], f[k]); f[k] = 0.f; }
       cnt = 0;
     }
   }
 #pragma unroll
-  for (int k = 0; k < W; ++k) acc[k] += static_cast<double>(f[k]);
-  block_reduce_store<W>(acc, partial);
+  for (int k = 0; k < W; ++k) df_acc(ah[k], al[k], f[k]);
+  block_reduce_store<W>(ah, al, partial);
 }
 
 template <int Q, int G>
@@ -268,9 +577,8 @@ static cudaError_t kraus_norms_q(const float2* psi, int n, const uint32_t* qubit
   if (grid <= 0) return cudaErrorInvalidConfiguration;
   const uint64_t need = (a.num_sets + kKrausThreads - 1) / kKrausThreads;
   const int g = static_cast<int>(need < static_cast<uint64_t>(grid) ? need : grid);
-  k_kraus_norms<Q, G><<<g, kKrausThreads, smem, st>>>(psi, a, scr.partial);
-  k_finalize<<<1, 64, 0, st>>>(scr.partial, g, G + 1, scr.result);
-  return cudaGetLastError();
+  k_kraus_norms<Q, G><<<g, kKrausThreads, smem, st>>>(psi, a, scr.partials());
+  return finalize(scr.partials(), g, G + 1, scr.result, st);
 }
 
 int kraus_group(int q) { return q <= 4 ? 16 : (q == 5 ? 4 : 1); }
@@ -286,23 +594,6 @@ cudaError_t launch_kraus_norms(const float2* psi, int n, int q, const uint32_t* 
   }
 }
 
-void rdm_unpack(int q, const double* r, double* rho) {
-  const int D = 1 << q;
-  int c = 0;
-  for (int b = 0; b < D; ++b) {
-    rho[2 * (b * D + b)] = r[c++];
-    rho[2 * (b * D + b) + 1] = 0.0;
-  }
-  for (int b = 0; b < D; ++b)
-    for (int a = b + 1; a < D; ++a) {
-      const double re = r[c++], im = r[c++];
-      rho[2 * (b * D + a)] = re;        // rho[b][a] = sum psi_b conj(psi_a)
-      rho[2 * (b * D + a) + 1] = im;
-      rho[2 * (a * D + b)] = re;        // Hermitian
-      rho[2 * (a * D + b) + 1] = -im;
-    }
-}
-
 // ---------------------------------------------------------------------------
 // Z-string expectations: result[0] = N, result[1+m] = sum_x |psi_x|^2 (-1)^popc(x & mask_m)
 // ---------------------------------------------------------------------------
@@ -316,12 +607,12 @@ constexpr int kExpChunk = 64;
 
 __global__ void __launch_bounds__(kRedThreads) k_expect(const float2* __restrict__ psi,
                                                         const __grid_constant__ ExpArgs a,
-                                                        double* __restrict__ partial) {
+                                                        float2* __restrict__ partial) {
   constexpr int W = kExpGroup + 1;
-  double acc[W];
-  float f[W];
+  cudaTriggerProgrammaticLaunchCompletion();
+  float ah[W], al[W], f[W];
 #pragma unroll
-  for (int c = 0; c < W; ++c) { acc[c] = 0.0; f[c] = 0.f; }
+  for (int c = 0; c < W; ++c) { ah[c] = 0.f; al[c] = 0.f; f[c] = 0.f; }
   int cnt = 0;
   const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x;
   for (uint64_t i = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < a.num_pairs;
@@ -341,13 +632,13 @@ __global__ void __launch_bounds__(kRedThreads) k_expect(const float2* __restrict
     }
     if (++cnt == kExpChunk) {
 #pragma unroll
-      for (int k = 0; k < W; ++k) { acc[k] += static_cast<double>(f[k]); f[k] = 0.f; }
+      for (int k = 0; k < W; ++k) { df_acc(ah[k], al[k], f[k]); f[k] = 0.f; }
       cnt = 0;
     }
   }
 #pragma unroll
-  for (int k = 0; k < W; ++k) acc[k] += static_cast<double>(f[k]);
-  block_reduce_store<W>(acc, partial);
+  for (int k = 0; k < W; ++k) df_acc(ah[k], al[k], f[k]);
+  block_reduce_store<W>(ah, al, partial);
 }
 
 // n >= 9: a warp takes blocks of 512 amplitudes and lane l holds the 16
@@ -360,7 +651,7 @@ __global__ void __launch_bounds__(kRedThreads) k_expect(const float2* __restrict
 // 8.  The parity over the lane bits (1..5) is fixed per thread and the one
 // over the block bits (>= 9) is one popc, so a mask costs a few instructions
 // per 16 amplitudes.  FP32 runs cover 8 blocks (128 amplitudes per thread),
-// then FP64.
+// then a carry.
 struct ExpWArgs {
   uint32_t mblk[kExpGroup];     // mask bits >= 9, shifted down by 9
   uint32_t mlane[kExpGroup];    // mask bits 1..5, shifted down by 1
@@ -373,13 +664,13 @@ constexpr int kExpWChunk = 8;
 
 __global__ void __launch_bounds__(kRedThreads) k_expect_wht(const float2* __restrict__ psi,
                                                             const __grid_constant__ ExpWArgs a,
-                                                            double* __restrict__ partial) {
+                                                            float2* __restrict__ partial) {
   constexpr int W = kExpGroup + 1;
   __shared__ float s_w[kRedThreads][17];        // each thread's transformed weights (padded row)
-  double acc[W];
-  float f[W];
+  cudaTriggerProgrammaticLaunchCompletion();
+  float ah[W], al[W], f[W];
 #pragma unroll
-  for (int c = 0; c < W; ++c) { acc[c] = 0.0; f[c] = 0.f; }
+  for (int c = 0; c < W; ++c) { ah[c] = 0.f; al[c] = 0.f; f[c] = 0.f; }
   const uint32_t lane = threadIdx.x & 31u;
   const uint64_t warp = (static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const uint64_t nwarps = (static_cast<uint64_t>(gridDim.x) * blockDim.x) >> 5;
@@ -428,13 +719,13 @@ __global__ void __launch_bounds__(kRedThreads) k_expect_wht(const float2* __rest
     }
     if (++cnt == kExpWChunk) {
 #pragma unroll
-      for (int k = 0; k < W; ++k) { acc[k] += static_cast<double>(f[k]); f[k] = 0.f; }
+      for (int k = 0; k < W; ++k) { df_acc(ah[k], al[k], f[k]); f[k] = 0.f; }
       cnt = 0;
     }
   }
 #pragma unroll
-  for (int k = 0; k < W; ++k) acc[k] += static_cast<double>(f[k]);
-  block_reduce_store<W>(acc, partial);
+  for (int k = 0; k < W; ++k) df_acc(ah[k], al[k], f[k]);
+  block_reduce_store<W>(ah, al, partial);
 }
 
 cudaError_t launch_expect(const float2* psi, int n, int nm, const uint64_t* masks,
@@ -454,9 +745,8 @@ cudaError_t launch_expect(const float2* psi, int n, int nm, const uint64_t* mask
     const int gridw = gridw_dev.get([] { return red_grid(k_expect_wht, ~0ull >> 1); });
     const uint64_t need = (a.num_blocks * 32 + kRedThreads - 1) / kRedThreads;
     const int g = static_cast<int>(need < static_cast<uint64_t>(gridw) ? need : gridw);
-    k_expect_wht<<<g, kRedThreads, 0, st>>>(psi, a, scr.partial);
-    k_finalize<<<1, 64, 0, st>>>(scr.partial, g, kExpGroup + 1, scr.result);
-    return cudaGetLastError();
+    k_expect_wht<<<g, kRedThreads, 0, st>>>(psi, a, scr.partials());
+    return finalize(scr.partials(), g, kExpGroup + 1, scr.result, st);
   }
   ExpArgs a;
   for (int m = 0; m < kExpGroup; ++m) a.masks[m] = m < nm ? masks[m] : 0;
@@ -466,9 +756,8 @@ cudaError_t launch_expect(const float2* psi, int n, int nm, const uint64_t* mask
   const int grid = grid_dev.get([] { return red_grid(k_expect, ~0ull >> 1); });
   const uint64_t need = (a.num_pairs + kRedThreads - 1) / kRedThreads;
   const int g = static_cast<int>(need < static_cast<uint64_t>(grid) ? need : grid);
-  k_expect<<<g, kRedThreads, 0, st>>>(psi, a, scr.partial);
-  k_finalize<<<1, 64, 0, st>>>(scr.partial, g, kExpGroup + 1, scr.result);
-  return cudaGetLastError();
+  k_expect<<<g, kRedThreads, 0, st>>>(psi, a, scr.partials());
+  return finalize(scr.partials(), g, kExpGroup + 1, scr.result, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -512,34 +801,69 @@ __device__ __forceinline__ void chunk_weights(const float2* __restrict__ psi, ui
   }
 }
 
-__global__ void k_cdf_sub(const float2* __restrict__ psi, uint64_t namps, uint64_t nsub,
-                          float* __restrict__ sub) {
+// Sums of a sub-block's 16 chunks, each in the order in which lane 31 of an
+// inclusive warp scan forms it (a binary tree over neighbouring lanes): lane
+// l (any l with the same low four bits) returns the sum of chunk l & 15.
+// Transposed: step o combines lanes o apart and halves the chunks a lane
+// holds, 16 exchanges for 16 chunks where one scan per chunk makes 80.
+__device__ __forceinline__ float chunk_sums(float (&p)[16], int lane) {
+  int c = 16;
+#pragma unroll
+  for (int o = 1; o < 16; o <<= 1) {
+    c >>= 1;
+    const bool up = lane & o;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (k >= c) break;
+      // chunks with bit o set go to the lanes with bit o set
+      const float keep = up ? p[2 * k + 1] : p[2 * k], send = up ? p[2 * k] : p[2 * k + 1];
+      p[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  return p[0] + __shfl_xor_sync(0xffffffffu, p[0], 16);
+}
+
+// One warp per sub-block, its 1024 amplitudes (8 KB) loaded before any
+// arithmetic.  Bound by HBM; n = 29: 782 -> 612 us (one chunk at a time, a
+// scan for each, before).
+__global__ void __launch_bounds__(256) k_cdf_sub(const float2* __restrict__ psi, uint64_t namps, uint64_t nsub,
+                                                 float* __restrict__ sub) {
+  constexpr int CH = 1 << (kCdfSubLog - kCdfChunkLog);
+  static_assert(CH == 16);
+  cudaTriggerProgrammaticLaunchCompletion();
   const int lane = threadIdx.x & 31;
   const uint64_t warp = (static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const uint64_t nwarps = (static_cast<uint64_t>(gridDim.x) * blockDim.x) >> 5;
   for (uint64_t s = warp; s < nsub; s += nwarps) {
-    float run = 0.f;
-    for (int c = 0; c < (1 << (kCdfSubLog - kCdfChunkLog)); ++c) {
+    float4 v[CH];
+#pragma unroll
+    for (int c = 0; c < CH; ++c) {
       const uint64_t x0 = (s << kCdfSubLog) + (static_cast<uint64_t>(c) << kCdfChunkLog) + 2 * lane;
-      float w0, w1;
-      chunk_weights(psi, namps, x0, w0, w1);
-      const float incl = warp_incl_scan_f(w0 + w1, lane);
-      run += __shfl_sync(0xffffffffu, incl, 31);
+      v[c] = x0 < namps ? __ldg(reinterpret_cast<const float4*>(psi + x0)) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
+    float p[CH];
+#pragma unroll
+    for (int c = 0; c < CH; ++c)
+      p[c] = fmaf(v[c].x, v[c].x, v[c].y * v[c].y) + fmaf(v[c].z, v[c].z, v[c].w * v[c].w);
+    const float sum = chunk_sums(p, lane);
+    float run = 0.f;
+#pragma unroll
+    for (int c = 0; c < CH; ++c) run += __shfl_sync(0xffffffffu, sum, c);
     if (lane == 0) sub[s] = run;
   }
 }
 
 // lane values of block b: (double)sub[2L] + (double)sub[2L+1]
-__device__ __forceinline__ void block_lane_values(const float* __restrict__ sub, uint64_t nsub,
+__device__ __forceinline__ void block_lane_values(const float* sub, uint64_t nsub,
                                                   uint64_t b, int lane, double& s0, double& s1) {
   const uint64_t i0 = (b << 6) + 2 * lane;
   s0 = i0 < nsub ? static_cast<double>(sub[i0]) : 0.0;
   s1 = i0 + 1 < nsub ? static_cast<double>(sub[i0 + 1]) : 0.0;
 }
 
-__global__ void k_cdf_blk(const float* __restrict__ sub, uint64_t nsub, uint64_t nblk,
-                          double* __restrict__ cum) {
+__global__ void k_cdf_blk(const float* sub, uint64_t nsub, uint64_t nblk, double* cum) {
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
   const int lane = threadIdx.x & 31;
   const uint64_t warp = (static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const uint64_t nwarps = (static_cast<uint64_t>(gridDim.x) * blockDim.x) >> 5;
@@ -551,45 +875,67 @@ __global__ void k_cdf_blk(const float* __restrict__ sub, uint64_t nsub, uint64_t
   }
 }
 
-// in-place inclusive scan of nblk doubles by one block of 1024 threads
-__global__ void __launch_bounds__(1024) k_cdf_scan(double* __restrict__ cum, uint64_t nblk) {
-  __shared__ double tot[1024];
+// In-place inclusive scan of nblk doubles by one block of 1024 threads, a
+// contiguous run per thread: warp scans of the run sums, then a scan of the
+// 32 warp totals (one thread chained the 1024 run sums before: 56-65 us at
+// 17 to 29 qubits, now 3 to 14).
+__global__ void __launch_bounds__(1024) k_cdf_scan(double* cum, uint64_t nblk) {
+  __shared__ double tot[32];
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint64_t per = (nblk + 1023) / 1024;
   const uint64_t lo = threadIdx.x * per;
   const uint64_t hi = lo + per < nblk ? lo + per : nblk;
-  double s = 0.0;
-  for (uint64_t i = lo; i < hi; ++i) s += cum[i];
-  tot[threadIdx.x] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double r = 0.0;
-    for (int t = 0; t < 1024; ++t) { const double v = tot[t]; tot[t] = r; r += v; }
+  const bool idle = (static_cast<uint64_t>(warp) << 5) * per >= nblk;   // the whole warp is past the end
+  double s = 0.0, incl = 0.0;
+  if (!idle) {
+    for (uint64_t i = lo; i < hi; ++i) s += cum[i];
+    incl = warp_incl_scan_d(s, lane);
   }
+  if (lane == 31) tot[warp] = incl;
   __syncthreads();
-  double r = tot[threadIdx.x];
+  if (warp == 0) tot[lane] = warp_incl_scan_d(tot[lane], lane);
+  __syncthreads();
+  if (idle) return;
+  double before = __shfl_up_sync(0xffffffffu, incl, 1);
+  if (lane == 0) before = 0.0;
+  double r = (warp ? tot[warp - 1] : 0.0) + before;
   for (uint64_t i = lo; i < hi; ++i) { r += cum[i]; cum[i] = r; }
+}
+
+// first b in [0, n) with t < cum[b], n - 1 if there is none: 32 probes a step.
+// cum[b - 1], when b > 0, was probed and is not above t.
+__device__ __forceinline__ uint64_t warp_search(const double* cum, uint64_t n, double t, int lane) {
+  uint64_t lo = 0, hi = n - 1;                           // the answer is in [lo, hi]
+  while (lo < hi) {
+    const uint64_t step = (hi - lo + 31) / 32;           // probes lo + step - 1, lo + 2 step - 1, ... below hi
+    const uint64_t p = lo + step * (lane + 1) - 1;
+    const unsigned hit = __ballot_sync(0xffffffffu, p < hi && t < cum[p]);
+    const unsigned in = __ballot_sync(0xffffffffu, p < hi);
+    const int first = hit ? __ffs(hit) - 1 : __popc(in); // probes before it are not above t
+    if (hit) hi = lo + step * (first + 1) - 1;
+    lo += step * first;
+  }
+  return lo;
 }
 
 // ro (optional): readout errors (Sec. V.A), 2 per qubit: qubit q of value b
 // is reported as 1 - b when u01(seed, traj, 2, (j << 6) | q) < ro[2q + b];
 // lane l decides qubits l and l + 32, and the flips are OR-combined.
-__global__ void k_sample(const float2* __restrict__ psi, uint64_t namps, const float* __restrict__ sub,
-                         uint64_t nsub, const double* __restrict__ cum, uint64_t nblk, uint64_t seed,
-                         uint64_t traj, uint32_t S, uint64_t* __restrict__ out, int n,
-                         const double* __restrict__ ro) {
+__global__ void __launch_bounds__(256) k_sample(const float2* __restrict__ psi, uint64_t namps, const float* sub,
+                                                uint64_t nsub, const double* cum, uint64_t nblk, uint64_t seed,
+                                                uint64_t traj, uint32_t S, uint64_t* __restrict__ out, int n,
+                                                const double* __restrict__ ro) {
+  constexpr int CH = 1 << (kCdfSubLog - kCdfChunkLog);
+  cudaGridDependencySynchronize();
   const int lane = threadIdx.x & 31;
   const uint64_t warp = (static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const uint64_t nwarps = (static_cast<uint64_t>(gridDim.x) * blockDim.x) >> 5;
   for (uint64_t j = warp; j < S; j += nwarps) {
     const double total = cum[nblk - 1];
     const double t = uniform01(seed, traj, kStreamSample, static_cast<uint32_t>(j)) * total;
-    // block: first b with t < cum[b]
-    uint64_t lo = 0, hi = nblk - 1;
-    while (lo < hi) {
-      const uint64_t mid = (lo + hi) >> 1;
-      if (t < cum[mid]) hi = mid; else lo = mid + 1;
-    }
-    const uint64_t b = lo;
+    const uint64_t b = warp_search(cum, nblk, t, lane);
     double trel = t - (b ? cum[b - 1] : 0.0);
     // sub-block inside the block (same lane values and scan as k_cdf_blk)
     double s0, s1;
@@ -606,13 +952,19 @@ __global__ void k_sample(const float2* __restrict__ psi, uint64_t namps, const f
     if (!(trel < eL + s0L)) { base = eL + s0L; sidx += 1; }
     if (sidx >= nsub) sidx = nsub - 1;
     trel -= base;
-    // chunks inside the sub-block (same chunk arithmetic as k_cdf_sub)
+    // chunks inside the sub-block (same chunk arithmetic as k_cdf_sub), all
+    // of it loaded before the search
+    float4 v[CH];
+#pragma unroll
+    for (int c = 0; c < CH; ++c) {
+      const uint64_t x0 = (sidx << kCdfSubLog) + (static_cast<uint64_t>(c) << kCdfChunkLog) + 2 * lane;
+      v[c] = x0 < namps ? __ldg(reinterpret_cast<const float4*>(psi + x0)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
     float run = 0.f;
     uint64_t x = ~0ull, last_nz = sidx << kCdfSubLog;
-    for (int c = 0; c < (1 << (kCdfSubLog - kCdfChunkLog)); ++c) {
-      const uint64_t x0 = (sidx << kCdfSubLog) + (static_cast<uint64_t>(c) << kCdfChunkLog) + 2 * lane;
-      float w0, w1;
-      chunk_weights(psi, namps, x0, w0, w1);
+#pragma unroll
+    for (int c = 0; c < CH; ++c) {
+      const float w0 = fmaf(v[c].x, v[c].x, v[c].y * v[c].y), w1 = fmaf(v[c].z, v[c].z, v[c].w * v[c].w);
       const float inc = warp_incl_scan_f(w0 + w1, lane);
       const float tot = __shfl_sync(0xffffffffu, inc, 31);
       const float cend = run + inc;
@@ -689,7 +1041,7 @@ __global__ void k_cdf_values(const float2* __restrict__ psi, uint64_t namps, con
 
 // the three table levels of the sampling CDF (sub-block runs, block scans,
 // FP64 table) into scr.cdf_sub / scr.cdf_cum
-static void build_cdf_tables(const float2* psi, int n, const Scratch& scr, cudaStream_t st) {
+static cudaError_t build_cdf_tables(const float2* psi, int n, const Scratch& scr, cudaStream_t st) {
   const uint64_t namps = 1ull << n;
   const uint64_t nsub = cdf_num_sub(n), nblk = cdf_num_blk(n);
   const int threads = 256, wpb = threads / 32;
@@ -699,13 +1051,16 @@ static void build_cdf_tables(const float2* psi, int n, const Scratch& scr, cudaS
   k_cdf_sub<<<static_cast<unsigned>(g), threads, 0, st>>>(psi, namps, nsub, scr.cdf_sub);
   uint64_t gb = (nblk + wpb - 1) / wpb;
   if (gb > cap) gb = cap;
-  k_cdf_blk<<<static_cast<unsigned>(gb), threads, 0, st>>>(scr.cdf_sub, nsub, nblk, scr.cdf_cum);
-  k_cdf_scan<<<1, 1024, 0, st>>>(scr.cdf_cum, nblk);
+  cudaError_t e = launch_dependent(k_cdf_blk, dim3(static_cast<unsigned>(gb)), threads, st, scr.cdf_sub, nsub, nblk,
+                                   scr.cdf_cum);
+  if (e == cudaSuccess) e = launch_dependent(k_cdf_scan, dim3(1), 1024, st, scr.cdf_cum, nblk);
+  return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
 cudaError_t launch_cdf_values(const float2* psi, int n, const Scratch& scr, double* out, cudaStream_t st) {
   if (n < 1) return cudaErrorInvalidValue;
-  build_cdf_tables(psi, n, scr, st);
+  const cudaError_t e = build_cdf_tables(psi, n, scr, st);
+  if (e != cudaSuccess) return e;
   const uint64_t nsub = cdf_num_sub(n);
   const int threads = 256, wpb = threads / 32;
   uint64_t g = (nsub + wpb - 1) / wpb;
@@ -722,14 +1077,12 @@ cudaError_t launch_sample(const float2* psi, int n, uint64_t seed, uint64_t traj
   const uint64_t nsub = cdf_num_sub(n), nblk = cdf_num_blk(n);
   const int threads = 256, wpb = threads / 32;
   const uint64_t cap = static_cast<uint64_t>(sm_count()) * 8;
-  build_cdf_tables(psi, n, scr, st);
-  if (S > 0) {
-    uint64_t gs = (S + wpb - 1) / wpb;
-    if (gs > cap) gs = cap;
-    k_sample<<<static_cast<unsigned>(gs), threads, 0, st>>>(psi, namps, scr.cdf_sub, nsub, scr.cdf_cum,
-                                                           nblk, seed, traj, S, out, n, readout);
-  }
-  return cudaGetLastError();
+  const cudaError_t e = build_cdf_tables(psi, n, scr, st);
+  if (e != cudaSuccess || S == 0) return e;
+  uint64_t gs = (S + wpb - 1) / wpb;
+  if (gs > cap) gs = cap;
+  return launch_dependent(k_sample, dim3(static_cast<unsigned>(gs)), threads, st, psi, namps, scr.cdf_sub, nsub,
+                          scr.cdf_cum, nblk, seed, traj, S, out, n, readout);
 }
 
 // ---------------------------------------------------------------------------

@@ -46,6 +46,9 @@ class PerDevice {
 constexpr int kRedThreads = 256;          // threads of the reduction kernels
 constexpr int kMaxRedBlocks = 152 * 8;    // upper bound of their grid
 constexpr int kRdmMaxQ = 3;               // reduced density matrix: q <= 3
+constexpr int kRdmMaxReals = 64;          // longest rdm result row
+constexpr int kResultDoubles = 64;
+constexpr int kPartialDoubles = kMaxRedBlocks * 64;
 constexpr int kExpGroup = 16;             // Z masks per expectation pass
 // CDF for sampling: chunk = 64 amplitudes (one warp, 128-bit loads),
 // sub-block = 16 chunks, block = 64 sub-blocks
@@ -55,18 +58,18 @@ inline uint64_t cdf_num_sub(int n) { return ((1ull << n) + (1ull << kCdfSubLog) 
 inline uint64_t cdf_num_blk(int n) { return (cdf_num_sub(n) + 63) >> 6; }
 
 struct Scratch {
-  double* partial = nullptr;   // kMaxRedBlocks * 64 doubles
-  double* result = nullptr;    // 64 doubles
+  double* partial = nullptr;   // kPartialDoubles doubles (held as that many double-floats)
+  double* result = nullptr;    // kResultDoubles doubles
   float* cdf_sub = nullptr;    // cdf_num_sub(n) floats
   double* cdf_cum = nullptr;   // cdf_num_blk(n) doubles
+  float2* partials() const { return reinterpret_cast<float2*>(partial); }
 };
-size_t scratch_partial_bytes();
 
 // ---- kernels ---------------------------------------------------------------
 // state <- U (2^k x 2^k row-major complex64, basis `targets` sorted ascending)
 cudaError_t launch_apply(float2* psi, int n, int k, const uint32_t* targets, const float2* U,
                          cudaStream_t st);
-// rho (4^q doubles, layout of rdm_unpack) of qubits Q into scr.result
+// rho (the 4^q reals that rdm_unpack takes) of qubits Q into scr.result
 cudaError_t launch_rdm(const float2* psi, int n, int q, const uint32_t* qubits, const Scratch& scr,
                        cudaStream_t st);
 // Channels on 4..6 qubits: N and P_i = |K_i psi|^2 for kraus_group(q)
@@ -126,9 +129,9 @@ cudaError_t launch_init_product(float2* psi, int n, int m, const FoldSpec& lo, c
 // psi *= f
 cudaError_t launch_scale(float2* psi, int n, float f, cudaStream_t st);
 
-// unpack the 4^q reals of an rdm result into a row-major complex matrix
-// rho[b][a] = sum psi_b conj(psi_a)
-void rdm_unpack(int q, const double* r, double* rho_interleaved);
+// unpack the reals of an rdm result into a row-major complex matrix
+// rho[b][a] = sum psi_b conj(psi_a), basis bit b <-> qubits[b]
+void rdm_unpack(int q, const uint32_t* qubits, const double* r, double* rho_interleaved);
 
 int sm_count();
 // binaryVersion / ptxVersion of the library's kernels on the current device

@@ -11,8 +11,8 @@
 //
 // Properties of that array:
 //   - it is kMaxRedBlocks * 64 + 64 doubles (608.5 KiB), enough for the
-//     largest reduction the kernels launch (q <= 3, i.e. 64 FP64 values per
-//     block); every GPU that loads the library holds it until the process
+//     largest reduction the kernels launch (q <= 3, up to 64 values
+//     per block); every GPU that loads the library holds it until the process
 //     exits;
 //   - every call on a device shares it and it keeps the last call's
 //     contents.  Nothing in it has to start at zero: every partial and the
@@ -35,7 +35,7 @@
 
 namespace qt {
 
-constexpr size_t kNoAllocDoubles = static_cast<size_t>(kMaxRedBlocks) * 64 + 64;
+constexpr size_t kNoAllocDoubles = static_cast<size_t>(kPartialDoubles) + kResultDoubles;
 
 static __device__ __align__(256) double g_noalloc_scratch[kNoAllocDoubles];
 
@@ -62,7 +62,7 @@ extern "C" qt_status qt_state_reduced_density_noalloc(const void* state, uint32_
     return set_error(QT_ERR_INVALID_ARG, "qt_state_reduced_density_noalloc: state not 16-byte aligned");
   if (n < 1 || n > QT_MAX_QUBITS)
     return set_error(QT_ERR_INVALID_ARG, "qt_state_reduced_density_noalloc: n=%u outside 1..%d", n, QT_MAX_QUBITS);
-  // the fixed scratch holds 64 FP64 values per block: q <= 3
+  // the fixed scratch is sized for q <= 3
   if (q < 1 || q > static_cast<uint32_t>(kRdmMaxQ) || q > n)
     return set_error(QT_ERR_UNSUPPORTED,
                      "qt_state_reduced_density_noalloc: q=%u exceeds the fixed scratch (q <= 3 and q <= n)", q);
@@ -78,17 +78,16 @@ extern "C" qt_status qt_state_reduced_density_noalloc(const void* state, uint32_
   qt_status s = noalloc_scratch(&scratch);
   if (s != QT_OK) return s;
   Scratch scr;
-  scr.partial = scratch;                                   // kMaxRedBlocks * 64 doubles
-  scr.result = scratch + static_cast<size_t>(kMaxRedBlocks) * 64;   // 64 doubles
+  scr.partial = scratch;
+  scr.result = scratch + kPartialDoubles;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t e = launch_rdm(static_cast<const float2*>(state), static_cast<int>(n), static_cast<int>(q), qubits,
                              scr, st);
-  double r[64];
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(r, scr.result, sizeof(double) << (2 * q), cudaMemcpyDeviceToHost, st);
+  double r[kRdmMaxReals];
+  if (e == cudaSuccess) e = cudaMemcpyAsync(r, scr.result, sizeof(double) << (2 * q), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess)
     return set_error(QT_ERR_CUDA, "qt_state_reduced_density_noalloc: %s", cudaGetErrorString(e));
-  rdm_unpack(static_cast<int>(q), r, out);
+  rdm_unpack(static_cast<int>(q), qubits, r, out);
   return QT_OK;
 }

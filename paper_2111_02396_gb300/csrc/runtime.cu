@@ -103,8 +103,8 @@ struct ScratchBufs {
   DevBuf partial, result, sub, cum;
   Scratch s;
   bool alloc(int n, cudaStream_t st) {
-    if (!partial.alloc(scratch_partial_bytes(), st)) return false;
-    if (!result.alloc(sizeof(double) * 64, st)) return false;
+    if (!partial.alloc(sizeof(double) * kPartialDoubles, st)) return false;
+    if (!result.alloc(sizeof(double) * kResultDoubles, st)) return false;
     if (!sub.alloc(sizeof(float) * cdf_num_sub(n), st)) return false;
     if (!cum.alloc(sizeof(double) * cdf_num_blk(n), st)) return false;
     s.partial = partial.as<double>();
@@ -112,6 +112,52 @@ struct ScratchBufs {
     s.cdf_sub = sub.as<float>();
     s.cdf_cum = cum.as<double>();
     return true;
+  }
+};
+
+// Probability pass of a channel on 4..6 qubits; keeps its buffers for the
+// next call.  Blocks until P and N are on the host.
+struct WideChannel {
+  DevBuf buf;
+  std::vector<float2> ops;
+  std::vector<double> rows;
+  uint64_t h2d = 0, d2h = 0, launches = 0;       // of the last call
+  qt_status run(const float2* psi, uint32_t n, uint32_t q, const uint32_t* qubits, uint32_t num_ops, const double* K,
+                double* P, double* N, cudaStream_t st) {
+    const int Q = static_cast<int>(q), D = 1 << Q;
+    const size_t mat = static_cast<size_t>(D) * D;
+    h2d = d2h = launches = 0;
+    // kraus_group(q) operators per pass, zero matrices padding the last group
+    const uint32_t G = static_cast<uint32_t>(kraus_group(Q));
+    const size_t scr_doubles = kPartialDoubles + kResultDoubles;
+    const size_t need = sizeof(double) * scr_doubles + sizeof(float2) * G * mat;
+    if (buf.bytes < need && !buf.alloc(need, st)) return set_error(QT_ERR_OUT_OF_MEMORY, "Kraus operator buffer");
+    Scratch scr;
+    scr.partial = buf.as<double>();
+    scr.result = scr.partial + kPartialDoubles;
+    float2* const kd = reinterpret_cast<float2*>(scr.partial + scr_doubles);
+    rows.resize(G + 1);
+    for (uint32_t g0 = 0; g0 < num_ops; g0 += G) {
+      ops.assign(G * mat, make_float2(0.f, 0.f));
+      for (uint32_t j = 0; j < G && g0 + j < num_ops; ++j)
+        for (size_t e = 0; e < mat; ++e) {
+          const double* k = K + 2 * (mat * (g0 + j) + e);
+          ops[j * mat + e] = make_float2(static_cast<float>(k[0]), static_cast<float>(k[1]));
+        }
+      QT_CUDA(cudaMemcpyAsync(kd, ops.data(), sizeof(float2) * G * mat, cudaMemcpyHostToDevice, st),
+              "cudaMemcpyAsync(Kraus operators)");
+      QT_CUDA(launch_kraus_norms(psi, static_cast<int>(n), Q, qubits, static_cast<int>(G), kd, scr, st),
+              "Kraus probability kernel launch");
+      QT_CUDA(cudaMemcpyAsync(rows.data(), scr.result, sizeof(double) * (G + 1), cudaMemcpyDeviceToHost, st),
+              "cudaMemcpyAsync(probabilities)");
+      QT_CUDA(cudaStreamSynchronize(st), "cudaStreamSynchronize(probabilities)");
+      h2d += sizeof(float2) * G * mat;
+      d2h += sizeof(double) * (G + 1);
+      launches += 2;
+      *N = rows[0];
+      for (uint32_t j = 0; j < G && g0 + j < num_ops; ++j) P[g0 + j] = rows[1 + j];
+    }
+    return QT_OK;
   }
 };
 
@@ -587,36 +633,17 @@ struct Controller {
     return QT_OK;
   }
 
-  // Channels on 4..6 qubits: P_i = |K_i psi|^2 on the device, kraus_group(q)
-  // operators per pass (zero matrices pad the last group); N from the same pass.
-  DevBuf kbuf;
-  std::vector<float2> ktmp;
+  // Channels on 4..6 qubits: the probabilities from the reduced density block,
+  // contracted with the operators on the device
+  WideChannel wide;
   qt_status kraus_probabilities(const float2* psi, const Op& op, double& N, double* P) {
     TraceRange tr("qt probability pass (wide channel)");
-    const int q = static_cast<int>(op.q), D = 1 << q, G = kraus_group(q);
-    const size_t mat = static_cast<size_t>(D) * D;
-    if (kbuf.bytes < sizeof(float2) * G * mat && !kbuf.alloc(sizeof(float2) * G * mat, R.st))
-      return set_error(QT_ERR_OUT_OF_MEMORY, "Kraus operator buffer");
-    for (uint32_t g0 = 0; g0 < op.num_ops; g0 += static_cast<uint32_t>(G)) {
-      ktmp.assign(G * mat, make_float2(0.f, 0.f));
-      for (uint32_t j = 0; j < static_cast<uint32_t>(G) && g0 + j < op.num_ops; ++j) {
-        const cd* K = op.kraus_op(g0 + j);
-        for (size_t e = 0; e < mat; ++e)
-          ktmp[j * mat + e] = make_float2(static_cast<float>(K[e].real()), static_cast<float>(K[e].imag()));
-      }
-      QT_CUDA(cudaMemcpyAsync(kbuf.p, ktmp.data(), sizeof(float2) * G * mat, cudaMemcpyHostToDevice, R.st),
-              "cudaMemcpyAsync(Kraus operators)");
-      QT_CUDA(launch_kraus_norms(psi, static_cast<int>(R.n), q, op.qubits, G, kbuf.as<float2>(), R.scr.s, R.st),
-              "Kraus probability kernel launch");
-      QT_CUDA(cudaMemcpyAsync(pinned, R.scr.s.result, sizeof(double) * (G + 1), cudaMemcpyDeviceToHost, R.st),
-              "cudaMemcpyAsync(probabilities)");
-      QT_CUDA(cudaStreamSynchronize(R.st), "cudaStreamSynchronize(probabilities)");
-      R.stats.h2d_bytes += sizeof(float2) * G * mat;
-      R.stats.d2h_bytes += sizeof(double) * (G + 1);
-      R.stats.kernel_launches += 2;
-      N = pinned[0];
-      for (uint32_t j = 0; j < static_cast<uint32_t>(G) && g0 + j < op.num_ops; ++j) P[g0 + j] = pinned[1 + j];
-    }
+    const qt_status s = wide.run(psi, R.n, op.q, op.qubits, op.num_ops, reinterpret_cast<const double*>(op.kraus.data()),
+                                 P, &N, R.st);
+    if (s != QT_OK) return s;
+    R.stats.h2d_bytes += wide.h2d;
+    R.stats.d2h_bytes += wide.d2h;
+    R.stats.kernel_launches += wide.launches;
     R.stats.prob_passes++;
     return QT_OK;
   }
@@ -640,7 +667,7 @@ struct Controller {
     R.stats.d2h_bytes += sizeof(double) * W;
     const int D = static_cast<int>(op.dim());
     double rho[2 * 64];
-    rdm_unpack(static_cast<int>(op.q), pinned, rho);
+    rdm_unpack(static_cast<int>(op.q), op.qubits, pinned, rho);
     N = 0.0;
     for (int b = 0; b < D; ++b) N += rho[2 * (b * D + b)];
     for (uint32_t i = 0; i < op.num_ops; ++i) {
@@ -1162,10 +1189,11 @@ qt_status qt_state_reduced_density(const void* state, uint32_t n, uint32_t q, co
   if (!scr.alloc(1, st)) return set_error(QT_ERR_OUT_OF_MEMORY, "qt_state_reduced_density: scratch");
   QT_CUDA(launch_rdm(static_cast<const float2*>(state), static_cast<int>(n), static_cast<int>(q), qubits, scr.s, st),
           "qt_state_reduced_density");
-  double r[64];
-  QT_CUDA(cudaMemcpyAsync(r, scr.s.result, sizeof(double) << (2 * q), cudaMemcpyDeviceToHost, st), "cudaMemcpyAsync");
+  double r[kRdmMaxReals];
+  QT_CUDA(cudaMemcpyAsync(r, scr.s.result, sizeof(double) << (2 * q), cudaMemcpyDeviceToHost, st),
+          "cudaMemcpyAsync");
   QT_CUDA(cudaStreamSynchronize(st), "cudaStreamSynchronize");
-  rdm_unpack(static_cast<int>(q), r, out);
+  rdm_unpack(static_cast<int>(q), qubits, r, out);
   return QT_OK;
 }
 
@@ -1183,15 +1211,16 @@ qt_status qt_state_kraus_probabilities(const void* state, uint32_t n, uint32_t q
   const int D = 1 << q;
   const size_t mat = static_cast<size_t>(D) * D;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  ScratchBufs scr;
-  if (!scr.alloc(1, st)) return set_error(QT_ERR_OUT_OF_MEMORY, "qt_state_kraus_probabilities: scratch");
   if (q <= kRdmMaxQ) {                     // P_i = tr(K_i^dag K_i rho) from the reduced density
+    ScratchBufs scr;
+    if (!scr.alloc(1, st)) return set_error(QT_ERR_OUT_OF_MEMORY, "qt_state_kraus_probabilities: scratch");
     QT_CUDA(launch_rdm(static_cast<const float2*>(state), static_cast<int>(n), static_cast<int>(q), qubits, scr.s, st),
             "qt_state_kraus_probabilities");
-    double r[64], rho[2 * 64];
-    QT_CUDA(cudaMemcpyAsync(r, scr.s.result, sizeof(double) << (2 * q), cudaMemcpyDeviceToHost, st), "cudaMemcpyAsync");
+    double r[kRdmMaxReals], rho[2 * 64];
+    QT_CUDA(cudaMemcpyAsync(r, scr.s.result, sizeof(double) << (2 * q), cudaMemcpyDeviceToHost, st),
+            "cudaMemcpyAsync");
     QT_CUDA(cudaStreamSynchronize(st), "cudaStreamSynchronize");
-    rdm_unpack(static_cast<int>(q), r, rho);
+    rdm_unpack(static_cast<int>(q), qubits, r, rho);
     *N = 0.0;
     for (int b = 0; b < D; ++b) *N += rho[2 * (b * D + b)];
     for (uint32_t i = 0; i < num_ops; ++i) {
@@ -1208,28 +1237,8 @@ qt_status qt_state_kraus_probabilities(const void* state, uint32_t n, uint32_t q
     }
     return QT_OK;
   }
-  const int G = kraus_group(static_cast<int>(q));
-  DevBuf kd;
-  if (!kd.alloc(sizeof(float2) * G * mat, st)) return set_error(QT_ERR_OUT_OF_MEMORY, "qt_state_kraus_probabilities: operators");
-  std::vector<float2> tmp;
-  for (uint32_t g0 = 0; g0 < num_ops; g0 += static_cast<uint32_t>(G)) {
-    tmp.assign(G * mat, make_float2(0.f, 0.f));
-    for (uint32_t j = 0; j < static_cast<uint32_t>(G) && g0 + j < num_ops; ++j)
-      for (size_t e = 0; e < mat; ++e) {
-        const double* K = ops + 2 * (mat * (g0 + j) + e);
-        tmp[j * mat + e] = make_float2(static_cast<float>(K[0]), static_cast<float>(K[1]));
-      }
-    QT_CUDA(cudaMemcpyAsync(kd.p, tmp.data(), sizeof(float2) * G * mat, cudaMemcpyHostToDevice, st), "cudaMemcpyAsync");
-    QT_CUDA(launch_kraus_norms(static_cast<const float2*>(state), static_cast<int>(n), static_cast<int>(q), qubits, G,
-                               kd.as<float2>(), scr.s, st),
-            "qt_state_kraus_probabilities");
-    double r[17];
-    QT_CUDA(cudaMemcpyAsync(r, scr.s.result, sizeof(double) * (G + 1), cudaMemcpyDeviceToHost, st), "cudaMemcpyAsync");
-    QT_CUDA(cudaStreamSynchronize(st), "cudaStreamSynchronize");
-    *N = r[0];
-    for (uint32_t j = 0; j < static_cast<uint32_t>(G) && g0 + j < num_ops; ++j) P[g0 + j] = r[1 + j];
-  }
-  return QT_OK;
+  WideChannel w;
+  return w.run(static_cast<const float2*>(state), n, q, qubits, num_ops, ops, P, N, st);
 }
 
 qt_status qt_state_sample(const void* state, uint32_t n, uint64_t seed, uint64_t traj, uint32_t S, uint64_t* out,
