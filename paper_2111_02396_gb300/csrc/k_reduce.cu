@@ -405,6 +405,223 @@ static cudaError_t rdm3_low(const float2* psi, int n, const uint32_t* s, const S
   return finalize(scr.partials(), static_cast<int>(g), 64, scr.result, st);
 }
 
+// ---------------------------------------------------------------------------
+// q = 4, 5 (k_gram): the block is a Hermitian rank-k update, 4 * 2^q FMA per
+// amplitude counting both triangles, so the lower triangle is cut into 4 x 4
+// complex tiles and a thread owns one (its "role": tile rows bi, columns bj)
+// for the gather sets of its group: 8 members from shared memory feed 64
+// FMAs.  Bound by FP32 FMA and the shared-memory reads that feed them.  A CTA
+// stages 4096 amplitudes at a time, one set after the other; the next tile's
+// loads are in flight while this one is multiplied.  Member m of a set sits
+// at m + m / 16 of a row of odd pitch: the blocks a warp reads together then
+// fall into different banks.  FP32 runs are carried in double-floats held in
+// shared memory, which leaves 128 registers a thread, two CTAs an SM.  A
+// run's length grows with the number of sets, for the reason given at
+// kRdmChunk; a wide channel's probabilities average the error of 4^q entries,
+// so its runs may be longer.
+// n = 25, q = 4 / 5: 138 / 158 us; the products K_i v that gave these
+// channels' probabilities before took 2719 / 1584 us for each 16 / 4 operators.
+// ---------------------------------------------------------------------------
+template <int Q>
+struct Gram {
+  static constexpr int D = 1 << Q;
+  static constexpr int NB = D / 4;                       // 4-member blocks
+  static constexpr int ROLES = NB * (NB + 1) / 2;        // tiles of the lower triangle
+  static constexpr int THREADS = 256;
+  static constexpr int GROUPS = THREADS / ROLES;         // 25, 7 sets at a time
+  static constexpr int TILE = 4096;                      // amplitudes staged at a time
+  static constexpr int SETS = TILE / D;
+  static constexpr int PITCH = D + 1;
+  static constexpr int OUT = ROLES * 32;
+  static constexpr size_t SMEM = sizeof(float2) * (SETS * PITCH + 32 * THREADS);
+  static constexpr int NCH = TILE / 2 / THREADS;         // 8 128-bit loads a thread and tile
+};
+
+template <int Q>
+struct GramArgs {
+  uint64_t offs[1 << Q];      // amplitude offset of member m within a set
+  uint64_t coff[8];           // what chunk c adds to a thread's address (amplitudes)
+  uint32_t cset[8], cmem[8];  // what chunk c adds to the thread's set and member
+  uint32_t ins[Q + 1];        // ascending bit positions to insert zeros at
+  uint64_t num_tiles;
+  int run;                    // sets summed in FP32 before the carry
+};
+
+// bi, bj (bj <= bi) of tile r of the lower triangle
+__device__ __forceinline__ void gram_tile(int r, int& bi, int& bj) {
+  bi = 0;
+  while ((bi + 1) * (bi + 2) / 2 <= r) ++bi;
+  bj = r - bi * (bi + 1) / 2;
+}
+
+template <int Q, bool LOW0>
+__global__ void __launch_bounds__(Gram<Q>::THREADS, 2) k_gram(const float2* __restrict__ psi,
+                                                              const __grid_constant__ GramArgs<Q> a,
+                                                              float2* __restrict__ partial) {
+  using G = Gram<Q>;
+  constexpr int NI = LOW0 ? Q : Q + 1;
+  constexpr int LOGJ = (LOW0 ? 12 : 11) - Q;             // log2 of the sets (set pairs) of a tile
+  extern __shared__ __align__(16) float2 s_gram[];
+  float2* const tile_s = s_gram;                         // [SETS][PITCH]
+  float2* const carry = s_gram + G::SETS * G::PITCH;     // [32][THREADS]
+  cudaTriggerProgrammaticLaunchCompletion();
+  const int tid = threadIdx.x;
+  // chunk c of this thread is 128-bit word e = tid + 256 c of the tile: set
+  // (pair) e mod 2^LOGJ, member (pair) e >> LOGJ; both split into a thread
+  // part and a part that only depends on c
+  const uint32_t j0 = tid & ((1u << (LOGJ < 8 ? LOGJ : 8)) - 1u);
+  const uint32_t m0 = LOGJ < 8 ? static_cast<uint32_t>(tid) >> LOGJ : 0u;
+  const uint32_t set0 = LOW0 ? j0 : 2u * j0, mem0 = LOW0 ? 2u * m0 : m0;
+  auto spread = [&](uint64_t x) {
+#pragma unroll
+    for (int b = 0; b < NI; ++b) {
+      const uint32_t s = a.ins[b];
+      x = ((x >> s) << (s + 1)) | (x & ((1ull << s) - 1ull));
+    }
+    return x;
+  };
+  const uint64_t toff = spread(j0) | a.offs[mem0];
+  const int role = tid % G::ROLES, group = tid / G::ROLES;
+  const bool active = group < G::GROUPS;
+  int bi, bj;
+  gram_tile(role, bi, bj);
+  const int xo = 4 * bi + (bi >> 2), yo = 4 * bj + (bj >> 2);
+  float f[32];
+#pragma unroll
+  for (int k = 0; k < 32; ++k) {
+    f[k] = 0.f;
+    carry[k * G::THREADS + tid] = make_float2(0.f, 0.f);
+  }
+  float4 buf[G::NCH];
+  auto load = [&](uint64_t tile) {
+    const uint64_t base = spread(tile << LOGJ) | toff;
+#pragma unroll
+    for (int c = 0; c < G::NCH; ++c) buf[c] = __ldg(reinterpret_cast<const float4*>(psi + (base | a.coff[c])));
+  };
+  auto flush = [&] {
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+      float2 c = carry[k * G::THREADS + tid];
+      df_acc(c.x, c.y, f[k]);
+      carry[k * G::THREADS + tid] = c;
+      f[k] = 0.f;
+    }
+  };
+  uint64_t tile = blockIdx.x;
+  load(tile);                                            // the grid has at most num_tiles blocks
+  int run = 0;
+  for (; tile < a.num_tiles; tile += gridDim.x) {
+#pragma unroll
+    for (int c = 0; c < G::NCH; ++c) {
+      const uint32_t m = mem0 + a.cmem[c];
+      float2* const d = tile_s + (set0 + a.cset[c]) * G::PITCH + m + (m >> 4);
+      d[0] = make_float2(buf[c].x, buf[c].y);
+      d[LOW0 ? 1 : G::PITCH] = make_float2(buf[c].z, buf[c].w);
+    }
+    __syncthreads();
+    if (tile + gridDim.x < a.num_tiles) load(tile + gridDim.x);
+    if (active) {
+      for (int s = group; s < G::SETS; s += G::GROUPS) {
+        const float2* const v = tile_s + s * G::PITCH;
+        float2 x[4], y[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { x[k] = v[xo + k]; y[k] = v[yo + k]; }
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            // x_p conj(y_q)
+            f[4 * p + q] = fmaf(x[p].x, y[q].x, fmaf(x[p].y, y[q].y, f[4 * p + q]));
+            f[16 + 4 * p + q] = fmaf(x[p].y, y[q].x, fmaf(-x[p].x, y[q].y, f[16 + 4 * p + q]));
+          }
+        if (++run == a.run) { flush(); run = 0; }
+      }
+    }
+    __syncthreads();                                     // the tile is read: its buffer is free
+  }
+  if (active) flush();
+  __syncthreads();
+  for (int o = tid; o < G::OUT; o += G::THREADS) {
+    const int r = o >> 5, k = o & 31;
+    float2 sum = make_float2(0.f, 0.f);
+    for (int g = 0; g < G::GROUPS; ++g) sum = df_add(sum, carry[k * G::THREADS + g * G::ROLES + r]);
+    partial[static_cast<size_t>(blockIdx.x) * G::OUT + o] = sum;
+  }
+}
+
+// rho (2^Q x 2^Q, entry [b][a] at b * 2^Q + a) as double-floats
+// (re.h, re.l, im.h, im.l) from the blocks' partial tiles
+template <int Q>
+__global__ void __launch_bounds__(kSumThreads) k_gram_matrix(const float2* partial, int nblocks, float4* rho) {
+  using G = Gram<Q>;
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+  const int col = blockIdx.x * 32 + threadIdx.x % 32;    // OUT is a multiple of 32: block = one role
+  float2 v = column_sum<32>(partial, nblocks, G::OUT, col);
+  if (threadIdx.x >= 32) return;
+  // lanes 0..15 hold the real parts of the tile's entries, 16..31 the imaginary ones
+  const float2 w = df_shfl_xor(v, 16);
+  int bi, bj;
+  gram_tile(static_cast<int>(blockIdx.x), bi, bj);
+  const int b = 4 * bi + ((threadIdx.x & 15) >> 2), c = 4 * bj + (threadIdx.x & 3);
+  if (b < c) return;                                     // upper half of a diagonal tile
+  if (threadIdx.x < 16) rho[b * G::D + c] = b == c ? make_float4(v.x, v.y, 0.f, 0.f) : make_float4(v.x, v.y, w.x, w.y);
+  else if (b > c) rho[c * G::D + b] = make_float4(w.x, w.y, -v.x, -v.y);
+}
+
+template <int Q, bool LOW0>
+static cudaError_t gram_low(const float2* psi, int n, const uint32_t* s, float2* partial, int max_blocks, int* blocks,
+                            cudaStream_t st) {
+  using G = Gram<Q>;
+  constexpr int LOGJ = (LOW0 ? 12 : 11) - Q;
+  GramArgs<Q> a{};
+  int ni = 0;
+  if (!LOW0) a.ins[ni++] = 0;
+  for (int b = 0; b < Q; ++b) a.ins[ni++] = s[b];
+  for (int m = 0; m < G::D; ++m) {
+    uint64_t o = 0;
+    for (int b = 0; b < Q; ++b)
+      if ((m >> b) & 1) o |= 1ull << s[b];
+    a.offs[m] = o;
+  }
+  for (int c = 0; c < 8; ++c) {
+    const uint32_t e = 256u * c;
+    const uint32_t j = e & ((1u << LOGJ) - 1u), m = e >> LOGJ;
+    a.cset[c] = LOW0 ? j : 2 * j;
+    a.cmem[c] = LOW0 ? 2 * m : m;
+    uint64_t x = j;
+    for (int b = 0; b < ni; ++b) x = ((x >> a.ins[b]) << (a.ins[b] + 1)) | (x & ((1ull << a.ins[b]) - 1ull));
+    a.coff[c] = x | a.offs[a.cmem[c]];
+  }
+  a.num_tiles = 1ull << (n - 12);                        // n - Q >= kGramMinLog: whole tiles
+  a.run = carry_run(0.03, n - Q, 32);
+  static PerDevice setup;
+  const int grid = setup.get([] {
+    if (cudaFuncSetAttribute(k_gram<Q, LOW0>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(G::SMEM)) !=
+        cudaSuccess)
+      return 0;
+    int occ = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_gram<Q, LOW0>, G::THREADS, G::SMEM);
+    return sm_count() * (occ > 0 ? occ : 1);
+  });
+  if (grid <= 0) return cudaErrorInvalidConfiguration;
+  uint64_t g = a.num_tiles;
+  if (g > static_cast<uint64_t>(grid)) g = grid;
+  if (g > static_cast<uint64_t>(max_blocks)) g = max_blocks;
+  *blocks = static_cast<int>(g);
+  k_gram<Q, LOW0><<<static_cast<unsigned>(g), G::THREADS, G::SMEM, st>>>(psi, a, partial);
+  return cudaGetLastError();
+}
+
+template <int Q>
+static cudaError_t gram_q(const float2* psi, int n, const uint32_t* qubits, float2* partial, int max_blocks, int* blocks,
+                          cudaStream_t st) {
+  uint32_t s[Q];
+  sort_qubits<Q>(qubits, s);
+  return s[0] == 0 ? gram_low<Q, true>(psi, n, s, partial, max_blocks, blocks, st)
+                   : gram_low<Q, false>(psi, n, s, partial, max_blocks, blocks, st);
+}
+
 template <int Q>
 static cudaError_t rdm_q(const float2* psi, int n, const uint32_t* qubits, const Scratch& scr, cudaStream_t st) {
   uint32_t s[Q];
@@ -469,9 +686,117 @@ void rdm_unpack(int q, const uint32_t* qubits, const double* r, double* rho) {
 }
 
 // ---------------------------------------------------------------------------
-// Branch probabilities of a channel on 4..6 qubits (Alg. 2 step 14): for G
-// Kraus operators at a time, P_i = <psi|K_i^dag K_i|psi> = sum over gather
-// sets of |K_i v|^2, plus N = <psi|psi>.  Each thread takes whole gather sets, staged
+// Branch probabilities of a channel on 4 or 5 qubits (Alg. 2 step 14).  With
+// rho the reduced density block, P_i = <psi|K_i^dag K_i|psi> is
+//   sum_j k_j rho k_j^dag   over the rows k_j of K_i,
+// so one pass over the state serves every operator of the channel, where
+// forming |K_i v|^2 per operator costs twice the arithmetic of rho each.  The
+// contraction (2^(3q) products per operator) is far below the pass but wants
+// more than FP32; FP64 is slow here, so rho enters as double-floats and the
+// products keep their FMA error term.  The operators are complex64.
+// From 2^18 gather sets on (kGramMinLog): there the FP32 rounding of either
+// form has averaged out and they agree to 7e-10 over 60 inputs each (q = 4,
+// 5).  Below, and for q = 6, whose rows of 128 FP32 terms leave a mean of
+// -6e-10 in k_kraus_norms at any size (the two then differ by up to 1.3e-9),
+// k_kraus_norms stays: a call's result is not to move by 1e-9.
+// ---------------------------------------------------------------------------
+// acc += x y, x a double-float
+__device__ __forceinline__ void df_mul_acc(float2& acc, float xh, float xl, float y) {
+  const float p = xh * y;
+  const float e = fmaf(xl, y, fmaf(xh, y, -p));
+  df_acc(acc.x, acc.y, p);
+  acc.y += e;
+}
+
+// block (x, i): 256 of the terms (eight b, entry a, row j) of operator i,
+// Re(k_ja sum_b rho[a][b] conj(k_jb)), summed into out[i * gridDim.x + x]
+template <int Q>
+__global__ void __launch_bounds__(256) k_kraus_trace(const float4* rho, const float2* __restrict__ ops, double* out) {
+  constexpr int D = 1 << Q;
+  __shared__ float2 s_sum[8];
+  cudaGridDependencySynchronize();
+  const int idx = blockIdx.x * 256 + threadIdx.x, a = idx % D, j = (idx / D) % D, b0 = idx / (D * D) * 8;
+  const float2* const k = ops + (static_cast<size_t>(blockIdx.y) * D + j) * D;
+  float2 tr = make_float2(0.f, 0.f), ti = make_float2(0.f, 0.f);
+#pragma unroll 4
+  for (int b = b0; b < b0 + 8; ++b) {
+    // rho[a][b] = conj(rho[b][a]); lanes read neighbouring a
+    const float4 r = rho[b * D + a];
+    const float2 c = __ldg(k + b);
+    // conj(r) conj(c)
+    df_mul_acc(tr, r.x, r.y, c.x);
+    df_mul_acc(tr, -r.z, -r.w, c.y);
+    df_mul_acc(ti, -r.x, -r.y, c.y);
+    df_mul_acc(ti, -r.z, -r.w, c.x);
+  }
+  const float2 c = __ldg(k + a);
+  float2 v[1] = {make_float2(0.f, 0.f)};
+  df_mul_acc(v[0], tr.x, tr.y, c.x);
+  df_mul_acc(v[0], ti.x, ti.y, -c.y);
+  const float2 s = df_warp_sum<1>(v, threadIdx.x & 31);
+  if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float2 r = s_sum[0];
+    for (int w = 1; w < 8; ++w) r = df_add(r, s_sum[w]);
+    out[blockIdx.y * gridDim.x + blockIdx.x] = df_value(r);
+  }
+}
+
+int kraus_slices(int q) { return (1 << (3 * q - 3)) / 256; }
+
+// the result rows, padded so that the operators after them are 16-byte aligned
+size_t kraus_results(int q, int nops) { return (static_cast<size_t>(nops) * kraus_slices(q) + 1) & ~size_t(1); }
+
+static int kraus_grid() { return sm_count() * 2; }
+
+size_t kraus_scratch_bytes(int q, int nops) {
+  const size_t D = 1ull << q, nb = D / 4, out = nb * (nb + 1) / 2 * 32;
+  return sizeof(double) * kraus_results(q, nops) + sizeof(float2) * nops * D * D + sizeof(float4) * D * D +
+         sizeof(float2) * kraus_grid() * out;
+}
+
+void kraus_sort_columns(int q, const uint32_t* qubits, const double* K, float2* out) {
+  const int D = 1 << q;
+  for (int a = 0; a < D; ++a) {                          // column of sorted-basis index a
+    int u = 0;
+    for (int b = 0; b < q; ++b) {
+      int pos = 0;
+      for (int k = 0; k < q; ++k) pos += qubits[k] < qubits[b];
+      u |= ((a >> pos) & 1) << b;
+    }
+    for (int j = 0; j < D; ++j)
+      out[j * D + a] = make_float2(static_cast<float>(K[2 * (j * D + u)]), static_cast<float>(K[2 * (j * D + u) + 1]));
+  }
+}
+
+template <int Q>
+static cudaError_t kraus_q(const float2* psi, int n, const uint32_t* qubits, int nops, void* scratch, cudaStream_t st) {
+  using G = Gram<Q>;
+  double* const out = static_cast<double*>(scratch);
+  float2* const ops = reinterpret_cast<float2*>(out + kraus_results(Q, nops));
+  float4* const rho = reinterpret_cast<float4*>(ops + static_cast<size_t>(nops) * G::D * G::D);
+  float2* const partial = reinterpret_cast<float2*>(rho + G::D * G::D);
+  int g = 0;
+  cudaError_t e = gram_q<Q>(psi, n, qubits, partial, kraus_grid(), &g, st);
+  if (e == cudaSuccess) e = launch_dependent(k_gram_matrix<Q>, dim3(G::ROLES), kSumThreads, st, partial, g, rho);
+  if (e == cudaSuccess)
+    e = launch_dependent(k_kraus_trace<Q>, dim3(kraus_slices(Q), nops), 256, st, rho, ops, out);
+  return e;
+}
+
+cudaError_t launch_kraus_probs(const float2* psi, int n, int q, const uint32_t* qubits, int nops, void* scratch,
+                               cudaStream_t st) {
+  if (q > n || nops < 1) return cudaErrorInvalidValue;
+  switch (q) {
+    case 4: return kraus_q<4>(psi, n, qubits, nops, scratch, st);
+    case 5: return kraus_q<5>(psi, n, qubits, nops, scratch, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+// Channels on 6 qubits and smaller states: for G operators at a time, P_i = sum over gather sets of
+// |K_i v|^2, plus N = <psi|psi>.  Each thread takes whole gather sets, staged
 // column-wise in shared memory (member m of thread t at v[m * blockDim + t],
 // conflict-free), with the G operators in shared memory.  Products and row
 // sums in FP32; runs of kKrausChunk sets in FP32, carried in double-floats.

@@ -127,6 +127,31 @@ struct WideChannel {
     const int Q = static_cast<int>(q), D = 1 << Q;
     const size_t mat = static_cast<size_t>(D) * D;
     h2d = d2h = launches = 0;
+    if (kraus_by_gram(static_cast<int>(n), Q)) {
+      // every operator in one pass, an identity after them (its P is N)
+      const int nops = static_cast<int>(num_ops) + 1, slices = kraus_slices(Q);
+      const size_t nres = static_cast<size_t>(nops) * slices, need = kraus_scratch_bytes(Q, nops);
+      if (buf.bytes < need && !buf.alloc(need, st)) return set_error(QT_ERR_OUT_OF_MEMORY, "Kraus operator buffer");
+      ops.assign(mat * nops, make_float2(0.f, 0.f));
+      for (uint32_t i = 0; i < num_ops; ++i) kraus_sort_columns(Q, qubits, K + 2 * mat * i, ops.data() + mat * i);
+      for (int j = 0; j < D; ++j) ops[mat * num_ops + static_cast<size_t>(j) * (D + 1)].x = 1.f;
+      rows.resize(nres);
+      double* const res = buf.as<double>();
+      h2d = sizeof(float2) * ops.size();
+      d2h = sizeof(double) * nres;
+      launches = 3;
+      QT_CUDA(cudaMemcpyAsync(res + kraus_results(Q, nops), ops.data(), h2d, cudaMemcpyHostToDevice, st),
+              "cudaMemcpyAsync(Kraus operators)");
+      QT_CUDA(launch_kraus_probs(psi, static_cast<int>(n), Q, qubits, nops, res, st), "Kraus probability kernel launch");
+      QT_CUDA(cudaMemcpyAsync(rows.data(), res, d2h, cudaMemcpyDeviceToHost, st), "cudaMemcpyAsync(probabilities)");
+      QT_CUDA(cudaStreamSynchronize(st), "cudaStreamSynchronize(probabilities)");
+      for (int i = 0; i < nops; ++i) {
+        double s = 0.0;
+        for (int k = 0; k < slices; ++k) s += rows[static_cast<size_t>(i) * slices + k];
+        (i < static_cast<int>(num_ops) ? P[i] : *N) = s;
+      }
+      return QT_OK;
+    }
     // kraus_group(q) operators per pass, zero matrices padding the last group
     const uint32_t G = static_cast<uint32_t>(kraus_group(Q));
     const size_t scr_doubles = kPartialDoubles + kResultDoubles;
