@@ -6,12 +6,13 @@
 // small circuits and its translation overhead dominates below 20 qubits,
 // Sec. IV.A).  Here every trajectory of the batch, each with its own
 // circuit, runs inside one persistent kernel:
-//   - one CTA per SM takes trajectories from an atomic counter, largest
-//     state first;
-//   - a state of up to 2^14 amplitudes lives in the CTA's shared memory;
-//     larger states live in a per-CTA slot of global memory (up to 2^20
-//     amplitudes, so they stream from DRAM, and each thread keeps 16
-//     amplitude loads in flight to cover the latency);
+//   - CTAs take trajectories from an atomic counter per class of state sizes,
+//     largest state first;
+//   - a state of up to 2^14 amplitudes lives in its CTA's shared memory, the
+//     CTA sized to it, so that an SM holds several small ones; larger states
+//     live in a per-CTA slot of global memory (up to 2^20 amplitudes, so they
+//     stream from DRAM, and each thread keeps 16 amplitude loads in flight to
+//     cover the latency);
 //   - stage 1 of Alg. 2 for every channel is decided on the device with the
 //     same Philox4x32-10 draws as the plain loop; stage-2 flush points cut
 //     the circuit into segments exactly as in the plain loop, and within a
@@ -39,6 +40,7 @@
 #include <vector>
 
 #include "kernels.h"
+#include "qt_dfloat.h"
 #include "qt_internal.h"
 #include "qt_philox.h"
 
@@ -51,6 +53,9 @@ constexpr int kMaxN = 20;           // widest state of the batched form
 // product-state start: sum of 2^w over the folded pieces (disjoint qubits,
 // w <= 6, n <= 20 give at most 3 * 64 + 4)
 constexpr int kFoldCols = 256;
+// classes of trajectories, one launch each (qt_batch::count)
+constexpr int kClasses = 5;
+inline int class_of(uint32_t n) { return n > 14 ? 0 : (n == 14 ? 1 : (n == 13 ? 2 : (n > 10 ? 3 : 4))); }
 
 struct Traj {
   uint32_t n, gate0, ngates, op0, nops, ch0, nch, chop0;   // ch0: output offset; chop0: ch_op table offset
@@ -64,11 +69,12 @@ struct Op {
   uint8_t kind, q, q0, q1;
   uint32_t set;
   int32_t channel;                  // relative channel ordinal, -1 for gates
-  uint32_t pad;
+  uint32_t gate;                    // fused gate that holds it (relative)
 };
 struct Set {
   uint32_t nk, q, def, pad;
   uint32_t mat, kraus, mtm, pbar;   // offsets: float2, float2, double, double
+  uint64_t thr0;                    // a draw of `bits` / 2^53 is below pbar[0] exactly when bits < thr0
 };
 struct Gate {
   uint8_t w, t[kMaxW];
@@ -98,71 +104,84 @@ struct Dev {
   const uint64_t* run;              // {seed, first_traj} of the current run (device copy)
   uint32_t num, S, keep;
   uint32_t per_traj;                // 1: seed, id and samples from each Traj (merged launches)
+  uint32_t lthreads;                // threads that the sums of a trajectory are split over (results depend
+                                    // on them, not on the CTA's own size)
+  uint32_t wmat;                    // widest fused gate of the launch
 };
 
 // ---------------------------------------------------------------------------
 // device helpers (all threads of the CTA call them together)
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint64_t insert_zeros(uint64_t x, int w, const int* sorted) {
+__device__ __forceinline__ uint32_t insert_zeros32(uint32_t x, int w, const int* sorted) {
   for (int b = 0; b < w; ++b) {
     const int s = sorted[b];
-    x = ((x >> s) << (s + 1)) | (x & ((1ull << s) - 1ull));
+    x = ((x >> s) << (s + 1)) | (x & ((1u << s) - 1u));
   }
   return x;
 }
 
-// psi <- A psi on qubits order[0..W) (basis bit b <-> order[b]); A (row-major) in smem
-template <int W, bool GLOBAL>
-__device__ void cta_apply_w(float2* psi, int n, const int* order, const float2* A) {
+// Where amplitude x of a shared-memory state sits: index bits 4..7 are mapped
+// linearly into bits 0..3.  The 16 lanes of an 8-byte access differ in the
+// four lowest bits that are no target; the map was searched for the fewest
+// bank conflicts over the contiguous target runs that chains fuse to (none
+// for runs of up to three) and all target sets below bit 10.
+__device__ __forceinline__ uint32_t sw(uint32_t x) {
+  constexpr uint64_t f = [] {
+    const uint32_t img[4] = {15, 10, 12, 8};
+    uint64_t t = 0;
+    for (int i = 0; i < 16; ++i) {
+      uint32_t v = 0;
+      for (int b = 0; b < 4; ++b)
+        if ((i >> b) & 1) v ^= img[b];
+      t |= static_cast<uint64_t>(v) << (4 * i);
+    }
+    return t;
+  }();
+  return x ^ (static_cast<uint32_t>(f >> ((x >> 2) & 60u)) & 15u);
+}
+
+// amplitude x of a state in global (plain) or shared (swizzled) memory
+template <bool SHARED>
+__device__ __forceinline__ uint32_t at(uint32_t x) {
+  return SHARED ? sw(x) : x;
+}
+
+// psi <- A psi for a state in shared memory; A (row-major) in shared memory,
+// read two entries at a time (a broadcast); t ascending
+template <int W>
+__device__ __forceinline__ void smem_apply(float2* psi, int n, const uint8_t* t, const float2* A) {
   constexpr int D = 1 << W;
   int sorted[W];
-  uint64_t off[D];
+  uint32_t off[D];
 #pragma unroll
-  for (int b = 0; b < W; ++b) sorted[b] = order[b];
-#pragma unroll
-  for (int i = 1; i < W; ++i)
-#pragma unroll
-    for (int j = i; j > 0; --j)
-      if (sorted[j - 1] > sorted[j]) { const int t = sorted[j]; sorted[j] = sorted[j - 1]; sorted[j - 1] = t; }
+  for (int b = 0; b < W; ++b) sorted[b] = t[b];
 #pragma unroll
   for (int m = 0; m < D; ++m) {
-    uint64_t o = 0;
+    uint32_t o = 0;
 #pragma unroll
     for (int b = 0; b < W; ++b)
-      if ((m >> b) & 1) o |= 1ull << order[b];
-    off[m] = o;
+      if ((m >> b) & 1) o |= 1u << sorted[b];
+    off[m] = sw(o);                    // sw distributes over disjoint bits
   }
-  // B sets per thread per round, all of their 16 amplitudes loaded before
-  // any arithmetic: a state in global memory needs that many loads in
-  // flight per thread to cover the memory latency (a shared-memory state
-  // does not, and there the extra registers cost more than they save)
-  constexpr int B = (!GLOBAL || D >= 16) ? 1 : 16 / D;
-  const uint64_t sets = 1ull << (n - W);
-  const uint64_t stride = static_cast<uint64_t>(blockDim.x);
-  for (uint64_t s0 = threadIdx.x; s0 < sets; s0 += B * stride) {
-    uint64_t base[B];
-    float2 v[B][D];
+  const uint32_t sets = 1u << (n - W);
+  for (uint32_t s = threadIdx.x; s < sets; s += blockDim.x) {
+    const uint32_t base = sw(insert_zeros32(s, W, sorted));
+    float2 v[D];
 #pragma unroll
-    for (int b = 0; b < B; ++b) {
-      const uint64_t s = s0 + b * stride;
-      base[b] = insert_zeros(s < sets ? s : s0, W, sorted);
+    for (int m = 0; m < D; ++m) v[m] = psi[base ^ off[m]];
+    constexpr int RU = W <= 3 ? D : 4;
+#pragma unroll RU
+    for (int j = 0; j < D; ++j) {
+      float xr = 0.f, xi = 0.f;
 #pragma unroll
-      for (int m = 0; m < D; ++m) v[b][m] = psi[base[b] | off[m]];
-    }
-#pragma unroll
-    for (int b = 0; b < B; ++b) {
-      if (s0 + b * stride >= sets) break;
-#pragma unroll
-      for (int j = 0; j < D; ++j) {
-        float xr = 0.f, xi = 0.f;
-#pragma unroll
-        for (int m = 0; m < D; ++m) {
-          const float2 a = A[j * D + m];
-          xr = fmaf(a.x, v[b][m].x, fmaf(-a.y, v[b][m].y, xr));
-          xi = fmaf(a.x, v[b][m].y, fmaf(a.y, v[b][m].x, xi));
-        }
-        psi[base[b] | off[j]] = make_float2(xr, xi);
+      for (int m = 0; m < D; m += 2) {
+        const float4 a = *reinterpret_cast<const float4*>(A + j * D + m);
+        xr = fmaf(a.x, v[m].x, fmaf(-a.y, v[m].y, xr));
+        xi = fmaf(a.x, v[m].y, fmaf(a.y, v[m].x, xi));
+        xr = fmaf(a.z, v[m + 1].x, fmaf(-a.w, v[m + 1].y, xr));
+        xi = fmaf(a.z, v[m + 1].y, fmaf(a.w, v[m + 1].x, xi));
       }
+      psi[base ^ off[j]] = make_float2(xr, xi);
     }
   }
 }
@@ -170,23 +189,20 @@ __device__ void cta_apply_w(float2* psi, int n, const int* order, const float2* 
 // widths 5 and 6: one gather set per thread, its 2^w members in a local
 // array (registers or, at w = 6, local memory); kept out of line so that its
 // register demand does not raise that of the rest of the kernel
-template <int W>
+template <int W, bool SHARED>
 __device__ __noinline__ void cta_apply_wide(float2* psi, int n, const int* order, const float2* A) {
   constexpr int D = 1 << W;
   int sorted[W];
   for (int b = 0; b < W; ++b) sorted[b] = order[b];
-  for (int i = 1; i < W; ++i)
-    for (int j = i; j > 0; --j)
-      if (sorted[j - 1] > sorted[j]) { const int t = sorted[j]; sorted[j] = sorted[j - 1]; sorted[j - 1] = t; }
-  const uint64_t sets = 1ull << (n - W);
-  for (uint64_t s = threadIdx.x; s < sets; s += blockDim.x) {
-    const uint64_t base = insert_zeros(s, W, sorted);
+  const uint32_t sets = 1u << (n - W);
+  for (uint32_t s = threadIdx.x; s < sets; s += blockDim.x) {
+    const uint32_t base = insert_zeros32(s, W, sorted);
     float2 v[D];
     for (int m = 0; m < D; ++m) {
-      uint64_t o = 0;
+      uint32_t o = 0;
       for (int b = 0; b < W; ++b)
-        if ((m >> b) & 1) o |= 1ull << order[b];
-      v[m] = psi[base | o];
+        if ((m >> b) & 1) o |= 1u << order[b];
+      v[m] = psi[at<SHARED>(base | o)];
     }
     for (int j = 0; j < D; ++j) {
       float xr = 0.f, xi = 0.f;
@@ -195,20 +211,12 @@ __device__ __noinline__ void cta_apply_wide(float2* psi, int n, const int* order
         xr = fmaf(a.x, v[m].x, fmaf(-a.y, v[m].y, xr));
         xi = fmaf(a.x, v[m].y, fmaf(a.y, v[m].x, xi));
       }
-      uint64_t o = 0;
+      uint32_t o = 0;
       for (int b = 0; b < W; ++b)
-        if ((j >> b) & 1) o |= 1ull << order[b];
-      psi[base | o] = make_float2(xr, xi);
+        if ((j >> b) & 1) o |= 1u << order[b];
+      psi[at<SHARED>(base | o)] = make_float2(xr, xi);
     }
   }
-}
-
-__device__ __forceinline__ uint32_t insert_zeros32(uint32_t x, int w, const int* sorted) {
-  for (int b = 0; b < w; ++b) {
-    const int s = sorted[b];
-    x = ((x >> s) << (s + 1)) | (x & ((1u << s) - 1u));
-  }
-  return x;
 }
 
 // psi <- A psi for a state in global memory (n <= 20, so 32-bit indices):
@@ -277,20 +285,15 @@ __device__ __noinline__ void cta_apply_glob(float2* __restrict__ psi, int n, con
   }
 }
 
-// Aglob: the matrix in global memory (scaled by `scale` while staged), or
-// smat itself when the matrix was composed in shared memory (scale unused).
-template <bool GLOBAL>
-__device__ void cta_apply(float2* psi, int n, int w, const int* order, const float2* Aglob, float scale,
-                          float2* smat) {
+// Aglob: the matrix in global memory, or smat itself when it was composed there
+__device__ void cta_apply(float2* psi, int n, int w, const int* order, const float2* Aglob, float2* smat) {
   const int D = 1 << w;
-  const bool staged = Aglob == smat;
   __syncthreads();                     // previous users of smat / psi are done
-  if (GLOBAL && w <= 4) {
+  if (w <= 4) {
     float4* A4 = reinterpret_cast<float4*>(smat + (1u << (2 * kMaxW)));
     for (int i = threadIdx.x; i < D * D; i += blockDim.x) {
       const float2 a = Aglob[i];
-      const float x = staged ? a.x : a.x * scale, y = staged ? a.y : a.y * scale;
-      A4[i] = make_float4(x, x, y, y);
+      A4[i] = make_float4(a.x, a.x, a.y, a.y);
     }
     __syncthreads();
     switch (w) {
@@ -301,24 +304,12 @@ __device__ void cta_apply(float2* psi, int n, int w, const int* order, const flo
     }
     return;
   }
-  if (!staged) {
-    for (int i = threadIdx.x; i < D * D; i += blockDim.x) {
-      const float2 a = Aglob[i];
-      smat[i] = make_float2(a.x * scale, a.y * scale);
-    }
+  if (Aglob != smat) {
+    for (int i = threadIdx.x; i < D * D; i += blockDim.x) smat[i] = Aglob[i];
     __syncthreads();
   }
-  if (!GLOBAL) {
-    switch (w) {
-      case 1: cta_apply_w<1, false>(psi, n, order, smat); return;
-      case 2: cta_apply_w<2, false>(psi, n, order, smat); return;
-      case 3: cta_apply_w<3, false>(psi, n, order, smat); return;
-      case 4: cta_apply_w<4, false>(psi, n, order, smat); return;
-      default: break;
-    }
-  }
-  if (w == 5) cta_apply_wide<5>(psi, n, order, smat);
-  else cta_apply_wide<6>(psi, n, order, smat);
+  if (w == 5) cta_apply_wide<5, false>(psi, n, order, smat);
+  else cta_apply_wide<6, false>(psi, n, order, smat);
 }
 
 __device__ __forceinline__ float2 cmul_add(float2 a, float2 x, float2 acc) {
@@ -329,14 +320,15 @@ __device__ __forceinline__ float2 cmul_add(float2 a, float2 x, float2 acc) {
 
 // M <- A M for the 2^q x 2^q operator A (q = 1, 2; index bit b <-> pos[b]
 // among the w basis bits of M), scaled by sc: every column of M is a vector
-// that A acts on, as in Alg. 1.  M is D x D row-major in shared memory.
-__device__ void cta_left_apply(float2* M, int w, int q, const int* pos, const float2* A, float sc) {
+// that A acts on, as in Alg. 1.  M is D x D row-major in shared memory; the
+// caller is thread tid of the nt that share the work.
+__device__ void left_apply(float2* M, int w, int q, const int* pos, const float2* A, float sc, int tid, int nt) {
   const int D = 1 << w;
   if (q == 1) {
     const float2 a00 = make_float2(A[0].x * sc, A[0].y * sc), a01 = make_float2(A[1].x * sc, A[1].y * sc);
     const float2 a10 = make_float2(A[2].x * sc, A[2].y * sc), a11 = make_float2(A[3].x * sc, A[3].y * sc);
     const int p = pos[0];
-    for (int u = threadIdx.x; u < (D >> 1) * D; u += blockDim.x) {
+    for (int u = tid; u < (D >> 1) * D; u += nt) {
       const int c = u & (D - 1), rr = u >> w;
       const int r0 = ((rr >> p) << (p + 1)) | (rr & ((1 << p) - 1)), r1 = r0 | (1 << p);
       const float2 x0 = M[r0 * D + c], x1 = M[r1 * D + c];
@@ -346,7 +338,7 @@ __device__ void cta_left_apply(float2* M, int w, int q, const int* pos, const fl
     return;
   }
   const int lo = pos[0] < pos[1] ? pos[0] : pos[1], hi = pos[0] < pos[1] ? pos[1] : pos[0];
-  for (int u = threadIdx.x; u < (D >> 2) * D; u += blockDim.x) {
+  for (int u = tid; u < (D >> 2) * D; u += nt) {
     const int c = u & (D - 1);
     int r = u >> w;
     r = ((r >> lo) << (lo + 1)) | (r & ((1 << lo) - 1));
@@ -371,53 +363,65 @@ __device__ void cta_left_apply(float2* M, int w, int q, const int* pos, const fl
   }
 }
 
-// reduced density of (q0[, q1]) -> out[0..W) (layout of rdm_unpack); thread 0 holds the result
-__device__ void cta_rdm(const float2* psi, int n, int q, const int* order, double* out, double (*red)[17]) {
-  const int D = 1 << q, W = D * D;
-  double acc[16];
-  float f[16];
-  for (int c = 0; c < 16; ++c) { acc[c] = 0.0; f[c] = 0.f; }
-  int sorted[2] = {order[0], q > 1 ? order[1] : 0};
-  if (q > 1 && sorted[0] > sorted[1]) { const int t = sorted[0]; sorted[0] = sorted[1]; sorted[1] = t; }
-  uint64_t off[4];
+// Reduced density of the Q qubits order[] -> out[0..4^Q) (layout of
+// rdm_unpack), written by thread 0.  The sets are dealt to `lthreads` logical
+// threads, FP32 runs of 16 sets each, whatever the CTA's size: logical warp
+// after logical warp for the CTA's warps.  Carries in double-floats.
+template <int Q, bool SHARED>
+__device__ void cta_rdm(const float2* psi, int n, const int* order, int lthreads, double* out, float2 (*red)[16]) {
+  constexpr int D = 1 << Q, W = D * D;
+  int sorted[Q];
+  uint32_t off[D];
+  for (int b = 0; b < Q; ++b) sorted[b] = order[b];
+  if (Q > 1 && sorted[0] > sorted[Q - 1]) { const int t = sorted[0]; sorted[0] = sorted[Q - 1]; sorted[Q - 1] = t; }
+#pragma unroll
   for (int m = 0; m < D; ++m) {
-    uint64_t o = 0;
-    for (int b = 0; b < q; ++b)
-      if ((m >> b) & 1) o |= 1ull << order[b];
+    uint32_t o = 0;
+    for (int b = 0; b < Q; ++b)
+      if ((m >> b) & 1) o |= 1u << order[b];
     off[m] = o;
   }
-  const uint64_t sets = 1ull << (n - q);
-  int cnt = 0;
-  for (uint64_t s = threadIdx.x; s < sets; s += blockDim.x) {
-    const uint64_t base = insert_zeros(s, q, sorted);
-    float2 v[4];
-    for (int m = 0; m < D; ++m) v[m] = psi[base | off[m]];
-    int c = 0;
-    for (int b = 0; b < D; ++b) { f[c] = fmaf(v[b].x, v[b].x, fmaf(v[b].y, v[b].y, f[c])); ++c; }
-    for (int b = 0; b < D; ++b)
-      for (int a = b + 1; a < D; ++a) {
-        f[c] = fmaf(v[b].x, v[a].x, fmaf(v[b].y, v[a].y, f[c])); ++c;
-        f[c] = fmaf(v[b].y, v[a].x, fmaf(-v[b].x, v[a].y, f[c])); ++c;
+  const uint32_t sets = 1u << (n - Q);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5, lw = lthreads >> 5;
+  for (int l = warp; l < lw; l += nw) {
+    float2 acc[W];
+    float f[W];
+#pragma unroll
+    for (int c = 0; c < W; ++c) { acc[c] = make_float2(0.f, 0.f); f[c] = 0.f; }
+    int cnt = 0;
+    for (uint32_t s = l * 32 + lane; s < sets; s += lthreads) {
+      const uint32_t base = insert_zeros32(s, Q, sorted);
+      float2 v[D];
+#pragma unroll
+      for (int m = 0; m < D; ++m) v[m] = psi[at<SHARED>(base | off[m])];
+      int c = 0;
+#pragma unroll
+      for (int b = 0; b < D; ++b) { f[c] = fmaf(v[b].x, v[b].x, fmaf(v[b].y, v[b].y, f[c])); ++c; }
+#pragma unroll
+      for (int b = 0; b < D; ++b)
+#pragma unroll
+        for (int a = b + 1; a < D; ++a) {
+          f[c] = fmaf(v[b].x, v[a].x, fmaf(v[b].y, v[a].y, f[c])); ++c;
+          f[c] = fmaf(v[b].y, v[a].x, fmaf(-v[b].x, v[a].y, f[c])); ++c;
+        }
+      if (++cnt == 16) {
+#pragma unroll
+        for (int k = 0; k < W; ++k) { df_acc(acc[k].x, acc[k].y, f[k]); f[k] = 0.f; }
+        cnt = 0;
       }
-    if (++cnt == 16) {
-      for (int k = 0; k < W; ++k) { acc[k] += static_cast<double>(f[k]); f[k] = 0.f; }
-      cnt = 0;
     }
-  }
-  for (int k = 0; k < W; ++k) acc[k] += static_cast<double>(f[k]);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int k = 0; k < W; ++k) {
-    double v = acc[k];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) red[warp][k] = v;
+#pragma unroll
+    for (int k = 0; k < W; ++k) df_acc(acc[k].x, acc[k].y, f[k]);
+    const float2 r = df_warp_sum<W>(acc, lane);
+    constexpr int per = 32 / W;
+    if (lane % per == 0) red[l][lane / per] = r;
   }
   __syncthreads();
-  if (threadIdx.x == 0)
-    for (int k = 0; k < W; ++k) {
-      double v = 0.0;
-      for (int w2 = 0; w2 < nw; ++w2) v += red[w2][k];
-      out[k] = v;
-    }
+  if (threadIdx.x < W) {
+    float2 v = make_float2(0.f, 0.f);
+    for (int w2 = 0; w2 < lw; ++w2) v = df_add(v, red[w2][threadIdx.x]);
+    out[threadIdx.x] = df_value(v);
+  }
   __syncthreads();
 }
 
@@ -430,57 +434,116 @@ __device__ __forceinline__ float warp_scan_f(float v, int lane) {
   return v;
 }
 
-// S samples: warp w owns a contiguous range of amplitudes; C(x) inside a
-// range is the running FP32 sum of 32-amplitude chunk totals plus the
-// chunk's warp scan; ranges are chained by an FP64 scan of their totals
+// S samples.  The amplitudes are cut into one contiguous range per logical
+// warp (lthreads / 32 of them); C(x) inside a range is the running FP32 sum
+// of 32-amplitude chunk totals plus the chunk's warp scan; ranges are chained
+// by an FP64 scan of their totals.  While the ranges are summed, each group of
+// chunks (a chunk of its own up to 2^14 amplitudes) notes the sum before it
+// and its largest C, so that a sample finds its group with one vote of the
+// warp instead of scanning the range.  32 samples draw at once, a lane each;
+// FP64 compares with FP32 sums are made in FP32 against the target rounded
+// down (f > t exactly when f > rd(t)).
+constexpr int kSampleGroups = 512;
+struct SampleScratch {
+  double wcum[16];
+  float before[kSampleGroups], most[kSampleGroups];
+};
+
+template <bool SHARED>
 __device__ void cta_sample(const float2* psi, int n, uint64_t seed, uint64_t traj, uint32_t S, uint64_t* out,
-                           double* wcum) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const uint64_t amps = 1ull << n;
-  uint64_t per = (amps + nw - 1) / nw;
-  per = (per + 31) & ~31ull;
+                           int lthreads, SampleScratch& sc) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5, lw = lthreads >> 5;
+  const uint32_t amps = 1u << n;
+  uint32_t per = (amps + lw - 1) / lw;
+  per = (per + 31) & ~31u;
+  const int chunks = static_cast<int>(per / 32);
+  const int gpr = min(chunks, kSampleGroups / lw), gch = chunks / gpr;   // groups per range, chunks per group
+  auto weight = [&](uint32_t x) {
+    float w = 0.f;
+    if (x < amps) { const float2 a = psi[at<SHARED>(x)]; w = fmaf(a.x, a.x, a.y * a.y); }
+    return w;
+  };
   __syncthreads();
-  {
-    const uint64_t lo = warp * per;
+  for (int r = warp; r < lw; r += nw) {
+    const uint32_t lo = r * per;
     float run = 0.f;
-    for (uint64_t c = lo; c < lo + per; c += 32) {
-      const uint64_t x = c + lane;
-      float w = 0.f;
-      if (x < amps) { const float2 a = psi[x]; w = fmaf(a.x, a.x, a.y * a.y); }
-      const float inc = warp_scan_f(w, lane);
-      run += __shfl_sync(0xffffffffu, inc, 31);
+    for (int g = 0; g < gpr; ++g) {
+      const float before = run;
+      float most = 0.f;
+#pragma unroll 4
+      for (int c = 0; c < gch; ++c) {
+        const float inc = warp_scan_f(weight(lo + (g * gch + c) * 32 + lane), lane);
+        most = fmaxf(most, run + inc);
+        run += __shfl_sync(0xffffffffu, inc, 31);
+      }
+      most = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(most)));   // not negative
+      if (lane == 0) { sc.before[r * gpr + g] = before; sc.most[r * gpr + g] = most; }
     }
-    if (lane == 0) wcum[warp] = static_cast<double>(run);
+    if (lane == 0) sc.wcum[r] = static_cast<double>(run);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
     double r = 0.0;
-    for (int w = 0; w < nw; ++w) { r += wcum[w]; wcum[w] = r; }
+    for (int w = 0; w < lw; ++w) { r += sc.wcum[w]; sc.wcum[w] = r; }
   }
   __syncthreads();
-  const double total = wcum[nw - 1];
-  for (uint32_t j = warp; j < S; j += nw) {
-    const double t = uniform01(seed, traj, kStreamSample, j) * total;
-    int r = 0;
-    while (r < nw - 1 && !(t < wcum[r])) ++r;
-    const double trel = t - (r ? wcum[r - 1] : 0.0);
-    const uint64_t lo = r * per;
-    float run = 0.f;
-    uint64_t x = ~0ull, last_nz = lo < amps ? lo : amps - 1;
-    for (uint64_t c = lo; c < lo + per; c += 32) {
-      const uint64_t xx = c + lane;
-      float w = 0.f;
-      if (xx < amps) { const float2 a = psi[xx]; w = fmaf(a.x, a.x, a.y * a.y); }
-      const float inc = warp_scan_f(w, lane);
-      const float tot = __shfl_sync(0xffffffffu, inc, 31);
-      const unsigned nz = __ballot_sync(0xffffffffu, w > 0.f);
-      if (nz) last_nz = c + 31 - __clz(nz);
-      const unsigned h = __ballot_sync(0xffffffffu, trel < static_cast<double>(run + inc));
-      if (h) { x = c + __ffs(h) - 1; break; }
-      run += tot;
+  const double total = sc.wcum[lw - 1];
+  const uint32_t batch = min(max((S + nw - 1) / nw, 8u), 32u);   // samples a warp draws at once
+  for (uint32_t j0 = warp * batch; j0 < S; j0 += nw * batch) {
+    // lane: sample j0 + lane
+    int range = 0;
+    float below = 0.f;                                     // its target inside the range, rounded down
+    double trel = 0.0;
+    const bool own = lane < static_cast<int>(batch) && j0 + lane < S;
+    if (own) {
+      const double t = uniform01(seed, traj, kStreamSample, j0 + lane) * total;
+      int last = lw - 1;
+      while (range < last) {                               // first range whose end is above t
+        const int mid = (range + last) >> 1;
+        if (t < sc.wcum[mid]) last = mid; else range = mid + 1;
+      }
+      trel = t - (range ? sc.wcum[range - 1] : 0.0);
+      below = __double2float_rd(trel);
     }
-    if (x == ~0ull || x >= amps) x = last_nz;
-    if (lane == 0) out[j] = x;
+    uint64_t mine = 0;
+    for (uint32_t i = 0; i < batch && j0 + i < S; ++i) {
+      const int r = __shfl_sync(0xffffffffu, range, i);
+      const float b = __shfl_sync(0xffffffffu, below, i);
+      const uint32_t lo = r * per;
+      int g = gpr;
+      for (int g0 = 0; g0 < gpr && g == gpr; g0 += 32) {
+        const unsigned hit = __ballot_sync(0xffffffffu, g0 + lane < gpr && sc.most[r * gpr + g0 + lane] > b);
+        if (hit) g = g0 + __ffs(hit) - 1;
+      }
+      uint64_t x = ~0ull;
+      if (g < gpr) {
+        float run = sc.before[r * gpr + g];
+        for (int c = 0; c < gch; ++c) {
+          const uint32_t x0 = lo + (g * gch + c) * 32;
+          const float inc = warp_scan_f(weight(x0 + lane), lane);
+          const unsigned h = __ballot_sync(0xffffffffu, run + inc > b);
+          if (h) { x = x0 + __ffs(h) - 1; break; }
+          run += __shfl_sync(0xffffffffu, inc, 31);
+        }
+      }
+      if (x >= amps) {
+        // rounding put the target past the range (or past the state): its last
+        // amplitude of non-zero weight, up to the chunk that would hold the target
+        float run = 0.f;
+        uint32_t last_nz = lo < amps ? lo : amps - 1;
+        for (uint32_t c = lo; c < lo + per; c += 32) {
+          const float w = weight(c + lane);
+          const float inc = warp_scan_f(w, lane);
+          const unsigned nz = __ballot_sync(0xffffffffu, w > 0.f);
+          if (nz) last_nz = c + 31 - __clz(nz);
+          if (__ballot_sync(0xffffffffu, run + inc > b)) break;
+          run += __shfl_sync(0xffffffffu, inc, 31);
+        }
+        x = last_nz;
+      }
+      if (lane == static_cast<int>(i)) mine = x;
+    }
+    if (own) out[j0 + lane] = mine;
   }
 }
 
@@ -490,35 +553,71 @@ __device__ void cta_sample(const float2* psi, int n, uint64_t seed, uint64_t tra
 // in stage 2 at the segment's start (op pend_pos) enters as its Kraus
 // operator pend_choice scaled by pend_scale; any other channel as its
 // stage-1 choice.
-__device__ __forceinline__ void cta_compose_piece(const Dev& d, const Traj& T, const Gate& G, uint32_t lo, uint32_t hi,
-                                  int pend_pos, int pend_choice, float pend_scale, float2* s_mat) {
-  const int D = 1 << G.w;
-  __syncthreads();                 // previous users of s_mat are done
-  for (int i = threadIdx.x; i < D * D; i += blockDim.x)
+//
+// The members' descriptors and operators are first gathered by all threads
+// (the table walk is four dependent loads, paid once for 64 members instead
+// of by each); up to 3 qubits one warp then multiplies on, without barriers.
+constexpr int kListMax = 64;
+struct MemberList {
+  float2 A[kListMax][16];
+  float scale[kListMax];
+  int8_t q[kListMax], p0[kListMax], p1[kListMax];    // q = 0: not in the segment
+};
+
+__device__ __noinline__ void cta_compose_piece(const Dev& d, const Traj& T, const Gate& G, uint32_t lo, uint32_t hi,
+                                               int pend_pos, int pend_choice, float pend_scale, float2* s_mat,
+                                               MemberList& list) {
+  const int D = 1 << G.w, tid = threadIdx.x, nt = blockDim.x;
+  __syncthreads();                 // previous users of s_mat and list are done
+  for (int i = tid; i < D * D; i += nt)
     s_mat[i] = make_float2((i >> G.w) == (i & (D - 1)) ? 1.f : 0.f, 0.f);
-  for (uint32_t mi = 0; mi < G.nmem; ++mi) {
-    const uint32_t pos = d.members[G.mem0 + mi];
-    if (pos < lo || pos >= hi) continue;
-    const Op op = d.ops[T.op0 + pos];
-    const Set st = d.sets[op.set];
-    const uint32_t dd = 1u << (2 * op.q);
-    const float2* A;
-    float sc = 1.f;
-    if (op.channel < 0) {
-      A = d.fmat + st.mat;
-    } else if (static_cast<int>(pos) == pend_pos) {
-      A = d.fmat + st.kraus + pend_choice * dd;
-      sc = pend_scale;
-    } else {
-      A = d.fmat + st.mat + d.kraus[T.ch0 + op.channel] * dd;
+  for (uint32_t m0 = 0; m0 < G.nmem; m0 += kListMax) {
+    const int cnt = static_cast<int>(min(G.nmem - m0, static_cast<uint32_t>(kListMax)));
+    if (m0) __syncthreads();
+    for (int i = tid; i < cnt * 4; i += nt) {            // four threads a member, four entries each
+      const int mi = i >> 2, part = i & 3;
+      const uint32_t pos = d.members[G.mem0 + m0 + mi];
+      int q = 0;
+      if (pos >= lo && pos < hi) {
+        const Op op = d.ops[T.op0 + pos];
+        const Set st = d.sets[op.set];
+        q = op.q;
+        const uint32_t dd = 1u << (2 * q);
+        const float2* A;
+        float sc = 1.f;
+        if (op.channel < 0) {
+          A = d.fmat + st.mat;
+        } else if (static_cast<int>(pos) == pend_pos) {
+          A = d.fmat + st.kraus + pend_choice * dd;
+          sc = pend_scale;
+        } else {
+          A = d.fmat + st.mat + d.kraus[T.ch0 + op.channel] * dd;
+        }
+        for (uint32_t e = part * 4; e < part * 4 + 4 && e < dd; ++e) list.A[mi][e] = A[e];
+        if (part == 0) {
+          int p0 = 0, p1 = 0;
+          for (int b = 0; b < G.w; ++b) {
+            if (G.t[b] == op.q0) p0 = b;
+            if (q > 1 && G.t[b] == op.q1) p1 = b;
+          }
+          list.scale[mi] = sc;
+          list.p0[mi] = static_cast<int8_t>(p0);
+          list.p1[mi] = static_cast<int8_t>(p1);
+        }
+      }
+      if (part == 0) list.q[mi] = static_cast<int8_t>(q);
     }
-    int p[2] = {0, 0};
-    for (int b = 0; b < G.w; ++b) {
-      if (G.t[b] == op.q0) p[0] = b;
-      if (op.q > 1 && G.t[b] == op.q1) p[1] = b;
+    __syncthreads();
+    const bool one_warp = G.w <= 3;
+    if (one_warp && tid >= 32) continue;
+    for (int mi = 0; mi < cnt; ++mi) {
+      const int q = list.q[mi];
+      if (q == 0) continue;
+      const int p[2] = {list.p0[mi], list.p1[mi]};
+      left_apply(s_mat, G.w, q, p, list.A[mi], list.scale[mi], tid, one_warp ? 32 : nt);
+      if (one_warp) __syncwarp();
+      else __syncthreads();        // the member's update is complete
     }
-    __syncthreads();               // the previous member's update is complete
-    cta_left_apply(s_mat, G.w, op.q, p, A, sc);
   }
 }
 
@@ -561,7 +660,7 @@ __device__ __forceinline__ float2 fold_factor(const FoldPiece& F, const float2* 
 }
 
 __device__ __noinline__ int cta_product_start(const Dev& d, const Traj& T, float2* psi, uint32_t hi,
-                                              float2* s_mat, float2* s_col, FoldPiece* s_fold) {
+                                              float2* s_mat, float2* s_col, FoldPiece* s_fold, MemberList& list) {
   __shared__ int s_split, s_nstr;
   __shared__ uint8_t s_str[kMaxN];
   const int tid = threadIdx.x;
@@ -580,7 +679,7 @@ __device__ __noinline__ int cta_product_start(const Dev& d, const Traj& T, float
     const int D = 1 << G.w;
     const float2* col = d.fmat + G.mat;          // column 0 of the precomputed matrix, stride D
     if (G.maxpos >= hi || d.gflag[T.gf0 + g]) {
-      cta_compose_piece(d, T, G, 0, hi, -1, 0, 1.f, s_mat);
+      cta_compose_piece(d, T, G, 0, hi, -1, 0, 1.f, s_mat, list);
       __syncthreads();
       col = s_mat;
     }
@@ -652,207 +751,337 @@ __device__ __noinline__ int cta_product_start(const Dev& d, const Traj& T, float
   return nf;
 }
 
-__device__ __forceinline__ int decide_stage1(const Set& st, const double* pbar, double r) {
-  double rr = r;
-  for (uint32_t i = 0; i < st.nk; ++i) {
-    if (rr < pbar[i]) return static_cast<int>(i);
-    rr -= pbar[i];
+// ---------------------------------------------------------------------------
+// the persistent kernels
+// ---------------------------------------------------------------------------
+// Flush points of the trajectory that a CTA works on: channels that stage 1
+// leaves undecided, in no order (past kFlushMax they are found in the stage
+// records instead).
+constexpr int kFlushMax = 64;
+struct TrajShared {
+  float2 red[16][16];
+  double rho[16];
+  SampleScratch sample;
+  MemberList list;
+  unsigned idx;
+  int nflush;                       // entries of flush[] (more than kFlushMax: overflowed)
+  uint32_t flush[kFlushMax];
+  int next;
+  float scale;
+  int pend_pos, pend_choice;
+};
+
+// Stage 1 of every channel from its draw and the lower bounds; fused gates
+// that hold a channel with another operator than its default (or an undecided
+// one) get their flag, so that the pass loop reads one flag per gate.  Nearly
+// every draw takes the first operator, which an integer compare settles.
+__device__ __forceinline__ void cta_stage1(const Dev& d, const Traj& T, uint64_t seed, uint64_t traj_id, TrajShared& sh) {
+  const int tid = threadIdx.x;
+  for (uint32_t g = tid; g < T.ngates; g += blockDim.x) d.gflag[T.gf0 + g] = 0;
+  if (tid == 0) { sh.pend_pos = -1; sh.pend_choice = 0; sh.scale = 1.f; sh.nflush = 0; }
+  __syncthreads();
+#pragma unroll 2
+  for (uint32_t c = tid; c < T.nch; c += blockDim.x) {
+    const Op op = d.ops[T.op0 + d.ch_op[T.chop0 + c]];
+    const Set& st = d.sets[op.set];
+    const uint64_t bits = uniform_bits(seed, traj_id, kStreamChannel, c);
+    int ch = -1;
+    if (bits < st.thr0) {
+      ch = 0;
+    } else {
+      const double* pbar = d.dmat + st.pbar;
+      double rr = static_cast<double>(bits) * 0x1.0p-53 - pbar[0];
+      for (uint32_t i = 1; i < st.nk; ++i) {
+        if (rr < pbar[i]) { ch = static_cast<int>(i); break; }
+        rr -= pbar[i];
+      }
+    }
+    d.kraus[T.ch0 + c] = ch;
+    d.stage[T.ch0 + c] = ch >= 0 ? 1 : 0;
+    if (ch != static_cast<int>(st.def)) d.gflag[T.gf0 + op.gate] = 1;
+    if (ch < 0) {
+      const int k = atomicAdd(&sh.nflush, 1);
+      if (k < kFlushMax) sh.flush[k] = c;
+    }
   }
-  return -1;
+  __syncthreads();
 }
 
-// ---------------------------------------------------------------------------
-// the persistent kernel
-// ---------------------------------------------------------------------------
-// GLOBAL = false: the launch's trajectories have states of <= 2^14 amplitudes,
-// held in the CTA's shared memory; GLOBAL = true: larger states, held in a
-// per-CTA slot of global memory (shared memory then holds only the matrix)
-template <bool GLOBAL>
-__global__ void __launch_bounds__(512) k_batch(const __grid_constant__ Dev d) {
-  extern __shared__ __align__(16) float2 s_dyn[];
-  float2* s_state = s_dyn;
-  float2* s_mat = GLOBAL ? s_dyn : s_dyn + (1u << kSmemNMax);   // the pass's matrix, up to 64 x 64
-  __shared__ double s_red[32][17];
-  __shared__ double s_rho[16];
-  __shared__ double s_wcum[32];
-  __shared__ unsigned s_idx;
-  __shared__ int s_next;
-  __shared__ float s_scale;
-  __shared__ int s_pend_pos, s_pend_choice;
-  __shared__ float2 s_col[kFoldCols];               // columns U[:, 0] of the folded pieces
-  __shared__ FoldPiece s_fold[kMaxN];
-  const int tid = threadIdx.x;
+// first flush point at or after channel cur, -1 if there is none
+__device__ __forceinline__ int cta_next_flush(const Dev& d, const Traj& T, uint32_t cur, TrajShared& sh) {
+  if (threadIdx.x < 32) {
+    uint32_t best = 0xffffffffu;
+    if (sh.nflush <= kFlushMax) {
+      for (int i = threadIdx.x; i < sh.nflush; i += 32)
+        if (sh.flush[i] >= cur) best = min(best, sh.flush[i]);
+    } else {
+      for (uint32_t c = cur + threadIdx.x; c < T.nch; c += 32)
+        if (d.stage[T.ch0 + c] == 0) { best = c; break; }
+    }
+    best = __reduce_min_sync(0xffffffffu, best);
+    if (threadIdx.x == 0) sh.next = static_cast<int>(best);
+  }
+  __syncthreads();
+  return sh.next;
+}
 
-  for (;;) {
-    __syncthreads();
-    if (tid == 0) s_idx = atomicAdd(d.counter, 1u);
-    __syncthreads();
-    const unsigned k = s_idx;
-    if (k >= d.num) break;
-    const uint32_t ti = d.order[k];
+// Stage 2 at the flush point: op hi, channel fch (Alg. 2 steps 12-20)
+template <bool SHARED>
+__device__ __noinline__ void cta_stage2(const Dev& d, const Traj& T, const float2* psi, uint32_t hi, int fch, uint64_t seed,
+                                        uint64_t traj_id, TrajShared& sh) {
+  const Op op = d.ops[T.op0 + hi];
+  const Set st = d.sets[op.set];
+  const int order[2] = {op.q0, op.q1};
+  __syncthreads();
+  if (op.q == 1) cta_rdm<1, SHARED>(psi, static_cast<int>(T.n), order, static_cast<int>(d.lthreads), sh.rho, sh.red);
+  else cta_rdm<2, SHARED>(psi, static_cast<int>(T.n), order, static_cast<int>(d.lthreads), sh.rho, sh.red);
+  if (threadIdx.x == 0) {
+    const int D = 1 << op.q;
+    double rho[2 * 16];
+    int c = 0;
+    for (int b = 0; b < D; ++b) { rho[2 * (b * D + b)] = sh.rho[c++]; rho[2 * (b * D + b) + 1] = 0.0; }
+    for (int b = 0; b < D; ++b)
+      for (int a = b + 1; a < D; ++a) {
+        const double re = sh.rho[c++], im = sh.rho[c++];
+        rho[2 * (b * D + a)] = re; rho[2 * (b * D + a) + 1] = im;
+        rho[2 * (a * D + b)] = re; rho[2 * (a * D + b) + 1] = -im;
+      }
+    double N = 0.0;
+    for (int b = 0; b < D; ++b) N += rho[2 * (b * D + b)];
+    const double* pbar = d.dmat + st.pbar;
+    double rr = uniform01(seed, traj_id, kStreamChannel, static_cast<uint32_t>(fch));
+    for (uint32_t i = 0; i < st.nk; ++i) rr -= pbar[i];
+    int chosen = -1, last = -1, last_pos = -1;
+    double Pc = 1.0;
+    for (uint32_t i = 0; i < st.nk; ++i) {
+      const double* M = d.dmat + st.mtm + static_cast<size_t>(i) * D * D * 2;
+      double P = 0.0;                                  // tr(M rho)
+      for (int a = 0; a < D; ++a)
+        for (int b = 0; b < D; ++b) {
+          const double mr = M[2 * (a * D + b)], mi2 = M[2 * (a * D + b) + 1];
+          const double rr2 = rho[2 * (b * D + a)], ri = rho[2 * (b * D + a) + 1];
+          P += mr * rr2 - mi2 * ri;
+        }
+      double dlt = P / N - pbar[i];
+      if (dlt < 0.0) dlt = 0.0;
+      if (dlt > 0.0) last = static_cast<int>(i);
+      if (P > 0.0) last_pos = static_cast<int>(i);
+      if (chosen < 0 && rr < dlt) { chosen = static_cast<int>(i); Pc = P; }
+      if (chosen < 0) rr -= dlt;
+    }
+    if (chosen < 0) {
+      chosen = last >= 0 ? last : (last_pos >= 0 ? last_pos : static_cast<int>(st.def));
+      const double* M = d.dmat + st.mtm + static_cast<size_t>(chosen) * D * D * 2;
+      Pc = 0.0;
+      for (int a = 0; a < D; ++a)
+        for (int b = 0; b < D; ++b)
+          Pc += M[2 * (a * D + b)] * rho[2 * (b * D + a)] - M[2 * (a * D + b) + 1] * rho[2 * (b * D + a) + 1];
+    }
+    d.kraus[T.ch0 + fch] = chosen;
+    d.stage[T.ch0 + fch] = 2;
+    sh.pend_pos = static_cast<int>(hi);
+    sh.pend_choice = chosen;
+    sh.scale = static_cast<float>(1.0 / sqrt(Pc > 0.0 ? Pc : 1.0));
+  }
+  __syncthreads();
+}
+
+// the next trajectory of the launch; false when there is none left
+__device__ __forceinline__ bool next_trajectory(const Dev& d, TrajShared& sh, uint32_t& ti) {
+  __syncthreads();
+  if (threadIdx.x == 0) sh.idx = atomicAdd(d.counter, 1u);
+  __syncthreads();
+  if (sh.idx >= d.num) return false;
+  ti = d.order[sh.idx];
+  return true;
+}
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// States of at most 2^14 amplitudes, held in the CTA's shared memory.  Passes
+// are short (2^n / 2^w sets over a few hundred threads), so what bounds them
+// is latency: the CTA is sized to the state (128 threads up to 10 qubits, 256
+// up to 13, 512 at 14) so that several trajectories share an SM; a window of
+// gate descriptors with what to do about each is brought to shared memory at
+// once; and the matrix of the next gate is copied (cp.async, two buffers)
+// while this one is applied, which leaves one barrier per gate.
+// 1600 trajectories of 8 to 12 qubits, k = 3: 4.14 -> 0.90 ms of device time
+// (every state had one CTA of 512 threads per SM before, and each gate fetched
+// its descriptor, flag and matrix in turn between two barriers).  Now 40 % of
+// the issue slots; 4 CTAs of 256 threads at 64 registers, or CTAs of 128
+// threads from 11 qubits on, measured 2-3 % slower.
+constexpr int kWindow = 128;        // gates of a descriptor window
+enum : uint8_t { kSkip = 0, kDefault = 1, kCompose = 2 };
+
+template <int TB, int MINB>
+__global__ void __launch_bounds__(TB, MINB) k_batch_smem(const __grid_constant__ Dev d, uint32_t max_amps) {
+  extern __shared__ __align__(16) float2 s_dyn[];
+  __shared__ TrajShared sh;
+  __shared__ Gate s_gate[kWindow];
+  __shared__ uint8_t s_kind[kWindow];
+  float2* const psi = s_dyn;
+  const uint32_t wbuf = min(d.wmat, 4u);
+  float2* const buf = s_dyn + max_amps;                  // two matrices of up to 2^wbuf
+  float2* const big = buf + (2u << (2 * wbuf));          // one wider matrix (wmat > 4)
+  const int tid = threadIdx.x;
+  uint32_t ti;
+  while (next_trajectory(d, sh, ti)) {
     const Traj T = d.traj[ti];
     const int n = static_cast<int>(T.n);
-    const uint64_t amps = 1ull << n;
+    const uint32_t amps = 1u << n;
     const uint64_t seed = d.per_traj ? T.seed : d.run[0];
     const uint64_t traj_id = d.per_traj ? T.tid : d.run[1] + ti;
     const uint32_t S = d.per_traj ? T.S : d.S;
     uint64_t* samples = d.samples + (d.per_traj ? T.soff : static_cast<uint64_t>(ti) * d.S);
-    float2* psi;
-    if (!GLOBAL) psi = s_state;
-    else psi = d.keep ? d.arena + T.arena_off : d.arena + static_cast<uint64_t>(blockIdx.x) * d.slot_amps;
-    // shared-memory states start from |0...0>; global-memory states from the
-    // product state that the first segment writes (cta_product_start)
-    if (!GLOBAL)
-      for (uint64_t x = tid; x < amps; x += blockDim.x) psi[x] = make_float2(x == 0 ? 1.f : 0.f, 0.f);
-    // stage 1 of every channel from its draw and the lower bounds
-    for (uint32_t c = tid; c < T.nch; c += blockDim.x) {
-      const Op op = d.ops[T.op0 + d.ch_op[T.chop0 + c]];
-      const Set st = d.sets[op.set];
-      const double r = uniform01(seed, traj_id, kStreamChannel, c);
-      const int ch = decide_stage1(st, d.dmat + st.pbar, r);
-      d.kraus[T.ch0 + c] = ch;
-      d.stage[T.ch0 + c] = ch >= 0 ? 1 : 0;
-    }
-    if (tid == 0) { s_pend_pos = -1; s_pend_choice = 0; s_scale = 1.f; }
-    __syncthreads();
-    // which fused gates cannot use their precomputed matrix because a member
-    // channel took a non-default stage-1 choice (or none): decided once per
-    // trajectory, one gate per thread, so that the pass loop below reads one
-    // flag per gate instead of chasing each member's tables
-    for (uint32_t g = tid; g < T.ngates; g += blockDim.x) {
-      const Gate G = d.gates[T.gate0 + g];
-      uint8_t fl = 0;
-      for (uint32_t mi = 0; mi < G.nmem && !fl; ++mi) {
-        const Op op = d.ops[T.op0 + d.members[G.mem0 + mi]];
-        if (op.channel >= 0 && d.kraus[T.ch0 + op.channel] != static_cast<int>(d.sets[op.set].def)) fl = 1;
-      }
-      d.gflag[T.gf0 + g] = fl;
-    }
-    __syncthreads();
+    for (uint32_t x = tid; x < amps; x += blockDim.x) psi[x] = make_float2(x == 0 ? 1.f : 0.f, 0.f);   // sw(0) = 0
+    cta_stage1(d, T, seed, traj_id, sh);
     uint32_t lo = 0, cur_ch = 0, nflush = 0;
     for (;;) {
-      // next flush point
-      if (tid == 0) {
-        int nx = -1;
-        for (uint32_t c = cur_ch; c < T.nch; ++c)
-          if (d.stage[T.ch0 + c] == 0) { nx = static_cast<int>(c); break; }
-        s_next = nx;
-      }
-      __syncthreads();
-      const int fch = s_next;
+      const int fch = cta_next_flush(d, T, cur_ch, sh);
       const uint32_t hi = fch >= 0 ? d.ch_op[T.chop0 + fch] : T.nops;
-      const int pend_pos = s_pend_pos, pend_choice = s_pend_choice;
-      const float pend_scale = s_scale;
-      // the product-state start pays on global-memory states, where a pass
-      // streams the state from DRAM; on shared-memory states (passes of a few
-      // microseconds) it measured slower than the passes it saves
-      const bool first = GLOBAL && lo == 0 && nflush == 0;
-      if constexpr (GLOBAL) {
-        if (first) {
-          const int nf = cta_product_start(d, T, psi, hi, s_mat, s_col, s_fold);
-          if (tid == 0 && d.folds) d.folds[ti] = static_cast<uint32_t>(nf);
+      const int pend_pos = sh.pend_pos, pend_choice = sh.pend_choice;
+      const float pend_scale = sh.scale;
+      // the channel decided in stage 2 at this segment's start is applied as
+      // its normalized Kraus operator, so the gate holding it is never default
+      const uint32_t pend_gate = pend_pos >= 0 ? d.ops[T.op0 + pend_pos].gate : 0xffffffffu;
+      // apply ops [lo, hi): fused gates restricted to the segment
+      for (uint32_t g0 = 0; g0 < T.ngates; g0 += kWindow) {
+        const int cnt = static_cast<int>(min(T.ngates - g0, static_cast<uint32_t>(kWindow)));
+        __syncthreads();                                 // the previous window and its buffers are done with
+        for (int i = tid; i < cnt; i += TB) {
+          const Gate G = d.gates[T.gate0 + g0 + i];
+          uint8_t kind = kSkip;
+          if (G.maxpos >= lo && G.minpos < hi)
+            kind = G.minpos >= lo && G.maxpos < hi && !d.gflag[T.gf0 + g0 + i] && g0 + i != pend_gate ? kDefault : kCompose;
+          s_gate[i] = G;
+          s_kind[i] = kind;
         }
+        __syncthreads();
+        auto next_active = [&](int g) {
+          while (g < cnt && s_kind[g] == kSkip) ++g;
+          return g;
+        };
+        auto prefetch = [&](int g, int b) {              // a default gate's matrix into buffer b
+          if (g < cnt && s_kind[g] == kDefault && s_gate[g].w <= 4) {
+            const float2* src = d.fmat + s_gate[g].mat;
+            float2* dst = buf + (static_cast<uint32_t>(b) << (2 * wbuf));
+            const int words = 1 << (2 * s_gate[g].w - 1);
+            for (int i = tid; i < words; i += TB) cp_async16(dst + 2 * i, src + 2 * i);
+          }
+        };
+        int g = next_active(0), b = 0;
+        prefetch(g, 0);
+        while (g < cnt) {
+          const int w = s_gate[g].w;
+          float2* A = w <= 4 ? buf + (static_cast<uint32_t>(b) << (2 * wbuf)) : big;
+          if (s_kind[g] == kCompose) {
+            // a piece that is cut by the segment or holds a non-default operator:
+            // its members in [lo, hi) as one matrix over the gate's qubits
+            const Gate G = s_gate[g];
+            cta_compose_piece(d, T, G, lo, hi, pend_pos, pend_choice, pend_scale, A, sh.list);
+          } else if (w > 4) {
+            __syncthreads();
+            const float2* src = d.fmat + s_gate[g].mat;
+            for (int i = tid; i < 1 << (2 * w); i += TB) A[i] = src[i];
+          } else {
+            cp_async_wait();
+          }
+          __syncthreads();                               // the matrix is there; the previous pass is complete
+          const int nx = next_active(g + 1);
+          prefetch(nx, b ^ 1);
+          const uint8_t* t = s_gate[g].t;
+          switch (w) {
+            case 1: smem_apply<1>(psi, n, t, A); break;
+            case 2: smem_apply<2>(psi, n, t, A); break;
+            case 3: smem_apply<3>(psi, n, t, A); break;
+            case 4: smem_apply<4>(psi, n, t, A); break;
+            default: {
+              int order[kMaxW];
+              for (int k = 0; k < w; ++k) order[k] = t[k];
+              if (w == 5) cta_apply_wide<5, true>(psi, n, order, A);
+              else cta_apply_wide<6, true>(psi, n, order, A);
+            }
+          }
+          g = nx;
+          b ^= 1;
+        }
+      }
+      if (fch < 0) break;
+      cta_stage2<true>(d, T, psi, hi, fch, seed, traj_id, sh);
+      ++nflush;
+      lo = hi;
+      cur_ch = static_cast<uint32_t>(fch) + 1;
+    }
+    __syncthreads();
+    if (S) cta_sample<true>(psi, n, seed, traj_id, S, samples, static_cast<int>(d.lthreads), sh.sample);
+    if (d.keep)
+      for (uint32_t x = tid; x < amps; x += blockDim.x) d.arena[T.arena_off + x] = psi[sw(x)];
+    if (tid == 0) {
+      d.flushes[ti] = nflush;
+      if (d.folds) d.folds[ti] = 0;
+    }
+  }
+}
+
+// Larger states, each in its CTA's slot of global memory
+__global__ void __launch_bounds__(512) k_batch_glob(const __grid_constant__ Dev d) {
+  extern __shared__ __align__(16) float2 s_dyn[];
+  float2* s_mat = s_dyn;                            // the pass's matrix, up to 64 x 64
+  __shared__ TrajShared sh;
+  __shared__ float2 s_col[kFoldCols];               // columns U[:, 0] of the folded pieces
+  __shared__ FoldPiece s_fold[kMaxN];
+  const int tid = threadIdx.x;
+  uint32_t ti;
+  while (next_trajectory(d, sh, ti)) {
+    const Traj T = d.traj[ti];
+    const int n = static_cast<int>(T.n);
+    const uint64_t seed = d.per_traj ? T.seed : d.run[0];
+    const uint64_t traj_id = d.per_traj ? T.tid : d.run[1] + ti;
+    const uint32_t S = d.per_traj ? T.S : d.S;
+    uint64_t* samples = d.samples + (d.per_traj ? T.soff : static_cast<uint64_t>(ti) * d.S);
+    float2* psi = d.keep ? d.arena + T.arena_off : d.arena + static_cast<uint64_t>(blockIdx.x) * d.slot_amps;
+    cta_stage1(d, T, seed, traj_id, sh);
+    uint32_t lo = 0, cur_ch = 0, nflush = 0;
+    for (;;) {
+      const int fch = cta_next_flush(d, T, cur_ch, sh);
+      const uint32_t hi = fch >= 0 ? d.ch_op[T.chop0 + fch] : T.nops;
+      const int pend_pos = sh.pend_pos, pend_choice = sh.pend_choice;
+      const float pend_scale = sh.scale;
+      const uint32_t pend_gate = pend_pos >= 0 ? d.ops[T.op0 + pend_pos].gate : 0xffffffffu;
+      const bool first = lo == 0 && nflush == 0;
+      if (first) {
+        const int nf = cta_product_start(d, T, psi, hi, s_mat, s_col, s_fold, sh.list);
+        if (tid == 0 && d.folds) d.folds[ti] = static_cast<uint32_t>(nf);
       }
       // apply ops [lo, hi): fused gates restricted to the segment (in the
       // first segment, those not folded into the initial state)
       for (uint32_t g = 0; g < T.ngates; ++g) {
         const Gate G = d.gates[T.gate0 + g];
         if (G.maxpos < lo || G.minpos >= hi) continue;
-        if (first && d.gflag[T.gf0 + g] == 2) continue;
-        bool dflt = G.minpos >= lo && G.maxpos < hi && !d.gflag[T.gf0 + g];
-        // the channel decided in stage 2 at this segment's start is applied as
-        // its normalized Kraus operator, so the gate holding it is never default
-        if (dflt && pend_pos >= 0 && static_cast<uint32_t>(pend_pos) >= G.minpos &&
-            static_cast<uint32_t>(pend_pos) <= G.maxpos)
-          for (uint32_t mi = 0; dflt && mi < G.nmem; ++mi)
-            if (static_cast<int>(d.members[G.mem0 + mi]) == pend_pos) dflt = false;
-        if (dflt) {
-          int order[kMaxW];
-          for (int b = 0; b < G.w; ++b) order[b] = G.t[b];
-          cta_apply<GLOBAL>(psi, n, G.w, order, d.fmat + G.mat, 1.f, s_mat);
-          continue;
-        }
-        // a piece that is cut by the segment or holds a non-default operator:
-        // its members in [lo, hi) are composed in FP32 in shared memory into
-        // one matrix over the gate's qubits (identity on qubits none of them
-        // touches), then applied in one pass
-        cta_compose_piece(d, T, G, lo, hi, pend_pos, pend_choice, pend_scale, s_mat);
+        const uint8_t flag = d.gflag[T.gf0 + g];
+        if (first && flag == 2) continue;
         int order[kMaxW];
         for (int b = 0; b < G.w; ++b) order[b] = G.t[b];
-        cta_apply<GLOBAL>(psi, n, G.w, order, s_mat, 1.f, s_mat);
+        if (G.minpos >= lo && G.maxpos < hi && !flag && g != pend_gate) {
+          cta_apply(psi, n, G.w, order, d.fmat + G.mat, s_mat);
+          continue;
+        }
+        cta_compose_piece(d, T, G, lo, hi, pend_pos, pend_choice, pend_scale, s_mat, sh.list);
+        cta_apply(psi, n, G.w, order, s_mat, s_mat);
       }
       if (fch < 0) break;
-      // stage 2 at the flush point (Alg. 2 steps 12-20)
-      {
-        const Op op = d.ops[T.op0 + hi];
-        const Set st = d.sets[op.set];
-        int order[2] = {op.q0, op.q1};
-        __syncthreads();
-        cta_rdm(psi, n, op.q, order, s_rho, s_red);
-        if (tid == 0) {
-          const int D = 1 << op.q;
-          double rho[2 * 16];
-          int c = 0;
-          for (int b = 0; b < D; ++b) { rho[2 * (b * D + b)] = s_rho[c++]; rho[2 * (b * D + b) + 1] = 0.0; }
-          for (int b = 0; b < D; ++b)
-            for (int a = b + 1; a < D; ++a) {
-              const double re = s_rho[c++], im = s_rho[c++];
-              rho[2 * (b * D + a)] = re; rho[2 * (b * D + a) + 1] = im;
-              rho[2 * (a * D + b)] = re; rho[2 * (a * D + b) + 1] = -im;
-            }
-          double N = 0.0;
-          for (int b = 0; b < D; ++b) N += rho[2 * (b * D + b)];
-          const double* pbar = d.dmat + st.pbar;
-          double rr = uniform01(seed, traj_id, kStreamChannel, static_cast<uint32_t>(fch));
-          for (uint32_t i = 0; i < st.nk; ++i) rr -= pbar[i];
-          int chosen = -1, last = -1, last_pos = -1;
-          double Pc = 1.0;
-          for (uint32_t i = 0; i < st.nk; ++i) {
-            const double* M = d.dmat + st.mtm + static_cast<size_t>(i) * D * D * 2;
-            double P = 0.0;                                  // tr(M rho)
-            for (int a = 0; a < D; ++a)
-              for (int b = 0; b < D; ++b) {
-                const double mr = M[2 * (a * D + b)], mi2 = M[2 * (a * D + b) + 1];
-                const double rr2 = rho[2 * (b * D + a)], ri = rho[2 * (b * D + a) + 1];
-                P += mr * rr2 - mi2 * ri;
-              }
-            double dlt = P / N - pbar[i];
-            if (dlt < 0.0) dlt = 0.0;
-            if (dlt > 0.0) last = static_cast<int>(i);
-            if (P > 0.0) last_pos = static_cast<int>(i);
-            if (chosen < 0 && rr < dlt) { chosen = static_cast<int>(i); Pc = P; }
-            if (chosen < 0) rr -= dlt;
-          }
-          if (chosen < 0) {
-            chosen = last >= 0 ? last : (last_pos >= 0 ? last_pos : static_cast<int>(st.def));
-            const double* M = d.dmat + st.mtm + static_cast<size_t>(chosen) * D * D * 2;
-            Pc = 0.0;
-            for (int a = 0; a < D; ++a)
-              for (int b = 0; b < D; ++b)
-                Pc += M[2 * (a * D + b)] * rho[2 * (b * D + a)] - M[2 * (a * D + b) + 1] * rho[2 * (b * D + a) + 1];
-          }
-          d.kraus[T.ch0 + fch] = chosen;
-          d.stage[T.ch0 + fch] = 2;
-          s_pend_pos = static_cast<int>(hi);
-          s_pend_choice = chosen;
-          s_scale = static_cast<float>(1.0 / sqrt(Pc > 0.0 ? Pc : 1.0));
-        }
-        __syncthreads();
-        ++nflush;
-        lo = hi;
-        cur_ch = static_cast<uint32_t>(fch) + 1;
-      }
+      cta_stage2<false>(d, T, psi, hi, fch, seed, traj_id, sh);
+      ++nflush;
+      lo = hi;
+      cur_ch = static_cast<uint32_t>(fch) + 1;
     }
     __syncthreads();
-    if (S) cta_sample(psi, n, seed, traj_id, S, samples, s_wcum);
-    if (d.keep && !GLOBAL) {
-      __syncthreads();
-      for (uint64_t x = tid; x < amps; x += blockDim.x) d.arena[T.arena_off + x] = psi[x];
-    }
-    if (tid == 0) {
-      d.flushes[ti] = nflush;
-      if (!GLOBAL && d.folds) d.folds[ti] = 0;
-    }
+    if (S) cta_sample<false>(psi, n, seed, traj_id, S, samples, static_cast<int>(d.lthreads), sh.sample);
+    if (tid == 0) d.flushes[ti] = nflush;
   }
 }
 
@@ -919,7 +1148,7 @@ struct qt_batch {
   std::vector<bt::Traj> traj;
   std::vector<uint32_t> order;
   DevMem tables, arena, outs, counter;
-  uint64_t* hrun = nullptr;         // pinned {seed, first_traj}; the graph copies it to counter+16
+  uint64_t* hrun = nullptr;         // pinned {seed, first_traj}; the graph copies it to counter+32
   bt::Dev dev{};
   size_t off_kraus = 0, off_stage = 0, off_samples = 0, off_flushes = 0, off_folds = 0, off_err = 0, off_gflag = 0;
   uint64_t total_gates = 0;         // sum of the trajectories' fused-gate counts (one flag each per run)
@@ -933,12 +1162,13 @@ struct qt_batch {
   std::vector<uint32_t> flushes, folds;
   double device_ms = 0.0;
   uint64_t gate_ops = 0, fused_gates = 0;
-  // trajectories with states in global memory (n > 14) come first in `order`;
-  // the two classes run as two persistent launches, the second on a side
-  // stream so that its CTAs take SMs as the first launch's CTAs retire
-  uint32_t nglob = 0;
-  cudaStream_t side = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  // Classes of trajectories by state size, largest first as in `order`: states
+  // in global memory (n > 14), then shared-memory states of 14, 13, 11..12 and
+  // up to 10 qubits.  Each is one persistent launch, on streams of their own so
+  // that their CTAs share the SMs.
+  uint32_t count[bt::kClasses] = {}, wmat[bt::kClasses] = {}, top_n[bt::kClasses] = {};
+  cudaStream_t side[bt::kClasses - 1] = {};
+  cudaEvent_t ev_fork = nullptr, ev_join[bt::kClasses - 1] = {};
   // CUDA graph of the launch sequence
   cudaGraphExec_t gexec = nullptr;
   cudaGraph_t graph = nullptr;
@@ -948,8 +1178,10 @@ struct qt_batch {
     if (graph) cudaGraphDestroy(graph);
     if (hrun) cudaFreeHost(hrun);
     if (ev_fork) cudaEventDestroy(ev_fork);
-    if (ev_join) cudaEventDestroy(ev_join);
-    if (side) cudaStreamDestroy(side);
+    for (auto e : ev_join)
+      if (e) cudaEventDestroy(e);
+    for (auto st : side)
+      if (st) cudaStreamDestroy(st);
   }
 };
 
@@ -964,7 +1196,7 @@ static qt_status pack_batch(qt_batch* B, uint32_t num, const qt_fused* const* fu
   B->total_ch = 0;
   B->total_amps = 0;
   B->max_n = 0;
-  B->nglob = 0;
+  for (int c = 0; c < bt::kClasses; ++c) B->count[c] = B->wmat[c] = B->top_n[c] = 0;
   B->total_gates = 0;
   B->gate_ops = 0;
   B->fused_gates = 0;
@@ -1047,6 +1279,7 @@ static qt_status pack_batch(qt_batch* B, uint32_t num, const qt_fused* const* fu
       if (op.channel >= 0) ch_op.push_back(oi);
       if (op.kind == QT_OP_GATE) B->gate_ops++;
     }
+    for (uint32_t oi = 0; oi < c.ops.size(); ++oi) ops[T.op0 + oi].gate = f->gate_of_op[oi];
     for (const FusedGate& fg : f->gates) {
       if (fg.targets.size() > static_cast<size_t>(bt::kMaxW))
         return set_error(QT_ERR_UNSUPPORTED, "%s: fused width %zu > %d in circuit %u", who, fg.targets.size(),
@@ -1088,6 +1321,9 @@ static qt_status pack_batch(qt_batch* B, uint32_t num, const qt_fused* const* fu
     S.pbar = static_cast<uint32_t>(dmat.size());
     for (double p : op.pbar) dmat.push_back(p);
     if (op.pbar.empty()) dmat.push_back(0.0);
+    // u01 = bits * 2^-53 exactly, so bits * 2^-53 < p is bits < ceil(p 2^53)
+    const double p0 = op.pbar.empty() ? 0.0 : op.pbar[0];
+    S.thr0 = p0 > 0.0 ? static_cast<uint64_t>(std::ceil(std::min(p0, 1.0) * 0x1.0p53)) : 0;
   }
   // processing order: largest states first
   B->order.resize(num);
@@ -1095,11 +1331,20 @@ static qt_status pack_batch(qt_batch* B, uint32_t num, const qt_fused* const* fu
   std::stable_sort(B->order.begin(), B->order.end(),
                    [&](uint32_t a, uint32_t b) { return B->traj[a].n > B->traj[b].n; });
   uint64_t soff = 0;
+  std::unordered_map<uint32_t, uint32_t> widest;      // widest fused gate of the circuit whose gates start here
   for (uint32_t i = 0; i < num; ++i) {
     bt::Traj& T = B->traj[i];
+    if (!widest.count(T.gate0)) {
+      uint32_t w = 1;
+      for (uint32_t g = 0; g < T.ngates; ++g) w = std::max<uint32_t>(w, gates[T.gate0 + g].w);
+      widest[T.gate0] = w;
+    }
     T.arena_off = B->total_amps;
     B->total_amps += 1ull << T.n;
-    if (T.n > static_cast<uint32_t>(bt::kSmemNMax)) B->nglob++;
+    const int cls = bt::class_of(T.n);
+    B->count[cls]++;
+    B->top_n[cls] = std::max(B->top_n[cls], T.n);
+    B->wmat[cls] = std::max(B->wmat[cls], widest[T.gate0]);
     T.seed = per ? per[i].seed : 0;
     T.tid = per ? per[i].traj : 0;
     T.S = per ? per[i].S : 0;
@@ -1150,71 +1395,112 @@ static qt_status pack_batch(qt_batch* B, uint32_t num, const qt_fused* const* fu
   return QT_OK;
 }
 
-// counters, pinned run parameters, and the side stream of the second launch
+// counters, pinned run parameters, and the side streams of the classes
 static qt_status init_batch_runtime(qt_batch* B, const char* who) {
   bt::Dev& d = B->dev;
-  // work counters of the two launches (2 x 4 B), error flag (4 B), run parameters at +16 (2 x 8 B)
-  if (!B->counter.alloc(32)) return set_error(QT_ERR_OUT_OF_MEMORY, "%s: counter", who);
+  // work counters of the launches (4 B each, 28 B), error flag (4 B), run parameters at +32 (2 x 8 B)
+  if (!B->counter.alloc(48)) return set_error(QT_ERR_OUT_OF_MEMORY, "%s: counter", who);
   d.counter = static_cast<unsigned int*>(B->counter.p);
-  d.err = reinterpret_cast<int*>(static_cast<unsigned int*>(B->counter.p) + 2);
-  d.run = reinterpret_cast<const uint64_t*>(static_cast<uint8_t*>(B->counter.p) + 16);
+  d.err = reinterpret_cast<int*>(static_cast<unsigned int*>(B->counter.p) + 7);
+  d.run = reinterpret_cast<const uint64_t*>(static_cast<uint8_t*>(B->counter.p) + 32);
   if (cudaMallocHost(&B->hrun, 2 * sizeof(uint64_t)) != cudaSuccess)
     return set_error(QT_ERR_OUT_OF_MEMORY, "%s: pinned parameters", who);
-  if (cudaStreamCreateWithFlags(&B->side, cudaStreamNonBlocking) != cudaSuccess ||
-      cudaEventCreateWithFlags(&B->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&B->ev_join, cudaEventDisableTiming) != cudaSuccess)
-    return set_error(QT_ERR_CUDA, "%s: side stream", who);
+  bool ok = cudaEventCreateWithFlags(&B->ev_fork, cudaEventDisableTiming) == cudaSuccess;
+  for (int c = 0; ok && c < bt::kClasses - 1; ++c)
+    ok = cudaStreamCreateWithFlags(&B->side[c], cudaStreamNonBlocking) == cudaSuccess &&
+         cudaEventCreateWithFlags(&B->ev_join[c], cudaEventDisableTiming) == cudaSuccess;
+  if (!ok) return set_error(QT_ERR_CUDA, "%s: side streams", who);
   return QT_OK;
 }
 
-// dynamic shared memory of the two launches: the matrix area (64 x 64
-// complex64) and, for global states, its 16 x 16 (x, x, y, y) expansion
-// behind it; the shared-memory class adds the 2^14-amplitude state
+// dynamic shared memory of the global class: the matrix area (64 x 64
+// complex64) and its 16 x 16 (x, x, y, y) expansion behind it
 constexpr size_t kSmemMat = sizeof(float2) * (1u << (2 * bt::kMaxW)) + sizeof(float4) * 256;
-constexpr size_t kSmemState = (sizeof(float2) << bt::kSmemNMax) + kSmemMat;
+// of a shared-memory class: the state, two matrices of up to 4 qubits and,
+// where there are wider gates, one of their width
+static size_t smem_class_bytes(uint32_t n, uint32_t wmat) {
+  const uint32_t wbuf = std::min(wmat, 4u);
+  return sizeof(float2) * ((size_t{1} << n) + (size_t{2} << (2 * wbuf)) + (wmat > 4 ? size_t{1} << (2 * wmat) : 0));
+}
+
+// The shared-memory classes ask for the largest carveout, so that their CTAs
+// fit an SM together; the global class keeps its L1.
+template <typename K>
+static cudaError_t smem_kernel_attr(K kern) {
+  const size_t most = smem_class_bytes(bt::kSmemNMax, bt::kMaxW);
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  return e;
+}
 
 static cudaError_t batch_kernel_attrs() {
   static PerDevice attr_set;
   return static_cast<cudaError_t>(attr_set.get([] {
-    cudaError_t e1 = cudaFuncSetAttribute(bt::k_batch<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          static_cast<int>(kSmemState));
-    if (e1 == cudaSuccess)
-      e1 = cudaFuncSetAttribute(bt::k_batch<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                static_cast<int>(kSmemMat));
-    return static_cast<int>(e1);
+    cudaError_t e = cudaFuncSetAttribute(bt::k_batch_glob, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(kSmemMat));
+    if (e == cudaSuccess) e = smem_kernel_attr(bt::k_batch_smem<512, 1>);
+    if (e == cudaSuccess) e = smem_kernel_attr(bt::k_batch_smem<256, 3>);
+    if (e == cudaSuccess) e = smem_kernel_attr(bt::k_batch_smem<128, 7>);
+    return static_cast<int>(e);
   }));
 }
 
-// One run's two persistent launches on stream s, with tables, outputs and
-// arena as d holds them: the work counters are zeroed, the global-memory
-// class launches on s and the shared-memory class on the side stream (forked
-// from and joined back into s), so that its CTAs take SMs as the first
-// launch's CTAs retire.
+template <typename K>
+static cudaError_t launch_smem_class(K kern, uint32_t threads, size_t smem, const bt::Dev& d, uint32_t amps, cudaStream_t s) {
+  int occ = 0;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, static_cast<int>(threads), smem);
+  if (e != cudaSuccess) return e;
+  const unsigned grid = static_cast<unsigned>(std::min<uint64_t>(static_cast<uint64_t>(sm_count()) * std::max(occ, 1), d.num));
+  kern<<<grid, threads, smem, s>>>(d, amps);
+  return cudaGetLastError();
+}
+
+// One run's persistent launches, with tables, outputs and arena as d holds
+// them: the work counters are zeroed on s, then every class launches, the
+// first one present on s and the others on side streams forked from and
+// joined back into s.  `threads` bounds a shared-memory class's CTA and fixes
+// the logical threads its sums are split over.
 static cudaError_t launch_classes(qt_batch* b, const bt::Dev& d, uint32_t threads, uint32_t threads_glob,
                                   cudaStream_t s) {
-  const uint32_t nglob = b->nglob, nsh = b->num - b->nglob;
-  const unsigned grid_g = static_cast<unsigned>(std::min<uint64_t>(sm_count(), nglob));
-  const unsigned grid_s = static_cast<unsigned>(std::min<uint64_t>(sm_count(), nsh));
-  bt::Dev dg = d, ds = d;
-  dg.num = nglob;
-  ds.order = d.order + nglob;
-  ds.num = nsh;
-  ds.counter = d.counter + 1;
-  cudaError_t r = cudaMemsetAsync(b->counter.p, 0, 2 * sizeof(unsigned int) + sizeof(int), s);
-  if (r != cudaSuccess) return r;
-  const bool both = nglob && nsh;
-  if (both) {
-    r = cudaEventRecord(b->ev_fork, s);
-    if (r == cudaSuccess) r = cudaStreamWaitEvent(b->side, b->ev_fork, 0);
-    if (r != cudaSuccess) return r;
+  cudaError_t r = cudaMemsetAsync(b->counter.p, 0, 32, s);
+  int present = 0;
+  for (uint32_t c : b->count) present += c != 0;
+  if (r == cudaSuccess && present > 1) r = cudaEventRecord(b->ev_fork, s);
+  uint32_t off = 0;
+  int used = 0;
+  for (int c = 0; c < bt::kClasses && r == cudaSuccess; ++c) {
+    if (!b->count[c]) continue;
+    cudaStream_t st = s;
+    if (used > 0) {
+      st = b->side[used - 1];
+      r = cudaStreamWaitEvent(st, b->ev_fork, 0);
+      if (r != cudaSuccess) return r;
+    }
+    bt::Dev dc = d;
+    dc.order = d.order + off;
+    dc.num = b->count[c];
+    dc.counter = d.counter + c;
+    dc.wmat = b->wmat[c];
+    if (c == 0) {
+      dc.lthreads = threads_glob;
+      const unsigned grid = static_cast<unsigned>(std::min<uint64_t>(sm_count(), dc.num));
+      bt::k_batch_glob<<<grid, threads_glob, kSmemMat, st>>>(dc);
+      r = cudaGetLastError();
+    } else {
+      dc.lthreads = threads;
+      const uint32_t tb = std::min(threads, c == 1 ? 512u : (c < 4 ? 256u : 128u));
+      const size_t smem = smem_class_bytes(b->top_n[c], dc.wmat);
+      const uint32_t amps = 1u << b->top_n[c];
+      r = tb == 512   ? launch_smem_class(bt::k_batch_smem<512, 1>, tb, smem, dc, amps, st)
+          : tb == 256 ? launch_smem_class(bt::k_batch_smem<256, 3>, tb, smem, dc, amps, st)
+                      : launch_smem_class(bt::k_batch_smem<128, 7>, tb, smem, dc, amps, st);
+    }
+    if (r == cudaSuccess && used > 0) r = cudaEventRecord(b->ev_join[used - 1], st);
+    off += b->count[c];
+    ++used;
   }
-  if (nglob) bt::k_batch<true><<<grid_g, threads_glob, kSmemMat, s>>>(dg);
-  if (nsh) bt::k_batch<false><<<grid_s, threads, kSmemState, both ? b->side : s>>>(ds);
-  r = cudaGetLastError();
-  if (r == cudaSuccess && both) {
-    r = cudaEventRecord(b->ev_join, b->side);
-    if (r == cudaSuccess) r = cudaStreamWaitEvent(s, b->ev_join, 0);
-  }
+  for (int k = 0; k + 1 < used && r == cudaSuccess; ++k) r = cudaStreamWaitEvent(s, b->ev_join[k], 0);
   return r;
 }
 
@@ -1342,7 +1628,7 @@ qt_status qt_batch_run(qt_batch* b, const qt_batch_params* p) {
   if (e != cudaSuccess) return set_error(QT_ERR_CUDA, "qt_batch_run: cudaEventCreate: %s", cudaGetErrorString(e));
   cudaEvent_t e0 = ev.a, e1 = ev.b;
   auto enqueue = [&](cudaStream_t s) -> cudaError_t {
-    cudaError_t r = cudaMemcpyAsync(static_cast<uint8_t*>(b->counter.p) + 16, b->hrun, 2 * sizeof(uint64_t),
+    cudaError_t r = cudaMemcpyAsync(static_cast<uint8_t*>(b->counter.p) + 32, b->hrun, 2 * sizeof(uint64_t),
                                     cudaMemcpyHostToDevice, s);
     if (r != cudaSuccess) return r;
     return launch_classes(b, d, threads, threads_glob, s);

@@ -40,14 +40,18 @@ QT_HD U32x4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
   return o;
 }
 
-// Uniform double in [0, 1) with 53 random bits: the top 27 bits of word 0
-// and the top 26 bits of word 1.
-QT_HD double uniform01(uint64_t seed, uint64_t traj, uint32_t stream, uint32_t index) {
+// Uniform draw of 53 random bits: the top 27 bits of word 0 and the top 26
+// bits of word 1.
+QT_HD uint64_t uniform_bits(uint64_t seed, uint64_t traj, uint32_t stream, uint32_t index) {
   const U32x4 w = philox4x32_10(static_cast<uint32_t>(traj), static_cast<uint32_t>(traj >> 32),
                                 stream, index, static_cast<uint32_t>(seed),
                                 static_cast<uint32_t>(seed >> 32));
-  const uint64_t bits = (static_cast<uint64_t>(w.v[0] >> 5) << 26) | (w.v[1] >> 6);
-  return static_cast<double>(bits) * 0x1.0p-53;
+  return (static_cast<uint64_t>(w.v[0] >> 5) << 26) | (w.v[1] >> 6);
+}
+
+// the same as a double in [0, 1)
+QT_HD double uniform01(uint64_t seed, uint64_t traj, uint32_t stream, uint32_t index) {
+  return static_cast<double>(uniform_bits(seed, traj, stream, index)) * 0x1.0p-53;
 }
 
 enum : uint32_t { kStreamChannel = 0, kStreamSample = 1, kStreamReadout = 2 };
