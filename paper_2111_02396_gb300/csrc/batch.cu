@@ -10,9 +10,8 @@
 //     largest state first;
 //   - a state of up to 2^14 amplitudes lives in its CTA's shared memory, the
 //     CTA sized to it, so that an SM holds several small ones; larger states
-//     live in a per-CTA slot of global memory (up to 2^20 amplitudes, so they
-//     stream from DRAM, and each thread keeps 16 amplitude loads in flight to
-//     cover the latency);
+//     live in a per-CTA slot of global memory (up to 2^20 amplitudes) and come
+//     to shared memory tile by tile, several gates to a sweep;
 //   - stage 1 of Alg. 2 for every channel is decided on the device with the
 //     same Philox4x32-10 draws as the plain loop; stage-2 flush points cut
 //     the circuit into segments exactly as in the plain loop, and within a
@@ -120,6 +119,29 @@ __device__ __forceinline__ uint32_t insert_zeros32(uint32_t x, int w, const int*
   return x;
 }
 
+// Clusters of the global class: the CTAs of one trajectory (all their threads
+// call cluster_sync together; it orders their global-memory accesses)
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t cluster_size() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// the 32-bit word at p of CTA 0's shared memory
+__device__ __forceinline__ uint32_t leader_word(const void* p) {
+  uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(p)), r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"(a));
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(r) : "r"(a) : "memory");
+  return r;
+}
+
 // Where amplitude x of a shared-memory state sits: index bits 4..7 are mapped
 // linearly into bits 0..3.  The 16 lanes of an 8-byte access differ in the
 // four lowest bits that are no target; the map was searched for the fewest
@@ -190,12 +212,13 @@ __device__ __forceinline__ void smem_apply(float2* psi, int n, const uint8_t* t,
 // array (registers or, at w = 6, local memory); kept out of line so that its
 // register demand does not raise that of the rest of the kernel
 template <int W, bool SHARED>
-__device__ __noinline__ void cta_apply_wide(float2* psi, int n, const int* order, const float2* A) {
+__device__ __noinline__ void cta_apply_wide(float2* psi, int n, const int* order, const float2* A, uint32_t first,
+                                            uint32_t stride) {
   constexpr int D = 1 << W;
   int sorted[W];
   for (int b = 0; b < W; ++b) sorted[b] = order[b];
   const uint32_t sets = 1u << (n - W);
-  for (uint32_t s = threadIdx.x; s < sets; s += blockDim.x) {
+  for (uint32_t s = first; s < sets; s += stride) {
     const uint32_t base = insert_zeros32(s, W, sorted);
     float2 v[D];
     for (int m = 0; m < D; ++m) {
@@ -219,97 +242,19 @@ __device__ __noinline__ void cta_apply_wide(float2* psi, int n, const int* order
   }
 }
 
-// psi <- A psi for a state in global memory (n <= 20, so 32-bit indices):
-// each thread gathers NL = 16 amplitudes (B = 16 / 2^W sets, 64 KB per SM of
-// 512 threads) before any arithmetic, so that enough loads are in flight
-// to cover DRAM latency; each matrix entry is one broadcast 128-bit shared load,
-// (a.x, a.x, a.y, a.y), reused by the thread's B sets; a complex
-// multiply-add is two packed FP32x2 FMAs into P = sum a.x (v.x, v.y) and
-// Q = sum a.y (v.x, v.y), and the output is (P.x - Q.y, P.y + Q.x).
-template <int W>
-__device__ __noinline__ void cta_apply_glob(float2* __restrict__ psi, int n, const int* order,
-                                            const float4* __restrict__ A4) {
-  constexpr int D = 1 << W;
-  constexpr int NL = 16;
-  constexpr int B = NL / D;
-  int sorted[W];
-  uint32_t off[D];
-#pragma unroll
-  for (int b = 0; b < W; ++b) sorted[b] = order[b];
-#pragma unroll
-  for (int i = 1; i < W; ++i)
-#pragma unroll
-    for (int j = i; j > 0; --j)
-      if (sorted[j - 1] > sorted[j]) { const int t = sorted[j]; sorted[j] = sorted[j - 1]; sorted[j - 1] = t; }
-#pragma unroll
-  for (int m = 0; m < D; ++m) {
-    uint32_t o = 0;
-#pragma unroll
-    for (int b = 0; b < W; ++b)
-      if ((m >> b) & 1) o |= 1u << order[b];
-    off[m] = o;
-  }
-  const uint32_t sets = 1u << (n - W);
-  const uint32_t stride = blockDim.x;
-  for (uint32_t s0 = threadIdx.x; s0 < sets; s0 += B * stride) {
-    uint32_t base[B];
-    float2 v[B][D];
-#pragma unroll
-    for (int b = 0; b < B; ++b) {
-      const uint32_t sb = s0 + b * stride;
-      base[b] = insert_zeros32(sb < sets ? sb : s0, W, sorted);
-#pragma unroll
-      for (int m = 0; m < D; ++m) v[b][m] = psi[base[b] | off[m]];
-    }
-    // rows one at a time: unrolling them lets the compiler hoist every
-    // matrix load of the pass into registers, which spills
-#pragma unroll 1
-    for (int j = 0; j < D; ++j) {
-      float2 P[B], Q[B];
-#pragma unroll
-      for (int b = 0; b < B; ++b) { P[b] = make_float2(0.f, 0.f); Q[b] = make_float2(0.f, 0.f); }
-#pragma unroll
-      for (int m = 0; m < D; ++m) {
-        const float4 a = A4[j * D + m];
-        const float2 ax = make_float2(a.x, a.y), ay = make_float2(a.z, a.w);
-#pragma unroll
-        for (int b = 0; b < B; ++b) {
-          P[b] = __ffma2_rn(ax, v[b][m], P[b]);
-          Q[b] = __ffma2_rn(ay, v[b][m], Q[b]);
-        }
-      }
-#pragma unroll
-      for (int b = 0; b < B; ++b)
-        if (s0 + b * stride < sets) psi[base[b] | off[j]] = make_float2(P[b].x - Q[b].y, P[b].y + Q[b].x);
-    }
-  }
-}
-
-// Aglob: the matrix in global memory, or smat itself when it was composed there
-__device__ void cta_apply(float2* psi, int n, int w, const int* order, const float2* Aglob, float2* smat) {
-  const int D = 1 << w;
+// a 5- or 6-qubit gate on a state in global memory; A is in global memory, or
+// smat itself when it was composed there
+__device__ void cta_apply_wide_glob(float2* psi, int n, const Gate& G, const float2* A, float2* smat) {
   __syncthreads();                     // previous users of smat / psi are done
-  if (w <= 4) {
-    float4* A4 = reinterpret_cast<float4*>(smat + (1u << (2 * kMaxW)));
-    for (int i = threadIdx.x; i < D * D; i += blockDim.x) {
-      const float2 a = Aglob[i];
-      A4[i] = make_float4(a.x, a.x, a.y, a.y);
-    }
-    __syncthreads();
-    switch (w) {
-      case 1: cta_apply_glob<1>(psi, n, order, A4); break;
-      case 2: cta_apply_glob<2>(psi, n, order, A4); break;
-      case 3: cta_apply_glob<3>(psi, n, order, A4); break;
-      default: cta_apply_glob<4>(psi, n, order, A4); break;
-    }
-    return;
-  }
-  if (Aglob != smat) {
-    for (int i = threadIdx.x; i < D * D; i += blockDim.x) smat[i] = Aglob[i];
+  if (A != smat) {
+    for (int i = threadIdx.x; i < 1 << (2 * G.w); i += blockDim.x) smat[i] = A[i];
     __syncthreads();
   }
-  if (w == 5) cta_apply_wide<5, false>(psi, n, order, smat);
-  else cta_apply_wide<6, false>(psi, n, order, smat);
+  int order[kMaxW];
+  for (int b = 0; b < G.w; ++b) order[b] = G.t[b];
+  const uint32_t first = cluster_rank() * blockDim.x + threadIdx.x, stride = cluster_size() * blockDim.x;
+  if (G.w == 5) cta_apply_wide<5, false>(psi, n, order, smat, first, stride);
+  else cta_apply_wide<6, false>(psi, n, order, smat, first, stride);
 }
 
 __device__ __forceinline__ float2 cmul_add(float2 a, float2 x, float2 acc) {
@@ -370,6 +315,7 @@ __device__ void left_apply(float2* M, int w, int q, const int* pos, const float2
 template <int Q, bool SHARED>
 __device__ void cta_rdm(const float2* psi, int n, const int* order, int lthreads, double* out, float2 (*red)[16]) {
   constexpr int D = 1 << Q, W = D * D;
+  constexpr int U = SHARED ? 1 : 8;                      // sets loaded at once from global memory
   int sorted[Q];
   uint32_t off[D];
   for (int b = 0; b < Q; ++b) sorted[b] = order[b];
@@ -389,22 +335,28 @@ __device__ void cta_rdm(const float2* psi, int n, const int* order, int lthreads
 #pragma unroll
     for (int c = 0; c < W; ++c) { acc[c] = make_float2(0.f, 0.f); f[c] = 0.f; }
     int cnt = 0;
-    for (uint32_t s = l * 32 + lane; s < sets; s += lthreads) {
-      const uint32_t base = insert_zeros32(s, Q, sorted);
-      float2 v[D];
+    for (uint32_t s0 = l * 32 + lane; s0 < sets; s0 += U * lthreads) {
+      float2 v[U][D];
 #pragma unroll
-      for (int m = 0; m < D; ++m) v[m] = psi[at<SHARED>(base | off[m])];
-      int c = 0;
+      for (int u = 0; u < U; ++u) {
+        const uint32_t s = s0 + u * lthreads, base = insert_zeros32(s, Q, sorted);
 #pragma unroll
-      for (int b = 0; b < D; ++b) { f[c] = fmaf(v[b].x, v[b].x, fmaf(v[b].y, v[b].y, f[c])); ++c; }
+        for (int m = 0; m < D; ++m) v[u][m] = s < sets ? psi[at<SHARED>(base | off[m])] : make_float2(0.f, 0.f);
+      }
 #pragma unroll
-      for (int b = 0; b < D; ++b)
+      for (int u = 0; u < U; ++u) {
+        int c = 0;
 #pragma unroll
-        for (int a = b + 1; a < D; ++a) {
-          f[c] = fmaf(v[b].x, v[a].x, fmaf(v[b].y, v[a].y, f[c])); ++c;
-          f[c] = fmaf(v[b].y, v[a].x, fmaf(-v[b].x, v[a].y, f[c])); ++c;
-        }
-      if (++cnt == 16) {
+        for (int b = 0; b < D; ++b) { f[c] = fmaf(v[u][b].x, v[u][b].x, fmaf(v[u][b].y, v[u][b].y, f[c])); ++c; }
+#pragma unroll
+        for (int b = 0; b < D; ++b)
+#pragma unroll
+          for (int a = b + 1; a < D; ++a) {
+            f[c] = fmaf(v[u][b].x, v[u][a].x, fmaf(v[u][b].y, v[u][a].y, f[c])); ++c;
+            f[c] = fmaf(v[u][b].y, v[u][a].x, fmaf(-v[u][b].x, v[u][a].y, f[c])); ++c;
+          }
+      }
+      if ((cnt += U) == 16) {
 #pragma unroll
         for (int k = 0; k < W; ++k) { df_acc(acc[k].x, acc[k].y, f[k]); f[k] = 0.f; }
         cnt = 0;
@@ -457,27 +409,40 @@ __device__ void cta_sample(const float2* psi, int n, uint64_t seed, uint64_t tra
   uint32_t per = (amps + lw - 1) / lw;
   per = (per + 31) & ~31u;
   const int chunks = static_cast<int>(per / 32);
-  const int gpr = min(chunks, kSampleGroups / lw), gch = chunks / gpr;   // groups per range, chunks per group
+  const int gpr = min(chunks, kSampleGroups / lw), gch = chunks / gpr;   // groups per range, chunks per group (2^k)
+  const int glog = 31 - __clz(gch);
+  // chunks loaded at once from global memory (2^15 amplitudes and more: every
+  // chunk is inside the state)
+  constexpr int U = SHARED ? 1 : 16;
   auto weight = [&](uint32_t x) {
     float w = 0.f;
-    if (x < amps) { const float2 a = psi[at<SHARED>(x)]; w = fmaf(a.x, a.x, a.y * a.y); }
+    if (!SHARED || x < amps) { const float2 a = psi[at<SHARED>(x)]; w = fmaf(a.x, a.x, a.y * a.y); }
     return w;
   };
   __syncthreads();
   for (int r = warp; r < lw; r += nw) {
     const uint32_t lo = r * per;
-    float run = 0.f;
-    for (int g = 0; g < gpr; ++g) {
-      const float before = run;
-      float most = 0.f;
-#pragma unroll 4
-      for (int c = 0; c < gch; ++c) {
-        const float inc = warp_scan_f(weight(lo + (g * gch + c) * 32 + lane), lane);
-        most = fmaxf(most, run + inc);
-        run += __shfl_sync(0xffffffffu, inc, 31);
+    float run = 0.f, most = 0.f;
+    for (int c0 = 0; c0 < chunks; c0 += U) {               // chunks is a multiple of U
+      float w[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) w[u] = weight(lo + (c0 + u) * 32 + lane);
+#pragma unroll
+      for (int u = 0; u < U; ++u) w[u] = warp_scan_f(w[u], lane);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int g = (c0 + u) >> glog;
+        if (((c0 + u) & (gch - 1)) == 0) {
+          if (lane == 0) sc.before[r * gpr + g] = run;
+          most = 0.f;
+        }
+        most = fmaxf(most, run + w[u]);
+        run += __shfl_sync(0xffffffffu, w[u], 31);
+        if (((c0 + u + 1) & (gch - 1)) == 0) {
+          const float all = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(most)));   // not negative
+          if (lane == 0) sc.most[r * gpr + g] = all;
+        }
       }
-      most = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(most)));   // not negative
-      if (lane == 0) { sc.before[r * gpr + g] = before; sc.most[r * gpr + g] = most; }
     }
     if (lane == 0) sc.wcum[r] = static_cast<double>(run);
   }
@@ -661,6 +626,7 @@ __device__ __forceinline__ float2 fold_factor(const FoldPiece& F, const float2* 
 
 __device__ __noinline__ int cta_product_start(const Dev& d, const Traj& T, float2* psi, uint32_t hi,
                                               float2* s_mat, float2* s_col, FoldPiece* s_fold, MemberList& list) {
+  const uint32_t rank = cluster_rank(), nranks = cluster_size();
   __shared__ int s_split, s_nstr;
   __shared__ uint8_t s_str[kMaxN];
   const int tid = threadIdx.x;
@@ -696,7 +662,7 @@ __device__ __noinline__ int cta_product_start(const Dev& d, const Traj& T, float
     off += D;
     ++nf;
   }
-  __syncthreads();                 // every thread has read the gate flags; s_fold is complete
+  cluster_sync();                  // every thread has read the gate flags; s_fold is complete
   if (tid < 32) {
     // lane c scores the split at m = c: fewest straddling pieces, then the
     // most even tables, among the splits whose tables fit s_mat
@@ -718,7 +684,8 @@ __device__ __noinline__ int cta_product_start(const Dev& d, const Traj& T, float
       s_nstr = ns;
     }
     // mark the folded gates for the pass loop
-    for (int f = tid; f < nf; f += 32) d.gflag[T.gf0 + s_fold[f].gate] = 2;
+    if (rank == 0)
+      for (int f = tid; f < nf; f += 32) d.gflag[T.gf0 + s_fold[f].gate] = 2;
   }
   __syncthreads();
   const int m = s_split, ns = s_nstr;
@@ -740,14 +707,12 @@ __device__ __noinline__ int cta_product_start(const Dev& d, const Traj& T, float
     else t_lo[y] = v;
   }
   __syncthreads();
-  const uint64_t amps = 1ull << n;
-  for (uint64_t x = tid; x < amps; x += blockDim.x) {
-    const uint32_t xi = static_cast<uint32_t>(x);
-    float2 v = cmul(t_lo[xi & lmask], t_hi[xi >> m]);
-    for (int j = 0; j < ns; ++j) v = cmul(v, fold_factor(s_fold[s_str[j]], s_col, xi));
+  for (uint32_t x = rank * blockDim.x + tid; x < 1u << n; x += nranks * blockDim.x) {
+    float2 v = cmul(t_lo[x & lmask], t_hi[x >> m]);
+    for (int j = 0; j < ns; ++j) v = cmul(v, fold_factor(s_fold[s_str[j]], s_col, x));
     psi[x] = v;
   }
-  __syncthreads();                 // the marks and the state are visible to the CTA
+  cluster_sync();                  // the marks and the state are visible to the cluster
   return nf;
 }
 
@@ -775,9 +740,13 @@ struct TrajShared {
 // that hold a channel with another operator than its default (or an undecided
 // one) get their flag, so that the pass loop reads one flag per gate.  Nearly
 // every draw takes the first operator, which an integer compare settles.
-__device__ __forceinline__ void cta_stage1(const Dev& d, const Traj& T, uint64_t seed, uint64_t traj_id, TrajShared& sh) {
+// Every CTA of a cluster makes its own list of flush points; the first one
+// writes the records and flags.
+__device__ __forceinline__ void cta_stage1(const Dev& d, const Traj& T, uint64_t seed, uint64_t traj_id, bool lead,
+                                           TrajShared& sh) {
   const int tid = threadIdx.x;
-  for (uint32_t g = tid; g < T.ngates; g += blockDim.x) d.gflag[T.gf0 + g] = 0;
+  if (lead)
+    for (uint32_t g = tid; g < T.ngates; g += blockDim.x) d.gflag[T.gf0 + g] = 0;
   if (tid == 0) { sh.pend_pos = -1; sh.pend_choice = 0; sh.scale = 1.f; sh.nflush = 0; }
   __syncthreads();
 #pragma unroll 2
@@ -796,9 +765,11 @@ __device__ __forceinline__ void cta_stage1(const Dev& d, const Traj& T, uint64_t
         rr -= pbar[i];
       }
     }
-    d.kraus[T.ch0 + c] = ch;
-    d.stage[T.ch0 + c] = ch >= 0 ? 1 : 0;
-    if (ch != static_cast<int>(st.def)) d.gflag[T.gf0 + op.gate] = 1;
+    if (lead) {
+      d.kraus[T.ch0 + c] = ch;
+      d.stage[T.ch0 + c] = ch >= 0 ? 1 : 0;
+      if (ch != static_cast<int>(st.def)) d.gflag[T.gf0 + op.gate] = 1;
+    }
     if (ch < 0) {
       const int k = atomicAdd(&sh.nflush, 1);
       if (k < kFlushMax) sh.flush[k] = c;
@@ -938,7 +909,7 @@ __global__ void __launch_bounds__(TB, MINB) k_batch_smem(const __grid_constant__
     const uint32_t S = d.per_traj ? T.S : d.S;
     uint64_t* samples = d.samples + (d.per_traj ? T.soff : static_cast<uint64_t>(ti) * d.S);
     for (uint32_t x = tid; x < amps; x += blockDim.x) psi[x] = make_float2(x == 0 ? 1.f : 0.f, 0.f);   // sw(0) = 0
-    cta_stage1(d, T, seed, traj_id, sh);
+    cta_stage1(d, T, seed, traj_id, true, sh);
     uint32_t lo = 0, cur_ch = 0, nflush = 0;
     for (;;) {
       const int fch = cta_next_flush(d, T, cur_ch, sh);
@@ -1002,8 +973,8 @@ __global__ void __launch_bounds__(TB, MINB) k_batch_smem(const __grid_constant__
             default: {
               int order[kMaxW];
               for (int k = 0; k < w; ++k) order[k] = t[k];
-              if (w == 5) cta_apply_wide<5, true>(psi, n, order, A);
-              else cta_apply_wide<6, true>(psi, n, order, A);
+              if (w == 5) cta_apply_wide<5, true>(psi, n, order, A, tid, blockDim.x);
+              else cta_apply_wide<6, true>(psi, n, order, A, tid, blockDim.x);
             }
           }
           g = nx;
@@ -1027,24 +998,180 @@ __global__ void __launch_bounds__(TB, MINB) k_batch_smem(const __grid_constant__
   }
 }
 
-// Larger states, each in its CTA's slot of global memory
-__global__ void __launch_bounds__(512) k_batch_glob(const __grid_constant__ Dev d) {
+// Larger states (2^15..2^20 amplitudes), each in its cluster's slot of global
+// memory (a cluster is one CTA in a batch with trajectories enough, see
+// glob_cluster).  One pass per gate was bound by the latency and traffic of
+// the slot (156 us a pass at 18 qubits, 13 bytes a clock and SM), so
+// consecutive gates share a sweep: in circuit order, gates are taken as long
+// as their qubits and the lowest kTileLow ones number at most kTileBits.  A
+// sweep brings the state tile by tile (2^13 amplitudes over the group's
+// qubits, rows of at least 128 bytes, cp.async) to shared memory, applies
+// every gate of the group and writes the tile back.  At 18 qubits and k = 3
+// that is about 43 sweeps for 164 gates; what bounds it now is the tile's
+// arithmetic and the shared-memory reads that feed it (4700 clocks a gate and
+// tile, of which the FMAs take 2050).  Gates keep their order and an amplitude
+// its operations: states and samples are those of one pass per gate, bit for
+// bit.  660 trajectories of 8 to 18 qubits: 21.2 -> 11.3 ms (18.8 with one
+// CTA per trajectory and both halves of it on one tile).
+constexpr int kTileBits = 13, kTileLow = 4;
+constexpr int kTileSets = 32;                              // members a thread holds
+constexpr int kGroupGates = 16, kGroupEntries = 1024;      // matrices of a sweep: at most 1024 entry pairs
+constexpr int kTileChunks = 1 << (kTileBits - 1);          // 16-byte chunks of a tile
+
+// place of amplitude x of a staged tile: as sw, but whole 16-byte chunks move
+__device__ __forceinline__ uint32_t sw16(uint32_t x) { return x ^ ((sw(x) ^ x) & 14u); }
+
+// the set bits of `mask`, ascending, receive the low bits of x
+__device__ __forceinline__ uint32_t deposit(uint32_t x, uint32_t mask) {
+  uint32_t r = 0;
+  for (uint32_t m = mask; m; m &= m - 1, x >>= 1)
+    if (x & 1u) r |= m & (0u - m);
+  return r;
+}
+
+struct Sweep {
+  uint8_t gate[kGroupGates], w[kGroupGates], pos[kGroupGates][4];   // window index, width, tile positions
+  uint16_t mat[kGroupGates];                                        // first entry of its matrix
+  uint16_t member[kGroupGates][16], step[kGroupGates][8];           // places of member m and of a thread's set b
+  int ng;
+  uint32_t tile, rest;                                              // qubit masks
+  uint32_t off[64], place[64];                                      // per chunk step: memory and tile offset
+};
+
+// sets of a w-qubit gate that a thread takes at once
+__host__ __device__ constexpr int tile_sets(int w) { return kTileSets >> w > 8 ? 8 : kTileSets >> w; }
+
+// psi <- A psi on a staged tile.  A shared-memory read returns 128 bytes a
+// clock however many lanes ask for the same word, so a matrix entry read for
+// one set costs as much as its FMAs: a thread takes B sets (32 / 2^W of them,
+// 128 registers of members) and two rows at a time.  M4 entry (row pair, m) is
+// (Re, Re, Im, Im) of the two rows, the members are held doubled, and packed
+// FMAs sum P = sum Re v and Q = sum Im v for both rows; the outputs are
+// (P.x - Q.y, P.y + Q.x).
+template <int W>
+__device__ __forceinline__ void tile_apply(float2* tile, const Sweep& g, int k, const float4* M4, int tid, int nt) {
+  constexpr int D = 1 << W, B = tile_sets(W);
+  int p[W];
+  uint32_t off[D], step[B];
+#pragma unroll
+  for (int b = 0; b < W; ++b) p[b] = g.pos[k][b];
+#pragma unroll
+  for (int m = 0; m < D; ++m) off[m] = g.member[k][m];
+#pragma unroll
+  for (int b = 0; b < B; ++b) step[b] = g.step[k][b];
+  constexpr uint32_t sets = 1u << (kTileBits - W);
+  for (uint32_t s0 = tid; s0 < sets; s0 += B * nt) {       // sets is a multiple of B nt
+    const uint32_t first = sw16(insert_zeros32(s0, W, p));
+    uint32_t base[B];
+    float2 vx[B][D], vy[B][D];
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+      base[b] = first ^ step[b];
+#pragma unroll
+      for (int m = 0; m < D; ++m) {
+        const float2 v = tile[base[b] ^ off[m]];
+        vx[b][m] = make_float2(v.x, v.x);
+        vy[b][m] = make_float2(v.y, v.y);
+      }
+    }
+#pragma unroll 1
+    for (int j = 0; j < D; j += 2) {
+      float2 px[B], py[B], qx[B], qy[B];
+#pragma unroll
+      for (int b = 0; b < B; ++b) px[b] = py[b] = qx[b] = qy[b] = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int m = 0; m < D; ++m) {
+        const float4 a = M4[(j >> 1) * D + m];
+        const float2 re = make_float2(a.x, a.y), im = make_float2(a.z, a.w);
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+          px[b] = __ffma2_rn(re, vx[b][m], px[b]);
+          py[b] = __ffma2_rn(re, vy[b][m], py[b]);
+          qx[b] = __ffma2_rn(im, vx[b][m], qx[b]);
+          qy[b] = __ffma2_rn(im, vy[b][m], qy[b]);
+        }
+      }
+      const uint32_t o0 = g.member[k][j], o1 = g.member[k][j + 1];
+#pragma unroll
+      for (int b = 0; b < B; ++b) {
+        tile[base[b] ^ o0] = make_float2(px[b].x - qy[b].x, py[b].x + qx[b].x);
+        tile[base[b] ^ o1] = make_float2(px[b].y - qy[b].y, py[b].y + qx[b].y);
+      }
+    }
+  }
+}
+
+__device__ __forceinline__ void cp_async16_l2(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst))), "l"(src)
+               : "memory");
+}
+
+// One sweep over the state: the group's matrices are in place.  Each half of
+// the CTA stages and works on tiles of its own (named barriers), so that one
+// half's copies, gathers and barriers pass under the other's arithmetic; the
+// tiles are dealt to the halves of all the cluster's CTAs.
+__device__ __noinline__ void cta_sweep(float2* __restrict__ psi, int n, float2* tiles, const float4* mats, const Sweep& g) {
+  const int half = threadIdx.x >= blockDim.x / 2, gs = blockDim.x / 2, tid = threadIdx.x - half * gs;
+  const int steps = kTileChunks / gs;
+  const uint32_t my_off = deposit(2u * tid, g.tile), my_place = sw16(2u * tid), rest = g.rest;
+  const int ntiles = 1 << (n - kTileBits);
+  float2* const tile = tiles + (half << kTileBits);
+  auto sync = [&] { asm volatile("bar.sync %0, %1;" ::"r"(1 + half), "r"(gs) : "memory"); };
+  for (int t = cluster_rank() * 2 + half; t < ntiles; t += cluster_size() * 2) {
+    float2* const mem = psi + (deposit(t, rest) | my_off);
+#pragma unroll 4
+    for (int i = 0; i < steps; ++i) cp_async16_l2(tile + (my_place ^ g.place[i]), mem + g.off[i]);
+    cp_async_wait();
+    sync();
+    for (int i = 0; i < g.ng; ++i) {
+      const float4* const M4 = mats + g.mat[i];
+      switch (g.w[i]) {
+        case 1: tile_apply<1>(tile, g, i, M4, tid, gs); break;
+        case 2: tile_apply<2>(tile, g, i, M4, tid, gs); break;
+        case 3: tile_apply<3>(tile, g, i, M4, tid, gs); break;
+        default: tile_apply<4>(tile, g, i, M4, tid, gs); break;
+      }
+      sync();
+    }
+#pragma unroll 4
+    for (int i = 0; i < steps; ++i)
+      *reinterpret_cast<float4*>(mem + g.off[i]) = *reinterpret_cast<const float4*>(tile + (my_place ^ g.place[i]));
+    // this thread's own chunks are in its registers: the next copies may overwrite
+    // them, and no one else reads this tile before the next barrier
+  }
+}
+
+constexpr int kGlobThreads = 256;
+
+__global__ void __launch_bounds__(kGlobThreads) k_batch_glob(const __grid_constant__ Dev d) {
   extern __shared__ __align__(16) float2 s_dyn[];
-  float2* s_mat = s_dyn;                            // the pass's matrix, up to 64 x 64
+  float2* const tiles = s_dyn;                      // two staged tiles; between sweeps, one matrix of up to
+  float2* const s_mat = s_dyn;                      // 64 x 64 or the product-state tables
+  float4* const mats = reinterpret_cast<float4*>(s_dyn + (2u << kTileBits));   // the sweep's matrices
   __shared__ TrajShared sh;
+  __shared__ Gate s_gate[kWindow];
+  __shared__ uint8_t s_kind[kWindow];
+  __shared__ Sweep s_sweep;
   __shared__ float2 s_col[kFoldCols];               // columns U[:, 0] of the folded pieces
   __shared__ FoldPiece s_fold[kMaxN];
-  const int tid = threadIdx.x;
-  uint32_t ti;
-  while (next_trajectory(d, sh, ti)) {
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const bool lead = cluster_rank() == 0;
+  for (;;) {
+    cluster_sync();                                 // the previous trajectory is done with
+    if (lead && tid == 0) sh.idx = atomicAdd(d.counter, 1u);
+    cluster_sync();
+    const uint32_t idx = leader_word(&sh.idx);
+    if (idx >= d.num) break;
+    const uint32_t ti = d.order[idx];
     const Traj T = d.traj[ti];
     const int n = static_cast<int>(T.n);
     const uint64_t seed = d.per_traj ? T.seed : d.run[0];
     const uint64_t traj_id = d.per_traj ? T.tid : d.run[1] + ti;
     const uint32_t S = d.per_traj ? T.S : d.S;
     uint64_t* samples = d.samples + (d.per_traj ? T.soff : static_cast<uint64_t>(ti) * d.S);
-    float2* psi = d.keep ? d.arena + T.arena_off : d.arena + static_cast<uint64_t>(blockIdx.x) * d.slot_amps;
-    cta_stage1(d, T, seed, traj_id, sh);
+    float2* psi = d.keep ? d.arena + T.arena_off : d.arena + blockIdx.x / cluster_size() * d.slot_amps;
+    cta_stage1(d, T, seed, traj_id, lead, sh);
+    cluster_sync();                                 // the records and flags are there
     uint32_t lo = 0, cur_ch = 0, nflush = 0;
     for (;;) {
       const int fch = cta_next_flush(d, T, cur_ch, sh);
@@ -1055,34 +1182,127 @@ __global__ void __launch_bounds__(512) k_batch_glob(const __grid_constant__ Dev 
       const bool first = lo == 0 && nflush == 0;
       if (first) {
         const int nf = cta_product_start(d, T, psi, hi, s_mat, s_col, s_fold, sh.list);
-        if (tid == 0 && d.folds) d.folds[ti] = static_cast<uint32_t>(nf);
+        if (lead && tid == 0 && d.folds) d.folds[ti] = static_cast<uint32_t>(nf);
       }
       // apply ops [lo, hi): fused gates restricted to the segment (in the
       // first segment, those not folded into the initial state)
-      for (uint32_t g = 0; g < T.ngates; ++g) {
-        const Gate G = d.gates[T.gate0 + g];
-        if (G.maxpos < lo || G.minpos >= hi) continue;
-        const uint8_t flag = d.gflag[T.gf0 + g];
-        if (first && flag == 2) continue;
-        int order[kMaxW];
-        for (int b = 0; b < G.w; ++b) order[b] = G.t[b];
-        if (G.minpos >= lo && G.maxpos < hi && !flag && g != pend_gate) {
-          cta_apply(psi, n, G.w, order, d.fmat + G.mat, s_mat);
-          continue;
+      for (uint32_t g0 = 0; g0 < T.ngates; g0 += kWindow) {
+        const int cnt = static_cast<int>(min(T.ngates - g0, static_cast<uint32_t>(kWindow)));
+        __syncthreads();                                 // the previous window is done with
+        for (int i = tid; i < cnt; i += nt) {
+          const Gate G = d.gates[T.gate0 + g0 + i];
+          const uint8_t flag = d.gflag[T.gf0 + g0 + i];
+          uint8_t kind = kSkip;
+          if (G.maxpos >= lo && G.minpos < hi && !(first && flag == 2))
+            kind = G.minpos >= lo && G.maxpos < hi && !flag && g0 + i != pend_gate ? kDefault : kCompose;
+          s_gate[i] = G;
+          s_kind[i] = kind;
         }
-        cta_compose_piece(d, T, G, lo, hi, pend_pos, pend_choice, pend_scale, s_mat, sh.list);
-        cta_apply(psi, n, G.w, order, s_mat, s_mat);
+        __syncthreads();
+        for (int g = 0; g < cnt;) {
+          if (s_kind[g] == kSkip) { ++g; continue; }
+          if (s_gate[g].w > 4) {                         // a pass of its own
+            const Gate G = s_gate[g];
+            const float2* A = d.fmat + G.mat;
+            if (s_kind[g] == kCompose) {
+              cta_compose_piece(d, T, G, lo, hi, pend_pos, pend_choice, pend_scale, s_mat, sh.list);
+              A = s_mat;
+            }
+            cta_apply_wide_glob(psi, n, G, A, s_mat);
+            cluster_sync();
+            ++g;
+            continue;
+          }
+          // the group: every thread walks the same descriptors
+          uint32_t mask = (1u << kTileLow) - 1u;
+          int ng = 0, entries = 0, end = g;
+          for (; end < cnt; ++end) {
+            if (s_kind[end] == kSkip) continue;
+            const int w = s_gate[end].w;
+            if (w > 4 || ng == kGroupGates || entries + (1 << (2 * w - 1)) > kGroupEntries) break;
+            const uint32_t m = mask | gate_mask(s_gate[end]);
+            if (__popc(m) > kTileBits) break;
+            mask = m;
+            entries += 1 << (2 * w - 1);
+            ++ng;
+          }
+          for (uint32_t q = 0; __popc(mask) < kTileBits; ++q) mask |= 1u << q;   // n >= 15: enough qubits
+          __syncthreads();
+          if (tid == 0) {
+            int k = 0, e = 0;
+            for (int i = g; i < end; ++i) {
+              if (s_kind[i] == kSkip) continue;
+              const int w = s_gate[i].w;
+              s_sweep.gate[k] = static_cast<uint8_t>(i);
+              s_sweep.w[k] = static_cast<uint8_t>(w);
+              for (int b = 0; b < w; ++b)
+                s_sweep.pos[k][b] = static_cast<uint8_t>(__popc(mask & ((1u << s_gate[i].t[b]) - 1u)));
+              s_sweep.mat[k] = static_cast<uint16_t>(e);
+              e += 1 << (2 * w - 1);
+              ++k;
+            }
+            s_sweep.ng = ng;
+            s_sweep.tile = mask;
+            s_sweep.rest = ((1u << n) - 1u) & ~mask;
+          }
+          if (tid >= 64 && tid < 128) {
+            const uint32_t l = static_cast<uint32_t>(nt) * (tid - 64);   // 2 x (nt / 2) threads of a half
+            s_sweep.off[tid - 64] = deposit(l, mask);
+            s_sweep.place[tid - 64] = sw16(l);
+          }
+          __syncthreads();
+          for (int x = tid; x < ng * 24; x += nt) {      // 16 members, 8 sets a gate
+            const int k = x / 24, e = x % 24, w = s_sweep.w[k];
+            int p[4];
+            for (int b = 0; b < w; ++b) p[b] = s_sweep.pos[k][b];
+            if (e < 16) {
+              uint32_t o = 0;
+              for (int b = 0; b < w; ++b)
+                if ((e >> b) & 1) o |= 1u << p[b];
+              s_sweep.member[k][e] = static_cast<uint16_t>(sw16(o));
+            } else {
+              s_sweep.step[k][e - 16] =
+                  static_cast<uint16_t>(sw16(insert_zeros32(static_cast<uint32_t>((e - 16) * (nt / 2)), w, p)));
+            }
+          }
+          for (int k = 0; k < ng; ++k) {
+            const int i = s_sweep.gate[k], w = s_sweep.w[k];
+            float4* const M4 = mats + s_sweep.mat[k];
+            const float2* A = d.fmat + s_gate[i].mat;
+            if (s_kind[i] == kCompose) {
+              const Gate G = s_gate[i];
+              cta_compose_piece(d, T, G, lo, hi, pend_pos, pend_choice, pend_scale, s_mat, sh.list);
+              __syncthreads();
+              A = s_mat;
+            }
+            for (int x = tid; x < 1 << (2 * w - 1); x += nt) {
+              const int r = (x >> w) << (w + 1) | (x & ((1 << w) - 1));   // row 2 (x >> w), column x mod 2^w
+              const float2 a0 = A[r], a1 = A[r + (1 << w)];
+              M4[x] = make_float4(a0.x, a1.x, a0.y, a1.y);
+            }
+          }
+          __syncthreads();                               // matrices complete, s_mat free for the tiles
+          cta_sweep(psi, n, tiles, mats, s_sweep);
+          cluster_sync();                                // the sweep is complete, and done with its shared memory
+          g = end;
+        }
       }
       if (fch < 0) break;
-      cta_stage2<false>(d, T, psi, hi, fch, seed, traj_id, sh);
+      if (lead) cta_stage2<false>(d, T, psi, hi, fch, seed, traj_id, sh);
+      cluster_sync();
+      if (!lead && tid == 0) {
+        sh.pend_pos = static_cast<int>(leader_word(&sh.pend_pos));
+        sh.pend_choice = static_cast<int>(leader_word(&sh.pend_choice));
+        sh.scale = __uint_as_float(leader_word(&sh.scale));
+      }
       ++nflush;
       lo = hi;
       cur_ch = static_cast<uint32_t>(fch) + 1;
     }
-    __syncthreads();
-    if (S) cta_sample<false>(psi, n, seed, traj_id, S, samples, static_cast<int>(d.lthreads), sh.sample);
-    if (tid == 0) d.flushes[ti] = nflush;
+    if (lead && S) cta_sample<false>(psi, n, seed, traj_id, S, samples, static_cast<int>(d.lthreads), sh.sample);
+    if (lead && tid == 0) d.flushes[ti] = nflush;
   }
+  cluster_sync();                                   // no CTA leaves while its shared memory may be read
 }
 
 }  // namespace bt
@@ -1413,9 +1633,9 @@ static qt_status init_batch_runtime(qt_batch* B, const char* who) {
   return QT_OK;
 }
 
-// dynamic shared memory of the global class: the matrix area (64 x 64
-// complex64) and its 16 x 16 (x, x, y, y) expansion behind it
-constexpr size_t kSmemMat = sizeof(float2) * (1u << (2 * bt::kMaxW)) + sizeof(float4) * 256;
+// dynamic shared memory of the global class: two tiles (one of them holds the
+// 64 x 64 matrix area between sweeps) and the matrices of a sweep
+constexpr size_t kSmemGlob = sizeof(float2) * (2u << bt::kTileBits) + sizeof(float4) * bt::kGroupEntries;
 // of a shared-memory class: the state, two matrices of up to 4 qubits and,
 // where there are wider gates, one of their width
 static size_t smem_class_bytes(uint32_t n, uint32_t wmat) {
@@ -1438,7 +1658,7 @@ static cudaError_t batch_kernel_attrs() {
   static PerDevice attr_set;
   return static_cast<cudaError_t>(attr_set.get([] {
     cudaError_t e = cudaFuncSetAttribute(bt::k_batch_glob, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(kSmemMat));
+                                         static_cast<int>(kSmemGlob));
     if (e == cudaSuccess) e = smem_kernel_attr(bt::k_batch_smem<512, 1>);
     if (e == cudaSuccess) e = smem_kernel_attr(bt::k_batch_smem<256, 3>);
     if (e == cudaSuccess) e = smem_kernel_attr(bt::k_batch_smem<128, 7>);
@@ -1454,6 +1674,36 @@ static cudaError_t launch_smem_class(K kern, uint32_t threads, size_t smem, cons
   const unsigned grid = static_cast<unsigned>(std::min<uint64_t>(static_cast<uint64_t>(sm_count()) * std::max(occ, 1), d.num));
   kern<<<grid, threads, smem, s>>>(d, amps);
   return cudaGetLastError();
+}
+
+// CTAs per trajectory of the global class: one where the batch has
+// trajectories enough to even out over the SMs, two below two per SM (240 of
+// 15 to 18 qubits: 17.6 ms with one, 12.1 with two, 14.4 with four, whose
+// smaller states have fewer tiles than the cluster has halves and whose
+// clusters leave SMs over), more where SMs would stay idle.
+static unsigned glob_cluster(uint32_t num, uint32_t top_n) {
+  const uint32_t sms = static_cast<uint32_t>(sm_count());
+  const unsigned most = std::min(8u, 1u << (top_n - bt::kTileBits - 1));   // at least a tile per half
+  unsigned c = num < 2 * sms ? 2 : 1;
+  while (c < most && num * c < sms) c *= 2;
+  return c;
+}
+
+static cudaError_t launch_glob_class(uint32_t threads, const bt::Dev& d, uint32_t top_n, cudaStream_t s) {
+  const unsigned c = glob_cluster(d.num, top_n);
+  const unsigned clusters = static_cast<unsigned>(std::min<uint64_t>(static_cast<uint64_t>(sm_count()) / c, d.num));
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = c;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(std::max(clusters, 1u) * c);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = kSmemGlob;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, bt::k_batch_glob, d);
 }
 
 // One run's persistent launches, with tables, outputs and arena as d holds
@@ -1484,9 +1734,7 @@ static cudaError_t launch_classes(qt_batch* b, const bt::Dev& d, uint32_t thread
     dc.wmat = b->wmat[c];
     if (c == 0) {
       dc.lthreads = threads_glob;
-      const unsigned grid = static_cast<unsigned>(std::min<uint64_t>(sm_count(), dc.num));
-      bt::k_batch_glob<<<grid, threads_glob, kSmemMat, st>>>(dc);
-      r = cudaGetLastError();
+      r = launch_glob_class(std::min<uint32_t>(threads_glob, bt::kGlobThreads), dc, b->top_n[c], st);
     } else {
       dc.lthreads = threads;
       const uint32_t tb = std::min(threads, c == 1 ? 512u : (c < 4 ? 256u : 128u));
