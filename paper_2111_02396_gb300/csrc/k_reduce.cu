@@ -795,7 +795,7 @@ cudaError_t launch_kraus_probs(const float2* psi, int n, int q, const uint32_t* 
   }
 }
 
-// Channels on 6 qubits and smaller states: for G operators at a time, P_i = sum over gather sets of
+// Channels on 4 and 5 qubits of smaller states: for G operators at a time, P_i = sum over gather sets of
 // |K_i v|^2, plus N = <psi|psi>.  Each thread takes whole gather sets, staged
 // column-wise in shared memory (member m of thread t at v[m * blockDim + t],
 // conflict-free), with the G operators in shared memory.  Products and row
@@ -914,7 +914,11 @@ cudaError_t launch_kraus_norms(const float2* psi, int n, int q, const uint32_t* 
   switch (q) {
     case 4: return kraus_norms_q<4, 16>(psi, n, qubits, ops_dev, scr, st);
     case 5: return kraus_norms_q<5, 4>(psi, n, qubits, ops_dev, scr, st);
-    case 6: return kraus_norms_q<6, 1>(psi, n, qubits, ops_dev, scr, st);
+    case 6: {                             // k_mat64.cu
+      int g = 0;
+      const cudaError_t e = launch_norms64(psi, n, qubits, ops_dev, scr.partials(), &g, st);
+      return e != cudaSuccess ? e : finalize(scr.partials(), g, 2, scr.result, st);
+    }
     default: return cudaErrorInvalidValue;
   }
 }

@@ -103,6 +103,10 @@ cudaError_t launch_sample(const float2* psi, int n, uint64_t seed, uint64_t traj
 cudaError_t launch_cdf_values(const float2* psi, int n, const Scratch& scr, double* out, cudaStream_t st);
 // 6-qubit fused gate on CUDA cores (FP32), matrix 64x64 row-major in device memory, n >= 13
 cudaError_t launch_apply6_fp32(float2* psi, int n, const uint32_t* targets, const float2* udev, cudaStream_t st);
+// per-block sums of |psi|^2 and |K psi|^2 (two double-floats a block) for one
+// 64 x 64 operator (basis bit b <-> qubits[b]), n >= 6
+cudaError_t launch_norms64(const float2* psi, int n, const uint32_t* qubits, const float2* kdev, float2* partial,
+                           int* blocks, cudaStream_t st);
 // multi-gate pass: up to kGroupMaxGates fused gates (width <= 4, targets
 // ascending, matrix row-major) whose qubits lie in {0..6} plus at most 6
 // higher qubits, applied in one pass over the state (n >= 7 + #high qubits)

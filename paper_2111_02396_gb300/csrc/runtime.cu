@@ -164,11 +164,11 @@ struct WideChannel {
     rows.resize(G + 1);
     for (uint32_t g0 = 0; g0 < num_ops; g0 += G) {
       ops.assign(G * mat, make_float2(0.f, 0.f));
-      for (uint32_t j = 0; j < G && g0 + j < num_ops; ++j)
-        for (size_t e = 0; e < mat; ++e) {
-          const double* k = K + 2 * (mat * (g0 + j) + e);
-          ops[j * mat + e] = make_float2(static_cast<float>(k[0]), static_cast<float>(k[1]));
-        }
+      for (uint32_t j = 0; j < G && g0 + j < num_ops; ++j) {
+        const double* k = K + 2 * mat * (g0 + j);
+        for (size_t e = 0; e < mat; ++e)
+          ops[j * mat + e] = make_float2(static_cast<float>(k[2 * e]), static_cast<float>(k[2 * e + 1]));
+      }
       QT_CUDA(cudaMemcpyAsync(kd, ops.data(), sizeof(float2) * G * mat, cudaMemcpyHostToDevice, st),
               "cudaMemcpyAsync(Kraus operators)");
       QT_CUDA(launch_kraus_norms(psi, static_cast<int>(n), Q, qubits, static_cast<int>(G), kd, scr, st),
