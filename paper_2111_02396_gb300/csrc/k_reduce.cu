@@ -8,6 +8,7 @@
 // so results are bitwise reproducible run to run.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "kernels.h"
@@ -128,11 +129,18 @@ static int red_grid(Kern kern, uint64_t work_items) {
 // with basis bit j = the j-th lowest qubit (the callers reorder).
 //
 // q = 1, 2 (k_rdm): every entry in registers, W = 4^q reals: the 2^q diagonal
-// entries, then (re, im) of each b < a.  Bound by HBM: a thread keeps 8
-// 128-bit loads in flight (LOW0: qubit 0 is in Q, so members 2j and 2j + 1 of
-// a set share a load; otherwise two neighbouring sets do).  n = 29: q = 1
-// 654 -> 634 us, q = 2 834 -> 686 us (one set of 8-byte loads at a time and FP64
-// carries before); 4 GiB read at the copy rate take 634.
+// entries, then (re, im) of each b < a.  Bound by HBM: a thread keeps 4 to 16
+// 128-bit loads in flight (LOW0: qubit 0 is in Q, so members 2j and 2j + 1 of a
+// set share a load; otherwise two neighbouring sets do).  A call at n =
+// 29: q = 1 754 -> 670 us, q = 2 901 -> 660 (one set of 8-byte loads at a time
+// and FP64 carries before); 4 GiB read at the copy rate take 634.
+//
+// The FP32 runs are fixed, whatever the launch: with T streams (rdm_blocks),
+// stream t takes the sets t, t + T, t + 2 T, ... and carries after every
+// kRdmChunk of them.  A run's rounding (1e-10 of an entry at 20 qubits) goes
+// into the branch that a channel picks, normalized by 1 / sqrt(P) and rounded
+// to FP32: other runs would give other last bits of the state.  A thread has
+// two streams, 2p and 2p + 1, or with LOW0 one.
 // ---------------------------------------------------------------------------
 template <int Q>
 struct RdmArgs {
@@ -141,82 +149,98 @@ struct RdmArgs {
   uint64_t num_groups;
 };
 
-// Sets summed in FP32 before the carry: 16, and every set by itself (FINE)
-// where there are fewer than 2^20 of them.  The rounding of a run of R sets
-// leaves about R / sqrt(3 sets) * 3e-8 of an entry: 3e-10 at 2^20 sets with
-// R = 16, but it no longer averages out in small states.
-constexpr int kRdmChunk = 16;
-constexpr int kRdmFineLog = 20;
+constexpr int kRdmChunk = 16;     // sets summed in FP32 before the carry
+constexpr int kRdmThreads = kRedThreads / 2;
 
-template <int Q, bool LOW0, bool FINE>
-__global__ void __launch_bounds__(kRedThreads) k_rdm(const float4* __restrict__ psi,
+// T: 8 (q = 2: 3) times kRedThreads an SM, not more than the sets need
+template <int Q>
+static int rdm_blocks(uint64_t sets) {
+  const uint64_t need = (sets + kRedThreads - 1) / kRedThreads;
+  return static_cast<int>(std::min<uint64_t>({need, static_cast<uint64_t>(sm_count()) * (Q == 1 ? 8 : 3),
+                                              static_cast<uint64_t>(kMaxRedBlocks)}));
+}
+
+// streams of a thread
+__host__ __device__ constexpr int rdm_streams(bool low0) { return low0 ? 1 : 2; }
+
+template <int Q, bool LOW0>
+__global__ void __launch_bounds__(kRdmThreads, Q == 1 && LOW0 ? 16 : 1) k_rdm(const float4* __restrict__ psi,
                                                      const __grid_constant__ RdmArgs<Q> a,
                                                      float2* __restrict__ partial) {
   constexpr int D = 1 << Q, W = D * D;
   constexpr int NV = LOW0 ? D / 2 : D;        // loads per group
   constexpr int SPG = LOW0 ? 1 : 2;           // sets per group
   constexpr int NI = LOW0 ? Q : Q + 1;        // zeros inserted into the group index
-  constexpr int U = 8 / NV;                   // groups in flight
+  constexpr int ST = rdm_streams(LOW0);
+  constexpr int U = (LOW0 ? 4 * Q : 8 * Q) / NV;   // groups in flight
   cudaTriggerProgrammaticLaunchCompletion();
-  float h[W], l[W], f[W];
+  float h[W], l[W], f[ST][W];
 #pragma unroll
-  for (int c = 0; c < W; ++c) { h[c] = 0.f; l[c] = 0.f; f[c] = 0.f; }
-  int cnt = 0;
+  for (int c = 0; c < W; ++c) { h[c] = l[c] = f[0][c] = f[ST - 1][c] = 0.f; }
+  auto carry = [&] {
+#pragma unroll
+    for (int t = 0; t < ST; ++t)
+#pragma unroll
+      for (int k = 0; k < W; ++k) { df_acc(h[k], l[k], f[t][k]); f[t][k] = 0.f; }
+  };
   const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x;
-  for (uint64_t i = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < a.num_groups;
-       i += U * stride) {
-    float4 v[U][NV];
+  auto load = [&](uint64_t g, float4 (&v)[NV]) {
+    uint64_t base = g;
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const uint64_t g = i + u * stride;
-      uint64_t base = g;
-#pragma unroll
-      for (int b = 0; b < NI; ++b) {
-        const uint32_t s = a.ins[b];
-        base = ((base >> s) << (s + 1)) | (base & ((1ull << s) - 1ull));
-      }
-#pragma unroll
-      for (int m = 0; m < NV; ++m)
-        v[u][m] = g < a.num_groups ? __ldg(psi + (base >> 1) + a.offs[m]) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int b = 0; b < NI; ++b) {
+      const uint32_t s = a.ins[b];
+      base = ((base >> s) << (s + 1)) | (base & ((1ull << s) - 1ull));
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u)
+    for (int m = 0; m < NV; ++m) v[m] = __ldg(psi + (base >> 1) + a.offs[m]);
+  };
+  auto add = [&](const float4 (&v)[NV]) {
 #pragma unroll
-      for (int s = 0; s < SPG; ++s) {
-        float2 x[D];
+    for (int s = 0; s < SPG; ++s) {
+      float2 x[D];
 #pragma unroll
-        for (int m = 0; m < D; ++m) {
-          const float4 w = v[u][LOW0 ? m / 2 : m];
-          const bool second = LOW0 ? (m & 1) : s == 1;
-          x[m] = second ? make_float2(w.z, w.w) : make_float2(w.x, w.y);
-        }
-        int c = 0;
-#pragma unroll
-        for (int b = 0; b < D; ++b) { f[c] = fmaf(x[b].x, x[b].x, fmaf(x[b].y, x[b].y, f[c])); ++c; }
-#pragma unroll
-        for (int b = 0; b < D; ++b)
-#pragma unroll
-          for (int aa = b + 1; aa < D; ++aa) {
-            // x_b conj(x_a)
-            f[c] = fmaf(x[b].x, x[aa].x, fmaf(x[b].y, x[aa].y, f[c])); ++c;
-            f[c] = fmaf(x[b].y, x[aa].x, fmaf(-x[b].x, x[aa].y, f[c])); ++c;
-          }
-        if constexpr (FINE) {
-#pragma unroll
-          for (int k = 0; k < W; ++k) { df_acc(h[k], l[k], f[k]); f[k] = 0.f; }
-        }
+      for (int m = 0; m < D; ++m) {
+        const float4 w = v[LOW0 ? m / 2 : m];
+        const bool second = LOW0 ? (m & 1) : s == 1;
+        x[m] = second ? make_float2(w.z, w.w) : make_float2(w.x, w.y);
       }
-    cnt += U * SPG;
-    if (!FINE && cnt == kRdmChunk) {
+      float* const r = f[LOW0 ? 0 : s];
+      int c = 0;
 #pragma unroll
-      for (int k = 0; k < W; ++k) { df_acc(h[k], l[k], f[k]); f[k] = 0.f; }
+      for (int b = 0; b < D; ++b) { r[c] = fmaf(x[b].x, x[b].x, fmaf(x[b].y, x[b].y, r[c])); ++c; }
+#pragma unroll
+      for (int b = 0; b < D; ++b)
+#pragma unroll
+        for (int aa = b + 1; aa < D; ++aa) {
+          // x_b conj(x_a)
+          r[c] = fmaf(x[b].x, x[aa].x, fmaf(x[b].y, x[aa].y, r[c])); ++c;
+          r[c] = fmaf(x[b].y, x[aa].x, fmaf(-x[b].x, x[aa].y, r[c])); ++c;
+        }
+    }
+  };
+  int cnt = 0;
+  uint64_t i = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  // whole batches: no condition between the loads, or they would wait for one another
+  for (; i + (U - 1) * stride < a.num_groups; i += U * stride) {
+    float4 v[U][NV];
+#pragma unroll
+    for (int u = 0; u < U; ++u) load(i + u * stride, v[u]);
+#pragma unroll
+    for (int u = 0; u < U; ++u) add(v[u]);
+    cnt += U * SPG;                           // sets of the ST streams
+    if (cnt == ST * kRdmChunk) {
+      carry();
       cnt = 0;
     }
   }
-  if constexpr (!FINE) {
 #pragma unroll
-    for (int k = 0; k < W; ++k) df_acc(h[k], l[k], f[k]);
-  }
+  for (int u = 0; u < U; ++u)
+    if (i + u * stride < a.num_groups) {
+      float4 v[NV];
+      load(i + u * stride, v);
+      add(v);
+    }
+  carry();
   block_reduce_store<W>(h, l, partial);
 }
 
@@ -228,9 +252,8 @@ static void sort_qubits(const uint32_t* qubits, uint32_t* s) {
     for (int j = i; j > 0 && s[j - 1] > s[j]; --j) { const uint32_t t = s[j]; s[j] = s[j - 1]; s[j - 1] = t; }
 }
 
-template <int Q, bool LOW0, bool FINE>
+template <int Q, bool LOW0>
 static cudaError_t rdm_low(const float2* psi, int n, const uint32_t* s, const Scratch& scr, cudaStream_t st) {
-  constexpr int U = 8 / (LOW0 ? (1 << Q) / 2 : (1 << Q));
   RdmArgs<Q> a{};
   int ni = 0;
   if (!LOW0) a.ins[ni++] = 0;
@@ -243,12 +266,8 @@ static cudaError_t rdm_low(const float2* psi, int n, const uint32_t* s, const Sc
     a.offs[m] = o >> 1;
   }
   a.num_groups = 1ull << (n - Q - (LOW0 ? 0 : 1));
-  static PerDevice grid_dev;
-  const int grid = grid_dev.get([] { return red_grid(k_rdm<Q, LOW0, FINE>, ~0ull >> 1); });
-  const uint64_t per = static_cast<uint64_t>(kRedThreads) * U;
-  const uint64_t need = (a.num_groups + per - 1) / per;
-  const int g = static_cast<int>(need < static_cast<uint64_t>(grid) ? need : grid);
-  k_rdm<Q, LOW0, FINE><<<g, kRedThreads, 0, st>>>(reinterpret_cast<const float4*>(psi), a, scr.partials());
+  const int g = rdm_blocks<Q>(1ull << (n - Q)) * (2 / rdm_streams(LOW0));
+  k_rdm<Q, LOW0><<<g, kRdmThreads, 0, st>>>(reinterpret_cast<const float4*>(psi), a, scr.partials());
   return finalize(scr.partials(), g, 1 << (2 * Q), scr.result, st);
 }
 
@@ -372,7 +391,9 @@ __global__ void __launch_bounds__(kRdm3Threads, 4) k_rdm3(const float4* __restri
   if (tid < 64) partial[static_cast<size_t>(blockIdx.x) * 64 + tid] = df_add(part[tid], part[tid + 64]);
 }
 
-// sets summed in FP32 before the carry: the bound given at kRdmChunk
+// Sets summed in FP32 before the carry.  The rounding of a run of R sets leaves
+// about R / sqrt(3 sets) * 3e-8 of an entry (3e-10 at 2^20 sets with R = 16),
+// but it does not average out in small states.
 static int carry_run(double scale, int log_sets, int cap) {
   const double r = scale * exp2(0.5 * log_sets);
   return r < 1.0 ? 1 : (r > cap ? cap : static_cast<int>(r));
@@ -417,7 +438,7 @@ static cudaError_t rdm3_low(const float2* psi, int n, const uint32_t* s, const S
 // fall into different banks.  FP32 runs are carried in double-floats held in
 // shared memory, which leaves 128 registers a thread, two CTAs an SM.  A
 // run's length grows with the number of sets, for the reason given at
-// kRdmChunk; a wide channel's probabilities average the error of 4^q entries,
+// carry_run; a wide channel's probabilities average the error of 4^q entries,
 // so its runs may be longer.
 // n = 25, q = 4 / 5: 138 / 158 us; the products K_i v that gave these
 // channels' probabilities before took 2719 / 1584 us for each 16 / 4 operators.
@@ -626,9 +647,7 @@ template <int Q>
 static cudaError_t rdm_q(const float2* psi, int n, const uint32_t* qubits, const Scratch& scr, cudaStream_t st) {
   uint32_t s[Q];
   sort_qubits<Q>(qubits, s);
-  if (n - Q < kRdmFineLog)
-    return s[0] == 0 ? rdm_low<Q, true, true>(psi, n, s, scr, st) : rdm_low<Q, false, true>(psi, n, s, scr, st);
-  return s[0] == 0 ? rdm_low<Q, true, false>(psi, n, s, scr, st) : rdm_low<Q, false, false>(psi, n, s, scr, st);
+  return s[0] == 0 ? rdm_low<Q, true>(psi, n, s, scr, st) : rdm_low<Q, false>(psi, n, s, scr, st);
 }
 
 cudaError_t launch_rdm(const float2* psi, int n, int q, const uint32_t* qubits, const Scratch& scr,
