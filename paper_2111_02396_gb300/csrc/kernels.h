@@ -107,17 +107,19 @@ cudaError_t launch_apply6_fp32(float2* psi, int n, const uint32_t* targets, cons
 // 64 x 64 operator (basis bit b <-> qubits[b]), n >= 6
 cudaError_t launch_norms64(const float2* psi, int n, const uint32_t* qubits, const float2* kdev, float2* partial,
                            int* blocks, cudaStream_t st);
-// multi-gate pass: up to kGroupMaxGates fused gates (width <= 4, targets
-// ascending, matrix row-major) whose qubits lie in {0..6} plus at most 6
-// higher qubits, applied in one pass over the state (n >= 7 + #high qubits)
-constexpr int kGroupMaxGates = 8;
-constexpr int kGroupMaxHigh = 6;
-struct GroupPiece {
+// multi-gate pass: up to kMultiGates fused gates (width <= 4, n >= 7 + width,
+// targets ascending, matrix row-major) whose qubits, with the lowest kMultiLow,
+// number at most kMultiBits, applied in order in one pass over the state;
+// multi_fits: whether they are
+constexpr int kMultiBits = 12, kMultiLow = 4, kMultiGates = 48, kMultiEntries = 2176;
+constexpr int kMultiFewLog = 12;
+struct MultiPiece {
   int k;
   uint32_t targets[4];
   const float2* u;
 };
-cudaError_t launch_apply_group(float2* psi, int n, int ng, const GroupPiece* pieces, cudaStream_t st);
+bool multi_fits(int n, int ng, const MultiPiece* pieces);
+cudaError_t launch_multi(float2* psi, int n, int ng, const MultiPiece* pieces, cudaStream_t st);
 // tensor-core path (split-TF32, k = 4..6, n >= k + 7): W is the real
 // embedding of U, row-major [2^(k+1) x 2^(k+1)] FP32 in device memory; *err
 // is set (nonzero) if a bounded wait in the kernel ran out

@@ -540,10 +540,6 @@ struct Controller {
     return launch_pieces(psi, rest);
   }
 
-  // Launch the pieces of a segment in order.  With QT_FLAG_MULTI_GATE, consecutive
-  // pieces (moved earlier past pieces they share no qubit with) whose qubits
-  // lie in {0..6} plus at most kGroupMaxHigh higher qubits share one
-  // multi-gate pass over the state.
   // Peephole merge of a segment's pieces, extending the fusion of Sec. III.B
   // across the cuts that flush points make: a piece moves forward to the
   // first later piece that shares a qubit with it (every piece in between
@@ -603,57 +599,53 @@ struct Controller {
     R.stats.merged_pieces += merged;
   }
 
+  // Launch the pieces of a segment.  Consecutive pieces that fit one tile share
+  // a pass over the state (multi_fits).  With QT_FLAG_MULTI_GATE a pass also
+  // takes later pieces, moved past pieces they share no qubit with.
   qt_status launch_pieces(float2* psi, std::vector<Piece>& pieces) {
     merge_pieces(pieces);
-    const bool group = (R.p.flags & QT_FLAG_MULTI_GATE) && R.n >= 8;
-    const int hmax = std::min<int>(kGroupMaxHigh, static_cast<int>(R.n) - 7);
-    const uint64_t low = (1ull << 7) - 1ull;
+    const int n = static_cast<int>(R.n);
+    const bool reorder = (R.p.flags & QT_FLAG_MULTI_GATE) != 0;
     std::vector<char> done(pieces.size(), 0);
-    std::vector<size_t> members;
+    MultiPiece mp[kMultiGates];
     for (size_t a = 0; a < pieces.size(); ++a) {
       if (done[a]) continue;
-      done[a] = 1;
-      members.assign(1, a);
-      const int wa = static_cast<int>(pieces[a].targets.size());
-      const bool groupable_a = group && wa <= 4 && !use_tc(wa) &&
-                               std::popcount(pieces[a].full & ~low) <= hmax;
-      if (groupable_a) {
-        uint64_t hm = pieces[a].full & ~low, blocked = 0;
-        for (size_t b = a + 1; b < pieces.size() && b < a + 64 &&
-                               members.size() < static_cast<size_t>(kGroupMaxGates); ++b) {
+      int ng = 0;
+      auto take = [&](size_t b) {                // whether piece b joins the pass
+        const Piece& P = pieces[b];
+        const int w = static_cast<int>(P.targets.size());
+        if (ng == kMultiGates || w > 4 || use_tc(w)) return false;
+        mp[ng].k = w;
+        for (int i = 0; i < w; ++i) mp[ng].targets[i] = P.targets[i];
+        mp[ng].u = P.u;
+        if (!multi_fits(n, ng + 1, mp)) return false;
+        ++ng;
+        done[b] = 1;
+        return true;
+      };
+      if (take(a)) {
+        uint64_t blocked = 0;                    // qubits of the pieces left behind
+        for (size_t b = a + 1; b < pieces.size() && b < a + 64; ++b) {
           if (done[b]) continue;
-          const Piece& P = pieces[b];
-          const int wb = static_cast<int>(P.targets.size());
-          if ((P.full & blocked) == 0 && wb <= 4 && std::popcount(hm | (P.full & ~low)) <= hmax) {
-            hm |= P.full & ~low;
-            members.push_back(b);
-            done[b] = 1;
-            continue;
-          }
-          blocked |= P.full;
+          if (!(pieces[b].full & blocked) && take(b)) continue;
+          if (!reorder) break;
+          blocked |= pieces[b].full;
         }
       }
-      if (members.size() == 1) {
+      done[a] = 1;
+      if (ng <= 1) {
         qt_status s = apply(psi, pieces[a].targets, pieces[a].u);
         if (s != QT_OK) return s;
         R.stats.fused_pieces++;
         continue;
       }
-      GroupPiece gp[kGroupMaxGates];
-      for (size_t i = 0; i < members.size(); ++i) {
-        const Piece& P = pieces[members[i]];
-        gp[i].k = static_cast<int>(P.targets.size());
-        for (size_t b = 0; b < P.targets.size(); ++b) gp[i].targets[b] = P.targets[b];
-        gp[i].u = P.u;
-        const size_t d = 1ull << P.targets.size();
-        R.stats.h2d_bytes += sizeof(float2) * d * d;
-      }
+      for (int i = 0; i < ng; ++i) R.stats.h2d_bytes += sizeof(float2) << (2 * mp[i].k);
       qt_status s = timed_launch([&](cudaError_t& e) {
-        e = launch_apply_group(psi, static_cast<int>(R.n), static_cast<int>(members.size()), gp, R.st);
+        e = launch_multi(psi, n, ng, mp, R.st);
         return QT_OK;
       }, "multi-gate pass launch", 0);
       if (s != QT_OK) return s;
-      R.stats.fused_pieces += members.size();
+      R.stats.fused_pieces += static_cast<uint64_t>(ng);
     }
     return QT_OK;
   }
