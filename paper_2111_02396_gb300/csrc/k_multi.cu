@@ -20,18 +20,21 @@
 //     each; latency and launches count.
 //   - Many tiles: 128 threads, 4 CTAs an SM; a thread takes 8 sets of 1 or 2
 //     qubits, 4 of 3, 2 of 4 (96 registers of members), so that an entry is
-//     loaded once for all of them.  A packed FMA takes a matrix pair from the
-//     constant bank only where it is used once; with several sets the pair is
-//     moved to registers, which pays from 4 sets on (2 sets: scalar FMAs).
-// Bound by issue (85% of the slots with 4-qubit gates) rather than HBM from two
-// gates a pass on.  Grouping pays at every size, so whatever fits is grouped.
-// Device time of a grid circuit, one pass a gate -> grouped, fused to at most
-// 2, 3 and 4 qubits (in ms; n = 28: 211, 121 and 70 gates in 47, 46 and 33 passes):
-//   n = 28   129 -> 58.8   79.6 -> 60.4   51.4 -> 48.2
-//   n = 20  1.57 -> 0.60   0.97 -> 0.56   0.69 -> 0.50
-//   n = 12 (with the probability passes) 0.18   0.18   0.20
-// and of 200 gates on random qubits, n = 26: 15.4 -> 6.6, 9.3 -> 6.4, 7.1 -> 6.3;
-// n = 13: 0.92 -> 0.23, 0.52 -> 0.22, 0.39 -> 0.21.
+//     loaded once for all of them.  The FMAs are scalar: they take an entry
+//     from its uniform register however often it is used, where a packed FMA
+//     takes a pair of them only once and otherwise wants it moved to registers
+//     (n = 28, packed and scalar: 2 qubits 58.8 and 51.8 ms, 3 qubits 60.4 and
+//     46.8).  64 threads with 4 sets of 4 qubits need 15% fewer instructions
+//     but leave 8 warps an SM: 51.8 ms for 45.2.
+// Bound by issue (82% of the slots with 4-qubit gates, 59% of them FMAs) rather
+// than HBM from two gates a pass on.  Grouping pays at every size, so whatever
+// fits is grouped.  Device time of a grid circuit, one pass a gate -> grouped,
+// fused to at most 2, 3 and 4 qubits (in ms; n = 28: 211, 121 and 70 gates in
+// 47, 46 and 33 passes):
+//   n = 28   129 -> 51.8   79.6 -> 46.8   51.4 -> 45.2
+//   n = 20  1.57 -> 0.60   0.97 -> 0.49   0.69 -> 0.49
+// and of 200 gates on random qubits, n = 26: 15.4 -> 5.8, 9.3 -> 4.9, 7.1 -> 6.0;
+// n = 13: 0.92 -> 0.22, 0.52 -> 0.19, 0.39 -> 0.21.
 #include <cuda_runtime.h>
 
 #include "kernels.h"
@@ -73,12 +76,10 @@ __device__ __forceinline__ uint32_t swizzle(uint32_t l, uint64_t t) {
 template <int K, int B, int T, int CAP>
 __device__ __forceinline__ void gate(float2* sm, const Args<CAP>& a, const Gate& g) {
   constexpr int M = 1 << K;
-  constexpr bool PACKED = B >= 4;
   const uint32_t sets = 1u << (a.bits - K);
   for (uint32_t s0 = threadIdx.x; s0 < sets; s0 += B * T) {   // B > 1: sets is a multiple of B T
     uint32_t base[B];
-    float2 sb[B][M];                               // (s, b) of member m
-    float2 aa[(B + 1) / 2][M];                     // a of two sets
+    float va[B][M], vb[B][M], vs[B][M];            // a, b and s = a + b of member m
     uint32_t s = s0;
 #pragma unroll
     for (int i = 0; i < K; ++i) {
@@ -92,43 +93,33 @@ __device__ __forceinline__ void gate(float2* sm, const Args<CAP>& a, const Gate&
 #pragma unroll
       for (int m = 0; m < M; ++m) {
         const float2 v = *slot(sm, base[b] ^ g.smoff[m]);
-        sb[b][m] = make_float2(v.x + v.y, v.y);
-        if (b & 1) aa[b / 2][m].y = v.x;
-        else aa[b / 2][m].x = v.x;
+        va[b][m] = v.x;
+        vb[b][m] = v.y;
+        vs[b][m] = v.x + v.y;
       }
     }
     const float4* const ce = a.ce + g.mat / 2;
     const float4* const ff = a.f + g.mat / 4;
-#pragma unroll 4
+#pragma unroll 8
     for (int j = 0; j < M; ++j) {
-      float2 tr[B], im[(B + 1) / 2];
+      float cs[B], eb[B], fa[B];
 #pragma unroll
-      for (int b = 0; b < B; ++b) tr[b] = im[b / 2] = make_float2(0.f, 0.f);
+      for (int b = 0; b < B; ++b) cs[b] = eb[b] = fa[b] = 0.f;
 #pragma unroll
       for (int m = 0; m < M; ++m) {
-        const int e = j * M + m;
-        const float4 x2 = ce[e >> 1], f4 = ff[e >> 2];
-        const float2 x = e & 1 ? make_float2(x2.z, x2.w) : make_float2(x2.x, x2.y);
-        const float f = e & 2 ? (e & 1 ? f4.w : f4.z) : (e & 1 ? f4.y : f4.x);
-        if constexpr (PACKED) {
+        const int x = j * M + m;
+        const float4 u = ce[x >> 1], w = ff[x >> 2];
+        const float c = x & 1 ? u.z : u.x, e = x & 1 ? u.w : u.y;
+        const float f = x & 2 ? (x & 1 ? w.w : w.z) : (x & 1 ? w.y : w.x);
 #pragma unroll
-          for (int b = 0; b < B; ++b) tr[b] = __ffma2_rn(x, sb[b][m], tr[b]);
-#pragma unroll
-          for (int b = 0; b < B / 2; ++b) im[b] = __ffma2_rn(make_float2(f, f), aa[b][m], im[b]);
-        } else {
-#pragma unroll
-          for (int b = 0; b < B; ++b) {
-            tr[b].x = fmaf(x.x, sb[b][m].x, tr[b].x);
-            tr[b].y = fmaf(x.y, sb[b][m].y, tr[b].y);
-            if (b & 1) im[b / 2].y = fmaf(f, aa[b / 2][m].y, im[b / 2].y);
-            else im[b / 2].x = fmaf(f, aa[b / 2][m].x, im[b / 2].x);
-          }
+        for (int b = 0; b < B; ++b) {
+          cs[b] = fmaf(c, vs[b][m], cs[b]);
+          eb[b] = fmaf(e, vb[b][m], eb[b]);
+          fa[b] = fmaf(f, va[b][m], fa[b]);
         }
       }
 #pragma unroll
-      for (int b = 0; b < B; ++b)
-        *slot(sm, base[b] ^ g.smoff[j]) =
-            make_float2(tr[b].x - tr[b].y, tr[b].x + (b & 1 ? im[b / 2].y : im[b / 2].x));
+      for (int b = 0; b < B; ++b) *slot(sm, base[b] ^ g.smoff[j]) = make_float2(cs[b] - eb[b], cs[b] + fa[b]);
     }
   }
 }
