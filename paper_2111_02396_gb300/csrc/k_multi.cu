@@ -16,8 +16,11 @@
 // What feeds the FMAs decides the form.  The matrix sits in the kernel
 // parameters and comes through uniform loads (8 bytes at most) from the
 // constant bank.
-//   - Few tiles (n <= kMultiFewLog: at most two an SM): 512 threads, a set
-//     each; latency and launches count.
+//   - One tile (n <= kMultiFewLog): 512 threads, a set each; what counts is the
+//     chain of dependent loads of a gate.  Whole warps drop out together where
+//     there are fewer sets, which keeps the matrix loads uniform (per-thread
+//     ones: n = 12, 26 -> 46 us a pass of 8 gates on 4 qubits; n = 10, 25 -> 33
+//     of 32 on 2).
 //   - Many tiles: 128 threads, 4 CTAs an SM; a thread takes 8 sets of 1 or 2
 //     qubits, 4 of 3, 2 of 4 (96 registers of members), so that an entry is
 //     loaded once for all of them.  The FMAs are scalar: they take an entry
@@ -31,7 +34,7 @@
 // fits is grouped.  Device time of a grid circuit, one pass a gate -> grouped,
 // fused to at most 2, 3 and 4 qubits (in ms; n = 28: 211, 121 and 70 gates in
 // 47, 46 and 33 passes):
-//   n = 28   129 -> 51.8   79.6 -> 46.8   51.4 -> 45.2
+//   n = 28   129 -> 51.0   79.6 -> 45.7   51.4 -> 44.6
 //   n = 20  1.57 -> 0.60   0.97 -> 0.49   0.69 -> 0.49
 // and of 200 gates on random qubits, n = 26: 15.4 -> 5.8, 9.3 -> 4.9, 7.1 -> 6.0;
 // n = 13: 0.92 -> 0.22, 0.52 -> 0.19, 0.39 -> 0.21.
@@ -74,10 +77,13 @@ __device__ __forceinline__ uint32_t swizzle(uint32_t l, uint64_t t) {
 }
 
 template <int K, int B, int T, int CAP>
-__device__ __forceinline__ void gate(float2* sm, const Args<CAP>& a, const Gate& g) {
+__device__ __forceinline__ void gate(float2* sm, const Args<CAP>& a, const Gate& g, uint32_t warp) {
   constexpr int M = 1 << K;
-  const uint32_t sets = 1u << (a.bits - K);
-  for (uint32_t s0 = threadIdx.x; s0 < sets; s0 += B * T) {   // B > 1: sets is a multiple of B T
+  const uint32_t sets = 1u << (a.bits - K);        // 128 or more; with B > 1 a multiple of B T
+  // whole warps loop together: a condition on the thread would make every
+  // matrix entry a per-thread load instead of a uniform one
+  for (uint32_t w = warp; w < sets; w += B * T) {
+    const uint32_t s0 = w + (threadIdx.x & 31u);
     uint32_t base[B];
     float va[B][M], vb[B][M], vs[B][M];            // a, b and s = a + b of member m
     uint32_t s = s0;
@@ -159,14 +165,15 @@ __global__ void __launch_bounds__(T, T == kThreads ? 4 : 1) k_multi(float2* __re
         sm[s1 + 2u * T * c] = make_float2(buf[c].z, buf[c].w);
       }
   }
+  const uint32_t warp = __shfl_sync(0xffffffffu, tid & ~31u, 0);   // first thread of the warp
   for (int i = 0; i < a.ng; ++i) {
     __syncthreads();
     const Gate& g = a.g[i];
     switch (g.k) {
-      case 1: gate<1, FEW ? 1 : 8, T, CAP>(sm, a, g); break;
-      case 2: gate<2, FEW ? 1 : 8, T, CAP>(sm, a, g); break;
-      case 3: gate<3, FEW ? 1 : 4, T, CAP>(sm, a, g); break;
-      default: gate<4, FEW ? 1 : 2, T, CAP>(sm, a, g); break;
+      case 1: gate<1, FEW ? 1 : 8, T, CAP>(sm, a, g, warp); break;
+      case 2: gate<2, FEW ? 1 : 8, T, CAP>(sm, a, g, warp); break;
+      case 3: gate<3, FEW ? 1 : 4, T, CAP>(sm, a, g, warp); break;
+      default: gate<4, FEW ? 1 : 2, T, CAP>(sm, a, g, warp); break;
     }
   }
   __syncthreads();
