@@ -55,8 +55,9 @@ struct alignas(16) Gate {       // the parameters stay 16-byte aligned from gate
   uint8_t k, tins[4], pad[7];
 };
 
-// CAP: matrix entries of a launch.  Parameters are copied with every launch,
-// so there is a small form for the common one or two gates.
+// CAP: matrix entries of a launch.  Parameters are copied with every launch
+// (12 us of the host for 32 KB, 4 for 12), so there are smaller forms: 512 for
+// the one or two gates common in large states, 1024 for 48 gates on 2 qubits.
 template <int CAP>
 struct alignas(16) Args {
   float4 ce[CAP / 2];         // (c, e) of two entries, row-major per gate
@@ -308,7 +309,9 @@ cudaError_t launch_multi(float2* psi, int n, int ng, const MultiPiece* p, cudaSt
   if (!multi_fits(n, ng, p)) return cudaErrorInvalidValue;
   int entries = 0;
   for (int i = 0; i < ng; ++i) entries += 1 << (2 * p[i].k);
-  return entries <= 512 ? launch_cap<512>(psi, n, ng, p, st) : launch_cap<kMultiEntries>(psi, n, ng, p, st);
+  if (entries <= 512) return launch_cap<512>(psi, n, ng, p, st);
+  if (entries <= 1024) return launch_cap<1024>(psi, n, ng, p, st);
+  return launch_cap<kMultiEntries>(psi, n, ng, p, st);
 }
 
 }  // namespace qt

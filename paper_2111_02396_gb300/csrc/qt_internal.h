@@ -65,9 +65,19 @@ void clear_error();
 // ---- host linear algebra (host_circuit.cpp) --------------------------------
 // smallest eigenvalue of a Hermitian d x d matrix (row-major)
 double hermitian_min_eig(int d, const cd* A);
-// v (2^w) <- A v where A acts on `q` qubits at positions pos[0..q-1] of the
-// w-qubit index (bit b of A's index <-> position pos[b])
-void apply_small(cd* v, int w, int q, const int* pos, const cd* A);
+// Product of small operators on w qubits, V (2^w x 2^w, row-major; there after
+// the first apply): V <- A V where A acts on `q` qubits at positions
+// pos[0..q-1] of the w-qubit index (bit b of A's index <-> position pos[b])
+struct SmallProduct {
+  int w = 0;
+  std::vector<double> re, im;
+  void start(int width);
+  void apply(int q, const int* pos, const cd* A);
+
+ private:
+  bool identity = true;
+  std::vector<double> ore, oim;
+};
 // matrix (row-major, 2^w x 2^w, basis `targets`) of the product of ops, in
 // order, each given by (op index, operator matrix)
 void compose(const Circuit& c, const std::vector<uint32_t>& targets,
