@@ -92,8 +92,8 @@ struct Dev {
   const uint32_t* order;
   float2* arena;                    // per-CTA slots, or per-trajectory when keeping states
   uint64_t slot_amps;               // amplitudes per CTA slot (0: use traj.arena_off)
-  int32_t* kraus;
-  int32_t* stage;
+  int8_t* kraus;                   // records: bytes (at most 64 operators), -1 undecided
+  int8_t* stage;
   uint8_t* gflag;                   // per fused gate of the run: a member channel holds a non-default stage-1 choice
   uint64_t* samples;
   uint32_t* flushes;
@@ -766,7 +766,7 @@ __device__ __forceinline__ void cta_stage1(const Dev& d, const Traj& T, uint64_t
       }
     }
     if (lead) {
-      d.kraus[T.ch0 + c] = ch;
+      d.kraus[T.ch0 + c] = static_cast<int8_t>(ch);
       d.stage[T.ch0 + c] = ch >= 0 ? 1 : 0;
       if (ch != static_cast<int>(st.def)) d.gflag[T.gf0 + op.gate] = 1;
     }
@@ -848,7 +848,7 @@ __device__ __noinline__ void cta_stage2(const Dev& d, const Traj& T, const float
         for (int b = 0; b < D; ++b)
           Pc += M[2 * (a * D + b)] * rho[2 * (b * D + a)] - M[2 * (a * D + b) + 1] * rho[2 * (b * D + a) + 1];
     }
-    d.kraus[T.ch0 + fch] = chosen;
+    d.kraus[T.ch0 + fch] = static_cast<int8_t>(chosen);
     d.stage[T.ch0 + fch] = 2;
     sh.pend_pos = static_cast<int>(hi);
     sh.pend_choice = chosen;
@@ -1377,7 +1377,7 @@ struct qt_batch {
   uint64_t lane_samples = 0;        // merged launches: total sample slots
   qt_batch_params last{};
   // results on the host
-  std::vector<int32_t> kraus, stage;
+  std::vector<int8_t> kraus, stage;
   std::vector<uint64_t> samples;
   std::vector<uint32_t> flushes, folds;
   double device_ms = 0.0;
@@ -1830,16 +1830,16 @@ qt_status qt_batch_run(qt_batch* b, const qt_batch_params* p) {
     b->keep = p->keep_states ? 1u : 0u;
     auto align = [](size_t x) { return (x + 255) & ~size_t(255); };
     size_t off = 0;
-    b->off_kraus = off; off = align(off + sizeof(int32_t) * std::max<uint32_t>(b->total_ch, 1));
-    b->off_stage = off; off = align(off + sizeof(int32_t) * std::max<uint32_t>(b->total_ch, 1));
+    b->off_kraus = off; off = align(off + std::max<size_t>(b->total_ch, 1));
+    b->off_stage = off; off = align(off + std::max<size_t>(b->total_ch, 1));
     b->off_samples = off; off = align(off + sizeof(uint64_t) * std::max<uint64_t>(uint64_t(b->num) * b->S, 1));
     b->off_flushes = off; off = align(off + sizeof(uint32_t) * b->num);
     b->off_folds = off; off = align(off + sizeof(uint32_t) * b->num);
     b->off_gflag = off; off = align(off + std::max<uint64_t>(b->total_gates, 1));
     if (!b->outs.alloc(off)) return set_error(QT_ERR_OUT_OF_MEMORY, "qt_batch_run: outputs");
     uint8_t* o = static_cast<uint8_t*>(b->outs.p);
-    d.kraus = reinterpret_cast<int32_t*>(o + b->off_kraus);
-    d.stage = reinterpret_cast<int32_t*>(o + b->off_stage);
+    d.kraus = reinterpret_cast<int8_t*>(o + b->off_kraus);
+    d.stage = reinterpret_cast<int8_t*>(o + b->off_stage);
     d.samples = reinterpret_cast<uint64_t*>(o + b->off_samples);
     d.flushes = reinterpret_cast<uint32_t*>(o + b->off_flushes);
     d.folds = reinterpret_cast<uint32_t*>(o + b->off_folds);
@@ -1906,8 +1906,8 @@ qt_status qt_batch_run(qt_batch* b, const qt_batch_params* p) {
   }
   if (e == cudaSuccess) e = cudaEventRecord(e1, st);
   b->last = *p;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(b->kraus.data(), d.kraus, sizeof(int32_t) * b->total_ch, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(b->stage.data(), d.stage, sizeof(int32_t) * b->total_ch, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(b->kraus.data(), d.kraus, b->total_ch, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(b->stage.data(), d.stage, b->total_ch, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess && b->S)
     e = cudaMemcpyAsync(b->samples.data(), d.samples, sizeof(uint64_t) * b->samples.size(), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(b->flushes.data(), d.flushes, sizeof(uint32_t) * b->num, cudaMemcpyDeviceToHost, st);
@@ -1936,8 +1936,8 @@ qt_status qt_batch_kraus_indices(const qt_batch* b, uint32_t i, int32_t* kraus, 
   const bt::Traj& T = b->traj[i];
   if (num_channels) *num_channels = T.nch;
   if ((kraus || stage) && cap < T.nch) return set_error(QT_ERR_INVALID_ARG, "qt_batch_kraus_indices: cap %zu < %u", cap, T.nch);
-  if (kraus && T.nch) std::memcpy(kraus, b->kraus.data() + T.ch0, sizeof(int32_t) * T.nch);
-  if (stage && T.nch) std::memcpy(stage, b->stage.data() + T.ch0, sizeof(int32_t) * T.nch);
+  if (kraus) std::copy_n(b->kraus.data() + T.ch0, T.nch, kraus);
+  if (stage) std::copy_n(b->stage.data() + T.ch0, T.nch, stage);
   return QT_OK;
 }
 
@@ -2102,16 +2102,16 @@ qt_status lane_run(BatchLane* L, uint32_t num, const LaneTraj* tr, uint64_t* sam
   if (s != QT_OK) return s;
   auto align = [](size_t x) { return (x + 255) & ~size_t(255); };
   size_t off = 0;
-  const size_t o_kraus = off; off = align(off + sizeof(int32_t) * std::max<uint32_t>(b->total_ch, 1));
-  const size_t o_stage = off; off = align(off + sizeof(int32_t) * std::max<uint32_t>(b->total_ch, 1));
+  const size_t o_kraus = off; off = align(off + std::max<size_t>(b->total_ch, 1));
+  const size_t o_stage = off; off = align(off + std::max<size_t>(b->total_ch, 1));
   const size_t o_samp = off; off = align(off + sizeof(uint64_t) * std::max<uint64_t>(b->lane_samples, 1));
   const size_t o_flush = off; off = align(off + sizeof(uint32_t) * num);
   const size_t o_gflag = off; off = align(off + std::max<uint64_t>(b->total_gates, 1));
   if (b->outs.bytes < off && !b->outs.alloc(off)) return set_error(QT_ERR_OUT_OF_MEMORY, "lane_run: outputs");
   uint8_t* o = static_cast<uint8_t*>(b->outs.p);
   bt::Dev d = b->dev;
-  d.kraus = reinterpret_cast<int32_t*>(o + o_kraus);
-  d.stage = reinterpret_cast<int32_t*>(o + o_stage);
+  d.kraus = reinterpret_cast<int8_t*>(o + o_kraus);
+  d.stage = reinterpret_cast<int8_t*>(o + o_stage);
   d.samples = reinterpret_cast<uint64_t*>(o + o_samp);
   d.flushes = reinterpret_cast<uint32_t*>(o + o_flush);
   d.folds = nullptr;
