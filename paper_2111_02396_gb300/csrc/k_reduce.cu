@@ -142,11 +142,31 @@ static int red_grid(Kern kern, uint64_t work_items) {
 // to FP32: other runs would give other last bits of the state.  A thread has
 // two streams, 2p and 2p + 1, or with LOW0 one.
 // ---------------------------------------------------------------------------
+// f + Im(b conj a), added as (-b.x a.y), (b.y a.x), or the other way round (rev)
+__device__ __forceinline__ float cross(float2 b, float2 a, float f, bool rev) {
+  const float u = rev ? b.y : -b.x, v = rev ? a.x : a.y, w = rev ? -b.x : b.y, z = rev ? a.y : a.x;
+  return fmaf(w, z, fmaf(u, v, f));
+}
+
+// whether sorted member b comes after member a in the caller's order of the
+// qubits (his basis bit j is the rank[j]-th lowest of them): the two products
+// of an imaginary part are added in that order, which shows in the last bits
+// of small states
+static bool member_after(int q, const int* rank, int b, int a) {
+  int ub = 0, ua = 0;
+  for (int j = 0; j < q; ++j) {
+    ub |= ((b >> rank[j]) & 1) << j;
+    ua |= ((a >> rank[j]) & 1) << j;
+  }
+  return ub > ua;
+}
+
 template <int Q>
 struct RdmArgs {
   uint64_t offs[1 << Q];      // 128-bit word offset of load m within a group
   uint32_t ins[Q + 1];        // ascending bit positions to insert zeros at
   uint64_t num_groups;
+  bool rev;                   // q = 2: the caller's members 1 and 2 are swapped
 };
 
 constexpr int kRdmChunk = 16;     // sets summed in FP32 before the carry
@@ -214,7 +234,7 @@ __global__ void __launch_bounds__(kRdmThreads, Q == 1 && LOW0 ? 16 : 1) k_rdm(co
         for (int aa = b + 1; aa < D; ++aa) {
           // x_b conj(x_a)
           r[c] = fmaf(x[b].x, x[aa].x, fmaf(x[b].y, x[aa].y, r[c])); ++c;
-          r[c] = fmaf(x[b].y, x[aa].x, fmaf(-x[b].x, x[aa].y, r[c])); ++c;
+          r[c] = cross(x[b], x[aa], r[c], Q == 2 && b == 1 && aa == 2 && a.rev); ++c;
         }
     }
   };
@@ -253,8 +273,10 @@ static void sort_qubits(const uint32_t* qubits, uint32_t* s) {
 }
 
 template <int Q, bool LOW0>
-static cudaError_t rdm_low(const float2* psi, int n, const uint32_t* s, const Scratch& scr, cudaStream_t st) {
+static cudaError_t rdm_low(const float2* psi, int n, const uint32_t* qubits, const uint32_t* s, const Scratch& scr,
+                           cudaStream_t st) {
   RdmArgs<Q> a{};
+  a.rev = Q == 2 && qubits[0] != s[0];
   int ni = 0;
   if (!LOW0) a.ins[ni++] = 0;
   for (int b = 0; b < Q; ++b) a.ins[ni++] = s[b];
@@ -286,11 +308,13 @@ struct Rdm3Args {
   uint32_t ins[4];            // ascending bit positions to insert zeros at
   uint64_t num_groups;
   int run;                    // sets summed in FP32 before the carry
+  uint32_t rev;               // pairs in the other order: bits 0..5 within a half, 8 + 4 y + x of the corner
 };
 
 constexpr int kRdm3Threads = 128;
+constexpr int kRdm3OrderLog = 18;   // fewer sets than this: imaginary parts in the caller's order (3e-11 of an entry beyond)
 
-template <bool LOW0>
+template <bool LOW0, bool PERM>
 __global__ void __launch_bounds__(kRdm3Threads, 4) k_rdm3(const float4* __restrict__ psi, const __grid_constant__ Rdm3Args a,
                                                           float2* __restrict__ partial) {
   constexpr int NV = LOW0 ? 2 : 4;            // loads per half-group
@@ -358,12 +382,13 @@ __global__ void __launch_bounds__(kRdm3Threads, 4) k_rdm3(const float4* __restri
         int c = 0;
 #pragma unroll
         for (int b = 0; b < 4; ++b) { f[c] = fmaf(own[b].x, own[b].x, fmaf(own[b].y, own[b].y, f[c])); ++c; }
+        int pair = 0;
 #pragma unroll
         for (int b = 0; b < 4; ++b)
 #pragma unroll
           for (int aa = b + 1; aa < 4; ++aa) {
             f[c] = fmaf(own[b].x, own[aa].x, fmaf(own[b].y, own[aa].y, f[c])); ++c;
-            f[c] = fmaf(own[b].y, own[aa].x, fmaf(-own[b].x, own[aa].y, f[c])); ++c;
+            f[c] = cross(own[b], own[aa], f[c], PERM && ((a.rev >> pair) & 1u)); ++c; ++pair;
           }
 #pragma unroll
         for (int p = 0; p < 4; ++p)
@@ -371,7 +396,7 @@ __global__ void __launch_bounds__(kRdm3Threads, 4) k_rdm3(const float4* __restri
           for (int q = 0; q < 2; ++q) {
             // y_q conj(x_p)
             f[c] = fmaf(y[q].x, x[p].x, fmaf(y[q].y, x[p].y, f[c])); ++c;
-            f[c] = fmaf(y[q].y, x[p].x, fmaf(-y[q].x, x[p].y, f[c])); ++c;
+            f[c] = cross(y[q], x[p], f[c], PERM && ((a.rev >> (8 + 4 * (upper ? q + 2 : q) + p)) & 1u)); ++c;
           }
         if (++run == a.run) { flush(); run = 0; }
       }
@@ -399,8 +424,9 @@ static int carry_run(double scale, int log_sets, int cap) {
   return r < 1.0 ? 1 : (r > cap ? cap : static_cast<int>(r));
 }
 
-template <bool LOW0>
-static cudaError_t rdm3_low(const float2* psi, int n, const uint32_t* s, const Scratch& scr, cudaStream_t st) {
+template <bool LOW0, bool PERM>
+static cudaError_t rdm3_low(const float2* psi, int n, const uint32_t* s, uint32_t rev, const Scratch& scr,
+                            cudaStream_t st) {
   Rdm3Args a{};
   int ni = 0;
   if (!LOW0) a.ins[ni++] = 0;
@@ -412,17 +438,18 @@ static cudaError_t rdm3_low(const float2* psi, int n, const uint32_t* s, const S
   a.half = (1ull << s[2]) >> 1;
   a.num_groups = 1ull << (n - 3 - (LOW0 ? 0 : 1));
   a.run = carry_run(0.01, n - 3, kRdmChunk);
+  a.rev = rev;
   static PerDevice grid_dev;
   const int grid = grid_dev.get([] {
     int occ = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_rdm3<LOW0>, kRdm3Threads, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_rdm3<LOW0, PERM>, kRdm3Threads, 0);
     return sm_count() * (occ > 0 ? occ : 1);
   });
   const uint64_t per = static_cast<uint64_t>(kRdm3Threads / 2) * (LOW0 ? 4 : 2);
   uint64_t g = (a.num_groups + per - 1) / per;
   if (g > static_cast<uint64_t>(grid)) g = grid;
   if (g > static_cast<uint64_t>(kPartialDoubles / 64)) g = kPartialDoubles / 64;
-  k_rdm3<LOW0><<<static_cast<unsigned>(g), kRdm3Threads, 0, st>>>(reinterpret_cast<const float4*>(psi), a, scr.partials());
+  k_rdm3<LOW0, PERM><<<static_cast<unsigned>(g), kRdm3Threads, 0, st>>>(reinterpret_cast<const float4*>(psi), a, scr.partials());
   return finalize(scr.partials(), static_cast<int>(g), 64, scr.result, st);
 }
 
@@ -647,7 +674,7 @@ template <int Q>
 static cudaError_t rdm_q(const float2* psi, int n, const uint32_t* qubits, const Scratch& scr, cudaStream_t st) {
   uint32_t s[Q];
   sort_qubits<Q>(qubits, s);
-  return s[0] == 0 ? rdm_low<Q, true>(psi, n, s, scr, st) : rdm_low<Q, false>(psi, n, s, scr, st);
+  return s[0] == 0 ? rdm_low<Q, true>(psi, n, qubits, s, scr, st) : rdm_low<Q, false>(psi, n, qubits, s, scr, st);
 }
 
 cudaError_t launch_rdm(const float2* psi, int n, int q, const uint32_t* qubits, const Scratch& scr,
@@ -659,7 +686,17 @@ cudaError_t launch_rdm(const float2* psi, int n, int q, const uint32_t* qubits, 
     case 3: {
       uint32_t s[3];
       sort_qubits<3>(qubits, s);
-      return s[0] == 0 ? rdm3_low<true>(psi, n, s, scr, st) : rdm3_low<false>(psi, n, s, scr, st);
+      uint32_t rev = 0;
+      if (n - 3 < kRdm3OrderLog) {
+        int rank[3], pair = 0;
+        for (int j = 0; j < 3; ++j) rank[j] = (qubits[j] > s[0]) + (qubits[j] > s[1]);
+        for (int b = 0; b < 4; ++b)
+          for (int a = b + 1; a < 4; ++a) rev |= static_cast<uint32_t>(member_after(3, rank, b, a)) << pair++;
+        for (int y = 0; y < 4; ++y)
+          for (int x = 0; x < 4; ++x) rev |= static_cast<uint32_t>(member_after(3, rank, y, 4 + x)) << (8 + 4 * y + x);
+      }
+      if (rev) return s[0] == 0 ? rdm3_low<true, true>(psi, n, s, rev, scr, st) : rdm3_low<false, true>(psi, n, s, rev, scr, st);
+      return s[0] == 0 ? rdm3_low<true, false>(psi, n, s, 0, scr, st) : rdm3_low<false, false>(psi, n, s, 0, scr, st);
     }
     default: return cudaErrorInvalidValue;
   }
