@@ -48,14 +48,14 @@ WORKLOAD = ("grid30: 5x6 grid, depth 20, sqrtX/sqrtY/sqrtW + CZ, amplitude dampi
 # the SHA-256 of the kernel code it was taken on, comments and blank lines left
 # out (null once the code changes).
 KNOWN_TRAFFIC = {
-    # k_apply_tile<4, 4, 8>: 4.244 GB per launch at n = 28 (dram read + write), x4 for n = 30
-    "5b97b48612739d2b": 4 * (2147519744 + 2096363776),
+    # k_multi: 4.235 GB per launch at n = 28 (dram read + write), x4 for n = 30
+    "4499e8d72652c16f": 4 * (2147680768 + 2087155200),
 }
 
 
-def kernel_source_hash() -> str:
+def kernel_source_hash(name: str) -> str:
     # code only: line comments and blank lines do not change the kernel
-    with open(os.path.join(ROOT, "paper_2111_02396_gb300", "csrc", "k_apply.cu")) as f:
+    with open(os.path.join(ROOT, "paper_2111_02396_gb300", "csrc", name)) as f:
         lines = (re.sub(r"//.*$", "", line).rstrip() for line in f)
         code = "\n".join(x for x in lines if x)
     return hashlib.sha256(code.encode()).hexdigest()[:16]
@@ -234,9 +234,9 @@ def bandwidth_probe(pkg, qs, sh):
     r = pkg.Run(f, 1, seed=0, time_kernels=True, stream=sh)
     st = r.stats()
     by_w = {}
-    for w in range(1, 8):
+    for w in range(8):
         if st["passes_by_width"][w]:
-            by_w[str(w)] = {"passes": st["passes_by_width"][w],
+            by_w[str(w) if w else "multi"] = {"passes": st["passes_by_width"][w],
                             "gbs": st["passes_by_width"][w] * (16 << 32) / (st["apply_ms_by_width"][w] / 1e3) / 1e9}
     return {"workload": "noiseless 4x8 grid (n = 32, 32 GiB complex64), depth 20, fused k = 4, one trajectory",
             "ms": st["device_ms"], "fused_passes": st["fused_passes"],
@@ -332,12 +332,14 @@ def run_ours(args):
     e2e = world * T * args.steps / e2e_s
 
     peak, peak_kind = measured_peaks()
-    # the dominant kernel: the gate width with the most fused-pass device time
-    wdom = max(range(1, 8), key=lambda w: ms_w[w])
+    # the dominant kernel: multi-gate passes (0) or the gate width with the most fused-pass device time
+    wdom = max(range(8), key=lambda w: ms_w[w])
     pass_bytes = 16 << N_QUBITS
     achieved = passes_w[wdom] * pass_bytes / (ms_w[wdom] / 1e3) / 1e9 if ms_w[wdom] > 0 else 0.0
     achieved_all = (apply_bytes / (apply_ms / 1e3)) / 1e9 if apply_ms > 0 else 0.0
-    traffic = KNOWN_TRAFFIC.get(kernel_source_hash()) if wdom == FUSE_K else None
+    traffic = KNOWN_TRAFFIC.get(kernel_source_hash("k_multi.cu" if wdom == 0 else "k_apply.cu")) if wdom in (0, FUSE_K) else None
+    kernel = ("k_multi (several fused gates per pass)" if wdom == 0 else
+              f"k_apply_tile<{wdom}> ({wdom}-qubit fused-gate apply)")
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms / args.steps, "higher_is_better": True,
@@ -349,7 +351,7 @@ def run_ours(args):
                    "flushes_per_traj": flushes / (T * args.steps),
                    "l2": "no flush: every pass streams the 8 GiB state (> 129 MB L2)",
                    "parallelism": "replicas" if world > 1 else "single GPU"},
-        "roofline": {"bound": "hbm", "kernel": f"k_apply_tile<{wdom}> ({wdom}-qubit fused-gate apply)",
+        "roofline": {"bound": "hbm" if wdom else "fp32 issue (peak and frac are HBM's)", "kernel": kernel,
                      "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "peak_kind": peak_kind,
                      "frac_of_8TBs_nominal": achieved / 8000.0,
@@ -659,8 +661,8 @@ PRECISION_WORKLOAD = ("precision: 4x8 grid (n=32) [2x13 grid (n=26) for the erro
 
 def precision_form(traj=32, traj_fp32_k6=4, oracle_traj=2, uuid=None):
     """Config 3: 6-qubit fused gates on tensor cores in split TF32 against two FP32
-    CUDA-core comparators: the same k = 6 plan (k_apply_tile6) and the same circuit
-    fused to k = 4 (k_apply_tile<4>, the plain loop's kernel).  Throughput and norm
+    CUDA-core comparators: the same k = 6 plan (csrc/k_mat64.cu) and the same circuit
+    fused to k = 4 (k_multi and k_apply_tile<4>, the plain loop's kernels).  Throughput and norm
     drift at n = 32, error against the FP64 oracle at n = 26."""
     import numpy as np
     import torch

@@ -58,7 +58,7 @@ typedef enum { QT_OP_GATE = 0, QT_OP_KRAUS = 1, QT_OP_MIXTURE = 2 } qt_op_kind;
 typedef enum { QT_DELAYED = 0, QT_EAGER = 1 } qt_mode;
 typedef enum { QT_FP32 = 0, QT_TF32X3 = 1 } qt_precision;
 #define QT_FLAG_TIME_KERNELS 1u
-#define QT_FLAG_MULTI_GATE 2u    /* group fused gates into multi-gate passes (opt-in) */
+#define QT_FLAG_MULTI_GATE 2u    /* fill multi-gate passes with later gates too (opt-in) */
 #define QT_FLAG_SHARE_PREFIX 4u  /* share the default-choice prefix between trajectories (opt-in) */
 
 #define QT_MAX_QUBITS 34      /* largest state: 2^34 complex64 = 128 GiB */
@@ -111,7 +111,9 @@ typedef struct {
   const uint64_t* z_masks;     /* num_z_masks masks (copied) */
   uint32_t keep_states;        /* 1: keep every final state on the device */
   uint32_t flags;              /* QT_FLAG_TIME_KERNELS: time each fused-gate pass;
-                                  QT_FLAG_MULTI_GATE: several fused gates per pass;
+                                  QT_FLAG_MULTI_GATE: consecutive fused gates that fit one tile
+                                  share a pass anyway (same results bit for bit); with the flag
+                                  a pass also takes later gates, past gates on other qubits;
                                   QT_FLAG_SHARE_PREFIX: delayed mode only -- stage 1 fixes, before
                                   any kernel runs, each trajectory's first channel whose draw
                                   leaves the default operator; the operators before it are the
@@ -255,7 +257,8 @@ qt_status qt_channel_lower_bounds(const qt_circuit* c, uint32_t channel, double*
 qt_status qt_state_apply(void* state, uint32_t n, uint32_t q, const uint32_t* qubits,
                          const double* U, uint32_t precision, void* stream);
 /* Reduced density block of qubits Q (q <= 3): rho[b][a] = sum_rest
- * psi[rest,b] conj(psi[rest,a]), FP64 accumulation; out host (re,im) FP64
+ * psi[rest,b] conj(psi[rest,a]), short FP32 runs summed in double-floats
+ * (two floats, ~48 bits); out host (re,im) FP64
  * 4^q complex, row-major.  P_i = tr(K_i^dag K_i rho) (Alg. 2 step 14). */
 qt_status qt_state_reduced_density(const void* state, uint32_t n, uint32_t q,
                                    const uint32_t* qubits, double* out, void* stream);
@@ -264,8 +267,10 @@ qt_status qt_state_reduced_density(const void* state, uint32_t n, uint32_t q,
  * a channel on qubits[0..q-1] (q <= 6; ops host, num_ops matrices 2^q x 2^q
  * row-major (re, im) FP64, basis bit b <-> qubits[b]) and N = <psi|psi>;
  * P and N host.  q <= 3 goes through the reduced density block; q = 4..6
- * evaluates |K_i psi|^2 per operator on the device (FP32 products, FP64
- * carry, fixed reduction order), 16, 4 or 1 operators per pass. */
+ * evaluates |K_i psi|^2 per operator on the device (FP32 products,
+ * double-float carry, fixed reduction order), 16, 4 or 1 operators per pass,
+ * or, for q <= 5 from n - q = 18 on, all operators from the reduced density
+ * block on the device. */
 qt_status qt_state_kraus_probabilities(const void* state, uint32_t n, uint32_t q, const uint32_t* qubits,
                                        uint32_t num_ops, const double* ops, double* P, double* N, void* stream);
 /* Measurement of every qubit (Sec. V.C) on a caller-owned state: S
@@ -313,7 +318,8 @@ typedef struct {
   uint32_t keep_states;        /* 1: keep final states for qt_batch_state */
   uint32_t use_graph;          /* replay the launch sequence as a CUDA graph (needs a stream) */
   uint32_t threads;            /* CTA size of trajectories whose states fit in shared memory
-                                  (n <= 14): 128, 256 or 512 (0 = 512) */
+                                  (n <= 14): 128, 256 or 512 (0 = 512), an upper bound: small
+                                  states take smaller CTAs, several per SM */
   void* stream;                /* cudaStream_t */
   uint32_t threads_global;     /* CTA size of trajectories whose states live in global memory
                                   (n > 14): 128, 256 or 512 (0 = threads) */
