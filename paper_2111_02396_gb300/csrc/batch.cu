@@ -1433,6 +1433,7 @@ static qt_status pack_batch(qt_batch* B, uint32_t num, const qt_fused* const* fu
   // a fused circuit that appears several times (e.g. many trajectories of one
   // request) is packed once; its trajectories share the tables
   std::unordered_map<const qt_fused*, uint32_t> first_use;
+  std::vector<uint32_t> widest(num, 1);               // widest fused gate of each trajectory's circuit
   for (uint32_t i = 0; i < num; ++i) {
     const qt_fused* f = fused[i];
     if (!f) return set_error(QT_ERR_INVALID_ARG, "%s: fused %u is NULL", who, i);
@@ -1446,6 +1447,7 @@ static qt_status pack_batch(qt_batch* B, uint32_t num, const qt_fused* const* fu
       T.gf0 = static_cast<uint32_t>(B->total_gates);
       B->total_gates += T.ngates;
       B->gate_ops += f->gate_ops;
+      widest[i] = widest[seen->second];
       continue;
     }
     first_use.emplace(f, i);
@@ -1506,6 +1508,7 @@ static qt_status pack_batch(qt_batch* B, uint32_t num, const qt_fused* const* fu
                          bt::kMaxW, i);
       bt::Gate g{};
       g.w = static_cast<uint8_t>(fg.targets.size());
+      widest[i] = std::max<uint32_t>(widest[i], g.w);
       for (size_t b = 0; b < fg.targets.size(); ++b) g.t[b] = static_cast<uint8_t>(fg.targets[b]);
       g.mat = static_cast<uint32_t>(fmat.size());
       for (const cd& x : fg.def) fmat.push_back(make_float2(static_cast<float>(x.real()), static_cast<float>(x.imag())));
@@ -1551,20 +1554,14 @@ static qt_status pack_batch(qt_batch* B, uint32_t num, const qt_fused* const* fu
   std::stable_sort(B->order.begin(), B->order.end(),
                    [&](uint32_t a, uint32_t b) { return B->traj[a].n > B->traj[b].n; });
   uint64_t soff = 0;
-  std::unordered_map<uint32_t, uint32_t> widest;      // widest fused gate of the circuit whose gates start here
   for (uint32_t i = 0; i < num; ++i) {
     bt::Traj& T = B->traj[i];
-    if (!widest.count(T.gate0)) {
-      uint32_t w = 1;
-      for (uint32_t g = 0; g < T.ngates; ++g) w = std::max<uint32_t>(w, gates[T.gate0 + g].w);
-      widest[T.gate0] = w;
-    }
     T.arena_off = B->total_amps;
     B->total_amps += 1ull << T.n;
     const int cls = bt::class_of(T.n);
     B->count[cls]++;
     B->top_n[cls] = std::max(B->top_n[cls], T.n);
-    B->wmat[cls] = std::max(B->wmat[cls], widest[T.gate0]);
+    B->wmat[cls] = std::max(B->wmat[cls], widest[i]);
     T.seed = per ? per[i].seed : 0;
     T.tid = per ? per[i].traj : 0;
     T.S = per ? per[i].S : 0;

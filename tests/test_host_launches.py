@@ -1,0 +1,67 @@
+"""Host code around the launches, on the CPU: libqt.so on a CUDA runtime that records kernels
+instead of running them (fake_cudart.cpp, preloaded into a child process)."""
+import os
+import subprocess
+import sys
+import textwrap
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+CUDA = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+
+PRELUDE = """
+import ctypes, os
+import numpy as np
+import paper_2111_02396_gb300 as qt
+import qtsynth as qs
+from paper_2111_02396_gb300.qt import QtError
+fake = ctypes.CDLL(os.environ["LD_PRELOAD"])
+fake.fake_launches.restype = ctypes.c_char_p
+fake.fake_set.argtypes = [ctypes.c_char_p, ctypes.c_size_t]
+qt.load()
+
+def launches(part=""):
+    rows = [x.split() for x in fake.fake_launches().decode().splitlines()]
+    return [(name, int(g), int(b), int(s)) for name, g, b, s in rows if part in name]
+"""
+
+
+@pytest.fixture(scope="module")
+def child(tmp_path_factory):
+    from paper_2111_02396_gb300 import build
+    build.build()
+    so = str(tmp_path_factory.mktemp("fake") / "libfake_cudart.so")
+    subprocess.run(["g++", "-shared", "-fPIC", "-O1", "-std=c++17", "-I", os.path.join(CUDA, "include"),
+                    os.path.join(HERE, "fake_cudart.cpp"), "-o", so], check=True)
+
+    def run(code):
+        env = dict(os.environ, LD_PRELOAD=so, PYTHONPATH=ROOT)
+        r = subprocess.run([sys.executable, "-c", PRELUDE + textwrap.dedent(code)], env=env, cwd=ROOT,
+                           capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0, r.stdout + r.stderr
+
+    return run
+
+
+@pytest.mark.parametrize("k", [3, 4, 6])
+@pytest.mark.parametrize("n", [9, 14])
+def test_batch_shared_memory_with_empty_circuits(child, k, n):
+    """The matrix buffers of a class are sized for its widest gate: an empty circuit, which has the
+    same first gate as the circuit packed after it, takes nothing from them."""
+    child(f"""
+    n, k = {n}, {k}
+    real = [qt.Fused(qt.Circuit.from_synth(qs.chain_circuit(n, 8, s, dep1=1e-2)), k) for s in (1, 2)]
+    empty = [qt.Fused(qt.Circuit.from_synth(qs.Circuit(m)), k) for m in (n, 2, 20)]
+    w = max(len(f.gate(g)["targets"]) for f in real for g in range(f.info()["num_fused"]))
+    assert w == k
+    narrow = min(w, 4)
+    need = 8 * ((1 << n) + (2 << 2 * narrow) + ((1 << 2 * w) if w > 4 else 0))
+    cls = "k_batch_smemILi512E" if n == 14 else "k_batch_smemILi128E"
+    for batch in (real, [empty[0]] + real, [empty[1], real[0], empty[0], real[1], real[0]], empty + real + empty):
+        fake.fake_clear()
+        qt.Batch(batch).run(seed=1)
+        got = [x[3] for x in launches(cls)]
+        assert got == [need], (batch, got, need)
+    """)
