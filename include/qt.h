@@ -268,9 +268,10 @@ qt_status qt_state_reduced_density(const void* state, uint32_t n, uint32_t q,
  * row-major (re, im) FP64, basis bit b <-> qubits[b]) and N = <psi|psi>;
  * P and N host.  q <= 3 goes through the reduced density block; q = 4..6
  * evaluates |K_i psi|^2 per operator on the device (FP32 products,
- * double-float carry, fixed reduction order), 16, 4 or 1 operators per pass,
- * or, for q <= 5 from n - q = 18 on, all operators from the reduced density
- * block on the device. */
+ * double-float carry, fixed reduction order), 16, 4 or 1 operators per pass;
+ * for q <= 5 from n - q = 18 on, one pass over the state gives every operator
+ * from the reduced density block, and only those whose terms cancel there (a
+ * state near the kernel of K_i) are evaluated as |K_i psi|^2. */
 qt_status qt_state_kraus_probabilities(const void* state, uint32_t n, uint32_t q, const uint32_t* qubits,
                                        uint32_t num_ops, const double* ops, double* P, double* N, void* stream);
 /* Measurement of every qubit (Sec. V.C) on a caller-owned state: S

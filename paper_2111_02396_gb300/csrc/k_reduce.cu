@@ -463,11 +463,10 @@ static cudaError_t rdm3_low(const float2* psi, int n, const uint32_t* s, uint32_
 // loads are in flight while this one is multiplied.  Member m of a set sits
 // at m + m / 16 of a row of odd pitch: the blocks a warp reads together then
 // fall into different banks.  FP32 runs are carried in double-floats held in
-// shared memory, which leaves 128 registers a thread, two CTAs an SM.  A
-// run's length grows with the number of sets, for the reason given at
-// carry_run; a wide channel's probabilities average the error of 4^q entries,
-// so its runs may be longer.
-// n = 25, q = 4 / 5: 138 / 158 us; the products K_i v that gave these
+// shared memory, which leaves 128 registers a thread, two CTAs an SM.  A run
+// is 12 sets, the longest for which probabilities from the block are no
+// further off than sums of |K_i v|^2 (rule at k_kraus_trace).
+// n = 25, q = 4 / 5: 151 / 184 us (138 / 158 with runs of 30); the products K_i v that gave these
 // channels' probabilities before took 2719 / 1584 us for each 16 / 4 operators.
 // ---------------------------------------------------------------------------
 template <int Q>
@@ -492,8 +491,9 @@ struct GramArgs {
   uint32_t cset[8], cmem[8];  // what chunk c adds to the thread's set and member
   uint32_t ins[Q + 1];        // ascending bit positions to insert zeros at
   uint64_t num_tiles;
-  int run;                    // sets summed in FP32 before the carry
 };
+
+constexpr int kGramRun = 12;  // sets summed in FP32 before the carry
 
 // bi, bj (bj <= bi) of tile r of the lower triangle
 __device__ __forceinline__ void gram_tile(int r, int& bi, int& bj) {
@@ -582,7 +582,7 @@ __global__ void __launch_bounds__(Gram<Q>::THREADS, 2) k_gram(const float2* __re
             f[4 * p + q] = fmaf(x[p].x, y[q].x, fmaf(x[p].y, y[q].y, f[4 * p + q]));
             f[16 + 4 * p + q] = fmaf(x[p].y, y[q].x, fmaf(-x[p].x, y[q].y, f[16 + 4 * p + q]));
           }
-        if (++run == a.run) { flush(); run = 0; }
+        if (++run == kGramRun) { flush(); run = 0; }
       }
     }
     __syncthreads();                                     // the tile is read: its buffer is free
@@ -642,7 +642,6 @@ static cudaError_t gram_low(const float2* psi, int n, const uint32_t* s, float2*
     a.coff[c] = x | a.offs[a.cmem[c]];
   }
   a.num_tiles = 1ull << (n - 12);                        // n - Q >= kGramMinLog: whole tiles
-  a.run = carry_run(0.03, n - Q, 32);
   static PerDevice setup;
   const int grid = setup.get([] {
     if (cudaFuncSetAttribute(k_gram<Q, LOW0>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(G::SMEM)) !=
@@ -750,11 +749,22 @@ void rdm_unpack(int q, const uint32_t* qubits, const double* r, double* rho) {
 // contraction (2^(3q) products per operator) is far below the pass but wants
 // more than FP32; FP64 is slow here, so rho enters as double-floats and the
 // products keep their FMA error term.  The operators are complex64.
-// From 2^18 gather sets on (kGramMinLog): there the FP32 rounding of either
-// form has averaged out and they agree to 7e-10 over 60 inputs each (q = 4,
-// 5).  Below, and for q = 6, whose rows of 128 FP32 terms leave a mean of
-// -6e-10 in k_kraus_norms at any size (the two then differ by up to 1.3e-9),
-// k_kraus_norms stays: a call's result is not to move by 1e-9.
+//
+// The rounding of rho's entries, independent of one another, moves P_i by about
+// 1.5e-7 E_i, E_i^2 = sum_ab |(K_i^dag K_i)_ab|^2 rho_aa rho_bb, and where the
+// terms of P_i cancel (a state near the kernel of K_i) that is all there is: a
+// true 1e-6 N comes out 10 % off, a true 0 negative.  |K_i v|^2 keeps its
+// relative accuracy, 1.5e-7 of P_i.  So an operator with E_i > P_i is left to
+// k_kraus_norms by the caller.  Relative errors with E_i <= P_i, runs of 12
+// sets, all sets alike (nothing averages out), 4-qubit operators, rms here /
+// of |K_i v|^2: E_i in (0.8, 1] P_i dense 1.2e-7 / 1.6e-7, a single entry 1.2e-7 /
+// 1.3e-7; in (1, 2] P_i, left out, 1.6e-7..1.9e-7 / 1.7e-7; runs of 16 sets, a
+// single entry 1.7e-7.  A maximally mixed rho has E_i <= P_i for every K_i.
+//
+// From 2^18 gather sets on (kGramMinLog), where on states whose sets differ
+// the FP32 rounding of both forms averages out below 1e-9.  For q = 6 the
+// rows of 128 FP32 terms of k_norms64 leave a mean of -6e-10 at any size, which
+// the two forms would then differ by; it has no such pass.
 // ---------------------------------------------------------------------------
 // acc += x y, x a double-float
 __device__ __forceinline__ void df_mul_acc(float2& acc, float xh, float xl, float y) {
@@ -765,12 +775,39 @@ __device__ __forceinline__ void df_mul_acc(float2& acc, float xh, float xl, floa
 }
 
 // block (x, i): 256 of the terms (eight b, entry a, row j) of operator i,
-// Re(k_ja sum_b rho[a][b] conj(k_jb)), summed into out[i * gridDim.x + x]
+// Re(k_ja sum_b rho[a][b] conj(k_jb)), summed into out[i * gridDim.x + x]; the
+// last block of an operator puts E_i there
 template <int Q>
 __global__ void __launch_bounds__(256) k_kraus_trace(const float4* rho, const float2* __restrict__ ops, double* out) {
   constexpr int D = 1 << Q;
   __shared__ float2 s_sum[8];
   cudaGridDependencySynchronize();
+  if (blockIdx.x == gridDim.x - 1) {
+    __shared__ double s_part[8];
+    const float2* const K = ops + static_cast<size_t>(blockIdx.y) * D * D;
+    double s = 0.0;                                        // products of four factors would leave FP32's range
+    for (int e = threadIdx.x; e < D * D; e += 256) {
+      const int x = e % D, y = e / D;
+      float gr = 0.f, gi = 0.f;
+#pragma unroll 8
+      for (int r = 0; r < D; ++r) {
+        const float2 u = __ldg(K + r * D + x), v = __ldg(K + r * D + y);
+        gr = fmaf(u.x, v.x, fmaf(u.y, v.y, gr));
+        gi = fmaf(u.x, v.y, fmaf(-u.y, v.x, gi));
+      }
+      const double g = gr, h = gi;
+      s += (g * g + h * h) * (static_cast<double>(rho[x * (D + 1)].x) * static_cast<double>(rho[y * (D + 1)].x));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int w = 1; w < 8; ++w) s += s_part[w];
+      out[blockIdx.y * gridDim.x + blockIdx.x] = sqrt(s);
+    }
+    return;
+  }
   const int idx = blockIdx.x * 256 + threadIdx.x, a = idx % D, j = (idx / D) % D, b0 = idx / (D * D) * 8;
   const float2* const k = ops + (static_cast<size_t>(blockIdx.y) * D + j) * D;
   float2 tr = make_float2(0.f, 0.f), ti = make_float2(0.f, 0.f);
@@ -799,7 +836,7 @@ __global__ void __launch_bounds__(256) k_kraus_trace(const float4* rho, const fl
   }
 }
 
-int kraus_slices(int q) { return (1 << (3 * q - 3)) / 256; }
+int kraus_slices(int q) { return (1 << (3 * q - 3)) / 256 + 1; }
 
 // the result rows, padded so that the operators after them are 16-byte aligned
 size_t kraus_results(int q, int nops) { return (static_cast<size_t>(nops) * kraus_slices(q) + 1) & ~size_t(1); }

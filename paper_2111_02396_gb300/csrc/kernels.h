@@ -75,8 +75,9 @@ cudaError_t launch_rdm(const float2* psi, int n, int q, const uint32_t* qubits, 
 // Channels on 4 or 5 qubits, at least 2^kGramMinLog gather sets: P_i =
 // <psi|K_i^dag K_i|psi> of nops operators.  scratch (kraus_scratch_bytes(q,
 // nops) bytes of device memory, 16-byte aligned) begins with the results,
-// nops x kraus_slices(q) doubles, P_i the sum of row i; from kraus_results(q,
-// nops) doubles on come the operators as kraus_sort_columns writes them (K
+// nops x kraus_slices(q) doubles: row i ends with E_i, and the others sum to
+// P_i, which is only good if E_i <= P_i (see k_kraus_trace).  From
+// kraus_results(q, nops) doubles on come the operators as kraus_sort_columns writes them (K
 // row-major (re, im) FP64, basis bit b <-> qubits[b]; 4^q complex64 each)
 constexpr int kGramMinLog = 18;
 inline bool kraus_by_gram(int n, int q) { return q <= 5 && n - q >= kGramMinLog; }
@@ -86,7 +87,7 @@ size_t kraus_scratch_bytes(int q, int nops);
 void kraus_sort_columns(int q, const uint32_t* qubits, const double* K, float2* out);
 cudaError_t launch_kraus_probs(const float2* psi, int n, int q, const uint32_t* qubits, int nops, void* scratch,
                                cudaStream_t st);
-// The other channels on 4..6 qubits: N and P_i = |K_i psi|^2 for kraus_group(q)
+// The other channels on 4..6 qubits, and operators that the above leaves: N and P_i = |K_i psi|^2 for kraus_group(q)
 // operators (16, 4, 1 for q = 4, 5, 6; pad with zero matrices) into
 // scr.result[0] (N) and scr.result[1..]; ops_dev: the operators, 2^q x 2^q
 // row-major complex64 in device memory, basis bit b <-> qubits[b]

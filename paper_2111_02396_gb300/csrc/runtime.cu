@@ -121,44 +121,66 @@ struct ScratchBufs {
 };
 
 // Probability pass of a channel on 4..6 qubits; keeps its buffers for the
-// next call.  Blocks until P and N are on the host.
+// next call.  Blocks until P and N are on the host.  Channels on 4 and 5 qubits
+// of large states take one pass for all operators (kraus_by_gram), and then
+// |K_i psi|^2 of those whose terms cancel in it.
 struct WideChannel {
   DevBuf buf;
   std::vector<float2> ops;
   std::vector<double> rows;
+  std::vector<uint32_t> todo;                    // operators for the direct form
   uint64_t h2d = 0, d2h = 0, launches = 0;       // of the last call
   qt_status run(const float2* psi, uint32_t n, uint32_t q, const uint32_t* qubits, uint32_t num_ops, const double* K,
                 double* P, double* N, cudaStream_t st) {
-    const int Q = static_cast<int>(q), D = 1 << Q;
-    const size_t mat = static_cast<size_t>(D) * D;
     h2d = d2h = launches = 0;
-    if (kraus_by_gram(static_cast<int>(n), Q)) {
-      // every operator in one pass, an identity after them (its P is N)
-      const int nops = static_cast<int>(num_ops) + 1, slices = kraus_slices(Q);
-      const size_t nres = static_cast<size_t>(nops) * slices, need = kraus_scratch_bytes(Q, nops);
-      if (buf.bytes < need && !buf.alloc(need, st)) return set_error(QT_ERR_OUT_OF_MEMORY, "Kraus operator buffer");
-      ops.assign(mat * nops, make_float2(0.f, 0.f));
-      for (uint32_t i = 0; i < num_ops; ++i) kraus_sort_columns(Q, qubits, K + 2 * mat * i, ops.data() + mat * i);
-      for (int j = 0; j < D; ++j) ops[mat * num_ops + static_cast<size_t>(j) * (D + 1)].x = 1.f;
-      rows.resize(nres);
-      double* const res = buf.as<double>();
-      h2d = sizeof(float2) * ops.size();
-      d2h = sizeof(double) * nres;
-      launches = 3;
-      QT_CUDA(cudaMemcpyAsync(res + kraus_results(Q, nops), ops.data(), h2d, cudaMemcpyHostToDevice, st),
-              "cudaMemcpyAsync(Kraus operators)");
-      QT_CUDA(launch_kraus_probs(psi, static_cast<int>(n), Q, qubits, nops, res, st), "Kraus probability kernel launch");
-      QT_CUDA(cudaMemcpyAsync(rows.data(), res, d2h, cudaMemcpyDeviceToHost, st), "cudaMemcpyAsync(probabilities)");
-      QT_CUDA(cudaStreamSynchronize(st), "cudaStreamSynchronize(probabilities)");
-      for (int i = 0; i < nops; ++i) {
-        double s = 0.0;
-        for (int k = 0; k < slices; ++k) s += rows[static_cast<size_t>(i) * slices + k];
-        (i < static_cast<int>(num_ops) ? P[i] : *N) = s;
-      }
-      return QT_OK;
+    todo.clear();
+    if (kraus_by_gram(static_cast<int>(n), static_cast<int>(q))) {
+      const qt_status s = gram(psi, n, q, qubits, num_ops, K, P, N, st);
+      if (s != QT_OK || todo.empty()) return s;
+      double n2 = 0.0;
+      return direct(psi, n, q, qubits, K, P, &n2, st);
     }
-    // kraus_group(q) operators per pass, zero matrices padding the last group
-    const uint32_t G = static_cast<uint32_t>(kraus_group(Q));
+    for (uint32_t i = 0; i < num_ops; ++i) todo.push_back(i);
+    return direct(psi, n, q, qubits, K, P, N, st);
+  }
+
+ private:
+  // every operator in one pass, an identity after them (its P is N)
+  qt_status gram(const float2* psi, uint32_t n, uint32_t q, const uint32_t* qubits, uint32_t num_ops, const double* K,
+                 double* P, double* N, cudaStream_t st) {
+    const int Q = static_cast<int>(q), D = 1 << Q, nops = static_cast<int>(num_ops) + 1, slices = kraus_slices(Q);
+    const size_t mat = static_cast<size_t>(D) * D, nres = static_cast<size_t>(nops) * slices,
+                 need = kraus_scratch_bytes(Q, nops);
+    if (buf.bytes < need && !buf.alloc(need, st)) return set_error(QT_ERR_OUT_OF_MEMORY, "Kraus operator buffer");
+    ops.assign(mat * nops, make_float2(0.f, 0.f));
+    for (uint32_t i = 0; i < num_ops; ++i) kraus_sort_columns(Q, qubits, K + 2 * mat * i, ops.data() + mat * i);
+    for (int j = 0; j < D; ++j) ops[mat * num_ops + static_cast<size_t>(j) * (D + 1)].x = 1.f;
+    rows.resize(nres);
+    double* const res = buf.as<double>();
+    h2d = sizeof(float2) * ops.size();
+    d2h = sizeof(double) * nres;
+    launches = 3;
+    QT_CUDA(cudaMemcpyAsync(res + kraus_results(Q, nops), ops.data(), h2d, cudaMemcpyHostToDevice, st),
+            "cudaMemcpyAsync(Kraus operators)");
+    QT_CUDA(launch_kraus_probs(psi, static_cast<int>(n), Q, qubits, nops, res, st), "Kraus probability kernel launch");
+    QT_CUDA(cudaMemcpyAsync(rows.data(), res, d2h, cudaMemcpyDeviceToHost, st), "cudaMemcpyAsync(probabilities)");
+    QT_CUDA(cudaStreamSynchronize(st), "cudaStreamSynchronize(probabilities)");
+    for (int i = 0; i < nops; ++i) {
+      const double* const r = rows.data() + static_cast<size_t>(i) * slices;
+      double s = 0.0;
+      for (int k = 0; k + 1 < slices; ++k) s += r[k];
+      if (i == static_cast<int>(num_ops)) *N = s;
+      else if (r[slices - 1] <= s) P[i] = s;
+      else todo.push_back(static_cast<uint32_t>(i));      // its terms cancel (or are NaN)
+    }
+    return QT_OK;
+  }
+
+  // the operators of todo, kraus_group(q) per pass, zero matrices padding the last group
+  qt_status direct(const float2* psi, uint32_t n, uint32_t q, const uint32_t* qubits, const double* K, double* P,
+                   double* N, cudaStream_t st) {
+    const int Q = static_cast<int>(q);
+    const size_t G = static_cast<size_t>(kraus_group(Q)), mat = size_t{1} << (2 * Q);
     const size_t scr_doubles = kPartialDoubles + kResultDoubles;
     const size_t need = sizeof(double) * scr_doubles + sizeof(float2) * G * mat;
     if (buf.bytes < need && !buf.alloc(need, st)) return set_error(QT_ERR_OUT_OF_MEMORY, "Kraus operator buffer");
@@ -167,10 +189,11 @@ struct WideChannel {
     scr.result = scr.partial + kPartialDoubles;
     float2* const kd = reinterpret_cast<float2*>(scr.partial + scr_doubles);
     rows.resize(G + 1);
-    for (uint32_t g0 = 0; g0 < num_ops; g0 += G) {
+    for (size_t g0 = 0; g0 < todo.size(); g0 += G) {
+      const size_t cnt = std::min(G, todo.size() - g0);
       ops.assign(G * mat, make_float2(0.f, 0.f));
-      for (uint32_t j = 0; j < G && g0 + j < num_ops; ++j) {
-        const double* k = K + 2 * mat * (g0 + j);
+      for (size_t j = 0; j < cnt; ++j) {
+        const double* k = K + 2 * mat * todo[g0 + j];
         for (size_t e = 0; e < mat; ++e)
           ops[j * mat + e] = make_float2(static_cast<float>(k[2 * e]), static_cast<float>(k[2 * e + 1]));
       }
@@ -185,7 +208,7 @@ struct WideChannel {
       d2h += sizeof(double) * (G + 1);
       launches += 2;
       *N = rows[0];
-      for (uint32_t j = 0; j < G && g0 + j < num_ops; ++j) P[g0 + j] = rows[1 + j];
+      for (size_t j = 0; j < cnt; ++j) P[todo[g0 + j]] = rows[1 + j];
     }
     return QT_OK;
   }
@@ -651,8 +674,7 @@ struct Controller {
     return QT_OK;
   }
 
-  // Channels on 4..6 qubits: the probabilities from the reduced density block,
-  // contracted with the operators on the device
+  // Channels on 4..6 qubits
   WideChannel wide;
   qt_status kraus_probabilities(const float2* psi, const Op& op, double& N, double* P) {
     TraceRange tr("qt probability pass (wide channel)");
