@@ -1700,7 +1700,9 @@ static cudaError_t launch_glob_class(uint32_t threads, const bt::Dev& d, uint32_
   cfg.stream = s;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, bt::k_batch_glob, d);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, bt::k_batch_glob, d);
+  if (e != cudaSuccess) cudaGetLastError();          // not for the calls that come after
+  return e;
 }
 
 // One run's persistent launches, with tables, outputs and arena as d holds

@@ -20,9 +20,12 @@ namespace qt {
 // A dependent launch: its blocks may become resident while the kernel before
 // it on the stream still runs, and wait there (cudaGridDependencySynchronize)
 // for that kernel's results.  The short kernels that follow a reduction start
-// without a launch gap this way.
+// without a launch gap this way.  An error of that kernel's launch is returned
+// instead; no error stays behind for the calls that come after.
 template <typename... P, typename... A>
 static cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, unsigned block, cudaStream_t st, A... args) {
+  const cudaError_t before = cudaGetLastError();
+  if (before != cudaSuccess) return before;
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
@@ -32,7 +35,9 @@ static cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, unsigned bloc
   cfg.stream = st;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
 }
 
 // ---------------------------------------------------------------------------

@@ -65,3 +65,47 @@ def test_batch_shared_memory_with_empty_circuits(child, k, n):
         got = [x[3] for x in launches(cls)]
         assert got == [need], (batch, got, need)
     """)
+
+
+@pytest.mark.parametrize("kernel,call", [
+    ("k_rdmILi1", "qt.qt_state_reduced_density(p, 12, [3])"),
+    ("k_rdmILi2", "qt.qt_state_reduced_density(p, 12, [0, 3])"),
+    ("k_rdm3", "qt.qt_state_reduced_density(p, 12, [5, 0, 3])"),
+    ("k_rdmILi2", "qt.qt_state_kraus_probabilities(p, 12, [7, 3], K(2))"),
+    ("k_kraus_normsILi4", "qt.qt_state_kraus_probabilities(p, 12, [7, 3, 1, 2], K(4))"),
+    ("k_norms64", "qt.qt_state_kraus_probabilities(p, 12, [7, 3, 1, 2, 4, 5], K(6))"),
+    ("k_gramILi4", "qt.qt_state_kraus_probabilities(p, 22, [7, 3, 1, 2], K(4))"),
+    ("k_gram_matrix", "qt.qt_state_kraus_probabilities(p, 23, [7, 3, 1, 2, 4], K(5))"),
+    ("k_kraus_trace", "qt.qt_state_kraus_probabilities(p, 22, [7, 3, 1, 2], K(4))"),
+    ("k_expect", "qt.qt_state_expect_z(p, 8, [1, 3])"),
+    ("k_expect_wht", "qt.qt_state_expect_z(p, 12, [1, 3])"),
+    ("k_finalize", "qt.qt_state_expect_z(p, 12, [1, 3])"),
+    ("k_cdf_sub", "qt.qt_state_sample(p, 12, 1, 0, 10)"),
+    ("k_cdf_blk", "qt.qt_state_sample(p, 12, 1, 0, 10)"),
+    ("k_cdf_scan", "qt.qt_state_sample(p, 12, 1, 0, 10)"),
+    ("k_sample", "qt.qt_state_sample(p, 12, 1, 0, 10)"),
+    ("k_apply", "qt.qt_state_apply(p, 12, [3, 1], np.eye(4))"),
+    ("k_batch_glob", "batch.run(seed=1)"),
+    ("k_batch_smem", "batch.run(seed=1)"),
+])
+def test_failed_launch_is_reported(child, kernel, call):
+    """A launch that the runtime refuses ends the call with an error, also where a dependent launch
+    follows it, and leaves nothing behind for the next call."""
+    child(f"""
+    K = lambda q: np.eye(1 << q)[None]
+    buf = np.zeros(1 << 16, np.complex64)
+    p = (buf.ctypes.data + 255) & ~255
+    batch = qt.Batch([qt.Fused(qt.Circuit.from_synth(qs.chain_circuit(n, 4, 1, dep1=1e-2)), 3) for n in (9, 16)])
+    call = lambda: {call}
+    call()
+    assert launches("{kernel}")
+    fake.fake_fail(b"{kernel}")
+    try:
+        call()
+    except QtError as e:
+        assert e.status == qt.qt.QT_ERR_CUDA
+    else:
+        raise AssertionError("the call returned a result")
+    fake.fake_fail(b"")
+    call()
+    """)
