@@ -105,14 +105,17 @@ struct ScratchBufs {
   DevBuf buf;
   Scratch s;
   double* extra = nullptr;                 // `more` doubles for the caller
+  static constexpr int kFlagDoubles = 8;
+  int* flag = nullptr;                     // a run's error flag, that many doubles before the results
   bool alloc(int n, cudaStream_t st, size_t more = 0) {
     auto up = [](size_t b) { return (b + 255) & ~static_cast<size_t>(255); };
-    const size_t part = up(sizeof(double) * kPartialDoubles), res = up(sizeof(double) * kResultDoubles),
+    const size_t part = up(sizeof(double) * kPartialDoubles), res = up(sizeof(double) * (kFlagDoubles + kResultDoubles)),
                  cum = up(sizeof(double) * cdf_num_blk(n)), sub = up(sizeof(float) * cdf_num_sub(n));
     if (!buf.alloc(part + res + cum + sub + sizeof(double) * more, st)) return false;
     char* const p = buf.as<char>();
     s.partial = reinterpret_cast<double*>(p);
-    s.result = reinterpret_cast<double*>(p + part);
+    flag = reinterpret_cast<int*>(p + part);
+    s.result = reinterpret_cast<double*>(p + part) + kFlagDoubles;
     s.cdf_cum = reinterpret_cast<double*>(p + part + res);
     s.cdf_sub = reinterpret_cast<float*>(p + part + res + cum);
     extra = reinterpret_cast<double*>(p + part + res + cum + sub);
@@ -282,11 +285,16 @@ struct Controller {
   }
   ~Controller() {
     if (pinned) cudaFreeHost(pinned);
+    if (err_host) {
+      cudaStreamSynchronize(R.st);          // a copy into it may be in flight on an error return
+      cudaFreeHost(err_host);
+    }
+    if (err_ev) cudaEventDestroy(err_ev);
     for (auto e : ev) cudaEventDestroy(e);
   }
 
   // tensor-core path buffers (split-TF32, widths 4..6)
-  DevBuf wbuf, errbuf;
+  DevBuf wbuf;
   std::vector<float> wtmp;
 
   // QT_TF32X3 sends 5- and 6-qubit pieces to the tensor cores; narrower
@@ -300,9 +308,9 @@ struct Controller {
     if (use_tc(k)) {
       if (!wbuf.p && !wbuf.alloc(sizeof(float) * 128 * 128, R.st))
         return set_error(QT_ERR_OUT_OF_MEMORY, "tensor-core matrix buffer");
-      if (!errbuf.p) {                      // device error flag of the tensor-core kernel, cleared once
-        if (!errbuf.alloc(sizeof(int), R.st)) return set_error(QT_ERR_OUT_OF_MEMORY, "error flag");
-        QT_CUDA(cudaMemsetAsync(errbuf.p, 0, sizeof(int), R.st), "cudaMemsetAsync");
+      if (!tc_used) {                       // device error flag of the tensor-core kernel, cleared once
+        QT_CUDA(cudaMemsetAsync(R.scr.flag, 0, sizeof(int), R.st), "cudaMemsetAsync");
+        tc_used = true;
       }
       const int N = 2 << k;
       wtmp.resize(static_cast<size_t>(N) * N);
@@ -310,7 +318,7 @@ struct Controller {
       QT_CUDA(cudaMemcpyAsync(wbuf.p, wtmp.data(), sizeof(float) * N * N, cudaMemcpyHostToDevice, R.st),
               "cudaMemcpyAsync(W)");
       R.stats.h2d_bytes += sizeof(float) * N * N;
-      QT_CUDA(launch_apply_tc(psi, static_cast<int>(R.n), k, targets.data(), wbuf.as<float>(), errbuf.as<int>(), R.st),
+      QT_CUDA(launch_apply_tc(psi, static_cast<int>(R.n), k, targets.data(), wbuf.as<float>(), R.scr.flag, R.st),
               "tensor-core apply kernel launch");
       return QT_OK;
     }
@@ -330,12 +338,40 @@ struct Controller {
     return QT_OK;
   }
 
+  // The error flag comes back with the results of every stage-2 read (whose
+  // choice would rest on a wrong state), and behind every fourth trajectory,
+  // where the host looks at the copy four trajectories later and so keeps
+  // planning ahead (16 of 17 qubits: 21.1 ms without, 21.9 with a look behind
+  // each).  Once the flag is set, waits give up at their first try.
+  static constexpr uint32_t kErrEvery = 4;
+  uint32_t finished = 0;                    // trajectories
+  bool tc_used = false;
+  int* err_host = nullptr;
+  cudaEvent_t err_ev = nullptr;             // recorded behind the last copy into err_host
+
+  qt_status device_error(int e) const {
+    if (tc_used && e) return set_error(QT_ERR_TIMEOUT, "tensor-core kernel: a bounded wait ran out (code %d)", e);
+    return QT_OK;
+  }
   qt_status check_device_error() {
-    if (!errbuf.p) return QT_OK;
+    if (!tc_used) return QT_OK;
     int e = 0;
-    QT_CUDA(cudaMemcpyAsync(&e, errbuf.p, sizeof(int), cudaMemcpyDeviceToHost, R.st), "cudaMemcpyAsync(err)");
+    QT_CUDA(cudaMemcpyAsync(&e, R.scr.flag, sizeof(int), cudaMemcpyDeviceToHost, R.st), "cudaMemcpyAsync(err)");
     QT_CUDA(cudaStreamSynchronize(R.st), "cudaStreamSynchronize(err)");
-    if (e) return set_error(QT_ERR_TIMEOUT, "tensor-core kernel: a bounded wait ran out (code %d)", e);
+    return device_error(e);
+  }
+  qt_status pass_device_error() {           // behind a trajectory
+    if (!tc_used || ++finished % kErrEvery) return QT_OK;
+    if (err_host) {
+      QT_CUDA(cudaEventSynchronize(err_ev), "cudaEventSynchronize(err)");
+      const qt_status s = device_error(*err_host);
+      if (s != QT_OK) return s;
+    } else {
+      QT_CUDA(cudaEventCreateWithFlags(&err_ev, cudaEventDisableTiming), "cudaEventCreate");
+      QT_CUDA(cudaMallocHost(&err_host, sizeof(int)), "cudaMallocHost");
+    }
+    QT_CUDA(cudaMemcpyAsync(err_host, R.scr.flag, sizeof(int), cudaMemcpyDeviceToHost, R.st), "cudaMemcpyAsync(err)");
+    QT_CUDA(cudaEventRecord(err_ev, R.st), "cudaEventRecord(err)");
     return QT_OK;
   }
 
@@ -678,8 +714,9 @@ struct Controller {
   WideChannel wide;
   qt_status kraus_probabilities(const float2* psi, const Op& op, double& N, double* P) {
     TraceRange tr("qt probability pass (wide channel)");
-    const qt_status s = wide.run(psi, R.n, op.q, op.qubits, op.num_ops, reinterpret_cast<const double*>(op.kraus.data()),
-                                 P, &N, R.st);
+    qt_status s = wide.run(psi, R.n, op.q, op.qubits, op.num_ops, reinterpret_cast<const double*>(op.kraus.data()),
+                           P, &N, R.st);
+    if (s == QT_OK) s = check_device_error();
     if (s != QT_OK) return s;
     R.stats.h2d_bytes += wide.h2d;
     R.stats.d2h_bytes += wide.d2h;
@@ -700,15 +737,20 @@ struct Controller {
             "probability kernel launch");
     const int W = 1 << (2 * op.q);
     if (!pinned) QT_CUDA(cudaMallocHost(&pinned, sizeof(double) * 128), "cudaMallocHost");
-    QT_CUDA(cudaMemcpyAsync(pinned, R.scr.s.result, sizeof(double) * W, cudaMemcpyDeviceToHost, R.st),
+    constexpr int F = ScratchBufs::kFlagDoubles;
+    QT_CUDA(cudaMemcpyAsync(pinned, R.scr.flag, sizeof(double) * (F + W), cudaMemcpyDeviceToHost, R.st),
             "cudaMemcpyAsync(probabilities)");
     QT_CUDA(cudaStreamSynchronize(R.st), "cudaStreamSynchronize(probabilities)");
     R.stats.prob_passes++;
     R.stats.kernel_launches += 2;
-    R.stats.d2h_bytes += sizeof(double) * W;
+    R.stats.d2h_bytes += sizeof(double) * (F + W);
+    int e;
+    std::memcpy(&e, pinned, sizeof(e));
+    const qt_status es = device_error(e);
+    if (es != QT_OK) return es;
     const int D = static_cast<int>(op.dim());
     double rho[2 * 64];
-    rdm_unpack(static_cast<int>(op.q), op.qubits, pinned, rho);
+    rdm_unpack(static_cast<int>(op.q), op.qubits, pinned + F, rho);
     N = 0.0;
     for (int b = 0; b < D; ++b) N += rho[2 * (b * D + b)];
     for (uint32_t i = 0; i < op.num_ops; ++i) {
@@ -807,6 +849,7 @@ struct Controller {
   qt_status finish_trajectory(uint32_t t, const float2* psi, uint64_t* d_samples) {
     qt_status s = measure(t, psi, d_samples);
     if (s == QT_OK) s = collect_timing();
+    if (s == QT_OK) s = pass_device_error();
     return s;
   }
 

@@ -16,19 +16,14 @@ thread_local Config pushed;
 std::map<const void*, std::string> kernel_names;
 std::string launches;                       // "name grid block smem" lines
 std::string fail_kernel, set_kernel;
-size_t set_offset = 0;
+int* flag = nullptr;                        // the last int cleared on the device
 cudaError_t last_error = cudaSuccess;
 
-cudaError_t launch(const void* kernel, dim3 grid, dim3 block, size_t smem, void** args) {
+cudaError_t launch(const void* kernel, dim3 grid, dim3 block, size_t smem) {
   const std::string& name = kernel_names[kernel];
   launches += name + " " + std::to_string(grid.x) + " " + std::to_string(block.x) + " " + std::to_string(smem) + "\n";
   if (!fail_kernel.empty() && name.find(fail_kernel) != std::string::npos) return last_error = cudaErrorLaunchOutOfResources;
-  // a device word that the kernel would set: a pointer inside its parameter block
-  if (!set_kernel.empty() && name.find(set_kernel) != std::string::npos) {
-    int* p;
-    std::memcpy(&p, static_cast<char*>(args[1]) + set_offset, sizeof(p));
-    *p = 1;
-  }
+  if (flag && !set_kernel.empty() && name.find(set_kernel) != std::string::npos) *flag = 1;
   return cudaSuccess;
 }
 
@@ -48,8 +43,8 @@ extern "C" {
 const char* fake_launches() { return launches.c_str(); }
 void fake_clear() { launches.clear(); }
 void fake_fail(const char* kernel) { fail_kernel = kernel; }
-// launches of `kernel` store 1 through the pointer at `offset` of their second parameter
-void fake_set(const char* kernel, size_t offset) { set_kernel = kernel; set_offset = offset; }
+// launches of `kernel` set the error flag, the last int that was cleared
+void fake_set(const char* kernel) { set_kernel = kernel; }
 
 void** __cudaRegisterFatBinary(void*) { return reinterpret_cast<void**>(token); }
 void __cudaRegisterFatBinaryEnd(void**) {}
@@ -73,14 +68,14 @@ cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* host) {
   *k = static_cast<cudaKernel_t>(const_cast<void*>(host));
   return cudaSuccess;
 }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3 block, void** args, size_t smem, cudaStream_t) {
-  return launch(k, grid, block, smem, args);
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3 block, void**, size_t smem, cudaStream_t) {
+  return launch(k, grid, block, smem);
 }
-cudaError_t cudaLaunchKernel(const void* k, dim3 grid, dim3 block, void** args, size_t smem, cudaStream_t) {
-  return launch(k, grid, block, smem, args);
+cudaError_t cudaLaunchKernel(const void* k, dim3 grid, dim3 block, void**, size_t smem, cudaStream_t) {
+  return launch(k, grid, block, smem);
 }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* k, void** args) {
-  return launch(k, c->gridDim, c->blockDim, c->dynamicSmemBytes, args);
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* k, void**) {
+  return launch(k, c->gridDim, c->blockDim, c->dynamicSmemBytes);
 }
 
 cudaError_t cudaGetLastError() { const cudaError_t e = last_error; last_error = cudaSuccess; return e; }
@@ -110,7 +105,11 @@ cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cu
   std::memcpy(d, s, n);
   return cudaSuccess;
 }
-cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t) { std::memset(d, v, n); return cudaSuccess; }
+cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t) {
+  if (n == sizeof(int)) flag = static_cast<int*>(d);
+  std::memset(d, v, n);
+  return cudaSuccess;
+}
 
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { return handle(s); }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }

@@ -19,7 +19,6 @@ import qtsynth as qs
 from paper_2111_02396_gb300.qt import QtError
 fake = ctypes.CDLL(os.environ["LD_PRELOAD"])
 fake.fake_launches.restype = ctypes.c_char_p
-fake.fake_set.argtypes = [ctypes.c_char_p, ctypes.c_size_t]
 qt.load()
 
 def launches(part=""):
@@ -108,4 +107,41 @@ def test_failed_launch_is_reported(child, kernel, call):
         raise AssertionError("the call returned a result")
     fake.fake_fail(b"")
     call()
+    """)
+
+
+@pytest.mark.parametrize("flushes,share,keep", [(False, False, False), (True, False, True), (True, True, False)])
+def test_timeout_flag_ends_a_run(child, flushes, share, keep):
+    """A tensor-core wait that ran out ends a run at the next stage-2 choice, or at the latest with the
+    eighth trajectory."""
+    child(f"""
+    n, T = 13, 40
+    c = qs.Circuit(n)
+    rng = np.random.default_rng(1)
+    for m in range(0, 12, 2):
+        q = sorted(int(x) for x in rng.choice(n, 6, replace=False))
+        c.gate(np.linalg.qr(rng.normal(size=(64, 64)) + 1j * rng.normal(size=(64, 64)))[0], tuple(q), m)
+        if {flushes}:
+            c.channel(qs.amplitude_damping(0.9), (q[0],), m + 1)
+    f = qt.Fused(qt.Circuit.from_synth(c), 6)
+    run = lambda t: qt.Run(f, t, seed=3, precision=qt.QT_TF32X3, share_prefix={share}, keep_states={keep})
+    run(1)
+    one = len(launches("k_apply_tc"))
+    fake.fake_clear()
+    st = run(T).stats()
+    assert len(launches("k_apply_tc")) > T
+    assert (st["prob_passes"] > 0) == {flushes}
+    fake.fake_clear()
+    fake.fake_set(b"k_apply_tc")
+    for t in (1, T):
+        try:
+            run(t)
+        except QtError as e:
+            assert e.status == qt.qt.QT_ERR_TIMEOUT
+        else:
+            raise AssertionError("the run returned")
+    got = len(launches("k_apply_tc"))                        # of t = 1 and of T
+    assert one > 2 and got <= (2 if {flushes} else 9) * one, (one, got)
+    fake.fake_set(b"")
+    run(2)
     """)
