@@ -457,7 +457,7 @@ void qt_server_destroy(qt_server* s);
  * memory -- e.g. an application that reserves all GPU memory for its own pool
  * at start-up, or a latency-critical loop that must not stall on cudaMalloc /
  * cudaFree).  Same arguments, result and precision as
- * qt_state_reduced_density; it calls no allocator of any kind.  Its FP64
+ * qt_state_reduced_density; it calls no allocator of any kind.  Its
  * scratch is one fixed array inside libqt.so: 1216 * 64 + 64 doubles
  * (608.5 KiB), which every GPU that loads the library holds until the process
  * exits; q must be <= 3 (larger requests are rejected with

@@ -37,6 +37,7 @@ struct Args {
   uint32_t ins[7];            // ascending bit positions to insert zeros at
   uint64_t num_sets, num_tiles;
   const float2* u;            // row-major matrix (device)
+  float down;                 // factor of the FP32 runs at their carry (norms)
 };
 
 // 16-byte word of (row m, sets 2 c, 2 c + 1) of a staged tile: the threads of
@@ -211,7 +212,7 @@ __global__ void __launch_bounds__(m64::kThreads, 2) k_norms64(const float2* __re
       }
       f[1] += row;
       if (++run == kNormRun) {
-        for (int k = 0; k < 2; ++k) { df_acc(h[k], l[k], f[k]); f[k] = 0.f; }
+        for (int k = 0; k < 2; ++k) { df_acc(h[k], l[k], f[k] * a.down); f[k] = 0.f; }
         run = 0;
       }
     }
@@ -219,7 +220,7 @@ __global__ void __launch_bounds__(m64::kThreads, 2) k_norms64(const float2* __re
   }
   if (set < m64::kSets) {
     for (int k = 0; k < 2; ++k) {
-      df_acc(h[k], l[k], f[k]);
+      df_acc(h[k], l[k], f[k] * a.down);
       float2 x = make_float2(h[k], l[k]);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) x = df_add(x, df_shfl_xor(x, o));
@@ -302,10 +303,11 @@ static cudaError_t norms64(const float2* psi, const m64::Args& a, float2* partia
   return cudaGetLastError();
 }
 
-cudaError_t launch_norms64(const float2* psi, int n, const uint32_t* qubits, const float2* kdev, float2* partial,
-                           int* blocks, cudaStream_t st) {
+cudaError_t launch_norms64(const float2* psi, int n, const uint32_t* qubits, const float2* kdev, float down,
+                           float2* partial, int* blocks, cudaStream_t st) {
   if (n < 6) return cudaErrorInvalidValue;
-  const m64::Args a = m64_args(n, qubits, kdev);
+  m64::Args a = m64_args(n, qubits, kdev);
+  a.down = down;
   return has_qubit0(qubits) ? norms64<true>(psi, a, partial, blocks, st) : norms64<false>(psi, a, partial, blocks, st);
 }
 

@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <mutex>
 
 #include "kernels.h"
@@ -172,6 +173,7 @@ struct RdmArgs {
   uint32_t ins[Q + 1];        // ascending bit positions to insert zeros at
   uint64_t num_groups;
   bool rev;                   // q = 2: the caller's members 1 and 2 are swapped
+  float down;                 // Scratch::down
 };
 
 constexpr int kRdmChunk = 16;     // sets summed in FP32 before the carry
@@ -206,7 +208,7 @@ __global__ void __launch_bounds__(kRdmThreads, Q == 1 && LOW0 ? 16 : 1) k_rdm(co
 #pragma unroll
     for (int t = 0; t < ST; ++t)
 #pragma unroll
-      for (int k = 0; k < W; ++k) { df_acc(h[k], l[k], f[t][k]); f[t][k] = 0.f; }
+      for (int k = 0; k < W; ++k) { df_acc(h[k], l[k], f[t][k] * a.down); f[t][k] = 0.f; }
   };
   const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x;
   auto load = [&](uint64_t g, float4 (&v)[NV]) {
@@ -282,6 +284,7 @@ static cudaError_t rdm_low(const float2* psi, int n, const uint32_t* qubits, con
                            cudaStream_t st) {
   RdmArgs<Q> a{};
   a.rev = Q == 2 && qubits[0] != s[0];
+  a.down = scr.down;
   int ni = 0;
   if (!LOW0) a.ins[ni++] = 0;
   for (int b = 0; b < Q; ++b) a.ins[ni++] = s[b];
@@ -314,6 +317,7 @@ struct Rdm3Args {
   uint64_t num_groups;
   int run;                    // sets summed in FP32 before the carry
   uint32_t rev;               // pairs in the other order: bits 0..5 within a half, 8 + 4 y + x of the corner
+  float down;                 // Scratch::down
 };
 
 constexpr int kRdm3Threads = 128;
@@ -338,7 +342,7 @@ __global__ void __launch_bounds__(kRdm3Threads, 4) k_rdm3(const float4* __restri
 #pragma unroll
     for (int k = 0; k < 32; ++k) {
       float2 c = carry[k][tid];
-      df_acc(c.x, c.y, f[k]);
+      df_acc(c.x, c.y, f[k] * a.down);
       carry[k][tid] = c;
       f[k] = 0.f;
     }
@@ -444,6 +448,7 @@ static cudaError_t rdm3_low(const float2* psi, int n, const uint32_t* s, uint32_
   a.num_groups = 1ull << (n - 3 - (LOW0 ? 0 : 1));
   a.run = carry_run(0.01, n - 3, kRdmChunk);
   a.rev = rev;
+  a.down = scr.down;
   static PerDevice grid_dev;
   const int grid = grid_dev.get([] {
     int occ = 0;
@@ -706,6 +711,22 @@ cudaError_t launch_rdm(const float2* psi, int n, int q, const uint32_t* qubits, 
   }
 }
 
+cudaError_t read_rdm(const float2* psi, int n, int q, const uint32_t* qubits, Scratch scr, cudaStream_t st, double* r) {
+  const int W = 1 << (2 * q);
+  for (;;) {
+    cudaError_t e = launch_rdm(psi, n, q, qubits, scr, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(r, scr.result, sizeof(double) * W, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return e;
+    if (scr.down != 1.f) {
+      for (int k = 0; k < W; ++k) r[k] /= scr.down;
+      return cudaSuccess;
+    }
+    if (std::all_of(r, r + W, [](double x) { return std::isfinite(x); })) return cudaSuccess;
+    scr.down = kRangeDown;
+  }
+}
+
 void rdm_unpack(int q, const uint32_t* qubits, const double* r, double* rho) {
   const int D = 1 << q;
   // basis index over `qubits` of basis index x over the sorted qubits
@@ -908,6 +929,7 @@ struct KrausArgs {
   uint32_t ins[Q];
   uint64_t num_sets;
   const float2* ops;            // G matrices 2^Q x 2^Q, row-major (basis bit b <-> qubits[b])
+  float down;                   // Scratch::down
 };
 
 template <int Q, int G>
@@ -959,12 +981,12 @@ __global__ void __launch_bounds__(kKrausThreads) k_kraus_norms(const float2* __r
     }
     if (++cnt == kKrausChunk) {
 #pragma unroll
-      for (int k = 0; k < W; ++k) { df_acc(ah[k], al[k], f[k]); f[k] = 0.f; }
+      for (int k = 0; k < W; ++k) { df_acc(ah[k], al[k], f[k] * a.down); f[k] = 0.f; }
       cnt = 0;
     }
   }
 #pragma unroll
-  for (int k = 0; k < W; ++k) df_acc(ah[k], al[k], f[k]);
+  for (int k = 0; k < W; ++k) df_acc(ah[k], al[k], f[k] * a.down);
   block_reduce_store<W>(ah, al, partial);
 }
 
@@ -986,6 +1008,7 @@ static cudaError_t kraus_norms_q(const float2* psi, int n, const uint32_t* qubit
   }
   a.num_sets = 1ull << (n - Q);
   a.ops = ops_dev;
+  a.down = scr.down;
   const size_t smem = sizeof(float2) * (static_cast<size_t>(G) * D * D + static_cast<size_t>(D) * kKrausThreads);
   static PerDevice setup;
   const int grid = setup.get([smem] {
@@ -1014,7 +1037,7 @@ cudaError_t launch_kraus_norms(const float2* psi, int n, int q, const uint32_t* 
     case 5: return kraus_norms_q<5, 4>(psi, n, qubits, ops_dev, scr, st);
     case 6: {                             // k_mat64.cu
       int g = 0;
-      const cudaError_t e = launch_norms64(psi, n, qubits, ops_dev, scr.partials(), &g, st);
+      const cudaError_t e = launch_norms64(psi, n, qubits, ops_dev, scr.down, scr.partials(), &g, st);
       return e != cudaSuccess ? e : finalize(scr.partials(), g, 2, scr.result, st);
     }
     default: return cudaErrorInvalidValue;
@@ -1028,6 +1051,7 @@ struct ExpArgs {
   uint64_t masks[kExpGroup];
   int nm;
   uint64_t num_pairs;
+  float down;                   // Scratch::down
 };
 
 constexpr int kExpChunk = 64;
@@ -1059,12 +1083,12 @@ __global__ void __launch_bounds__(kRedThreads) k_expect(const float2* __restrict
     }
     if (++cnt == kExpChunk) {
 #pragma unroll
-      for (int k = 0; k < W; ++k) { df_acc(ah[k], al[k], f[k]); f[k] = 0.f; }
+      for (int k = 0; k < W; ++k) { df_acc(ah[k], al[k], f[k] * a.down); f[k] = 0.f; }
       cnt = 0;
     }
   }
 #pragma unroll
-  for (int k = 0; k < W; ++k) df_acc(ah[k], al[k], f[k]);
+  for (int k = 0; k < W; ++k) df_acc(ah[k], al[k], f[k] * a.down);
   block_reduce_store<W>(ah, al, partial);
 }
 
@@ -1085,6 +1109,7 @@ struct ExpWArgs {
   uint32_t u[kExpGroup];        // mask bits (0, 6, 7, 8) as a 4-bit index
   int nm;
   uint64_t num_blocks;          // 2^(n - 9)
+  float down;                   // Scratch::down
 };
 
 constexpr int kExpWChunk = 8;
@@ -1146,12 +1171,12 @@ __global__ void __launch_bounds__(kRedThreads) k_expect_wht(const float2* __rest
     }
     if (++cnt == kExpWChunk) {
 #pragma unroll
-      for (int k = 0; k < W; ++k) { df_acc(ah[k], al[k], f[k]); f[k] = 0.f; }
+      for (int k = 0; k < W; ++k) { df_acc(ah[k], al[k], f[k] * a.down); f[k] = 0.f; }
       cnt = 0;
     }
   }
 #pragma unroll
-  for (int k = 0; k < W; ++k) df_acc(ah[k], al[k], f[k]);
+  for (int k = 0; k < W; ++k) df_acc(ah[k], al[k], f[k] * a.down);
   block_reduce_store<W>(ah, al, partial);
 }
 
@@ -1168,6 +1193,7 @@ cudaError_t launch_expect(const float2* psi, int n, int nm, const uint64_t* mask
     }
     a.nm = nm;
     a.num_blocks = 1ull << (n - 9);
+    a.down = scr.down;
     static PerDevice gridw_dev;
     const int gridw = gridw_dev.get([] { return red_grid(k_expect_wht, ~0ull >> 1); });
     const uint64_t need = (a.num_blocks * 32 + kRedThreads - 1) / kRedThreads;
@@ -1179,6 +1205,7 @@ cudaError_t launch_expect(const float2* psi, int n, int nm, const uint64_t* mask
   for (int m = 0; m < kExpGroup; ++m) a.masks[m] = m < nm ? masks[m] : 0;
   a.nm = nm;
   a.num_pairs = 1ull << (n - 1);
+  a.down = scr.down;
   static PerDevice grid_dev;
   const int grid = grid_dev.get([] { return red_grid(k_expect, ~0ull >> 1); });
   const uint64_t need = (a.num_pairs + kRedThreads - 1) / kRedThreads;

@@ -57,11 +57,17 @@ constexpr int kCdfChunkLog = 6, kCdfSubLog = 10, kCdfBlkLog = 16;
 inline uint64_t cdf_num_sub(int n) { return ((1ull << n) + (1ull << kCdfSubLog) - 1) >> kCdfSubLog; }
 inline uint64_t cdf_num_blk(int n) { return (cdf_num_sub(n) + 63) >> 6; }
 
+constexpr float kRangeDown = 0x1p-64f;    // 2^34 amplitudes of 2^127 stay finite
 struct Scratch {
   double* partial = nullptr;   // kPartialDoubles doubles (held as that many double-floats)
   double* result = nullptr;    // kResultDoubles doubles
   float* cdf_sub = nullptr;    // cdf_num_sub(n) floats
   double* cdf_cum = nullptr;   // cdf_num_blk(n) doubles
+  // factor of the FP32 runs at their carry (a power of two): the results of
+  // launch_rdm, launch_expect and launch_kraus_norms come out times it.
+  // Double-floats have FP32's range, so the sums of a caller's state of norm^2
+  // beyond 2^128 need kRangeDown
+  float down = 1.f;
   float2* partials() const { return reinterpret_cast<float2*>(partial); }
 };
 
@@ -72,6 +78,9 @@ cudaError_t launch_apply(float2* psi, int n, int k, const uint32_t* targets, con
 // rho (the 4^q reals that rdm_unpack takes) of qubits Q into scr.result
 cudaError_t launch_rdm(const float2* psi, int n, int q, const uint32_t* qubits, const Scratch& scr,
                        cudaStream_t st);
+// the same on the host (blocks), where a density beyond FP32's range is read
+// a second time with kRangeDown
+cudaError_t read_rdm(const float2* psi, int n, int q, const uint32_t* qubits, Scratch scr, cudaStream_t st, double* r);
 // Channels on 4 or 5 qubits, at least 2^kGramMinLog gather sets: P_i =
 // <psi|K_i^dag K_i|psi> of nops operators.  scratch (kraus_scratch_bytes(q,
 // nops) bytes of device memory, 16-byte aligned) begins with the results,
@@ -105,9 +114,9 @@ cudaError_t launch_cdf_values(const float2* psi, int n, const Scratch& scr, doub
 // 6-qubit fused gate on CUDA cores (FP32), matrix 64x64 row-major in device memory, n >= 13
 cudaError_t launch_apply6_fp32(float2* psi, int n, const uint32_t* targets, const float2* udev, cudaStream_t st);
 // per-block sums of |psi|^2 and |K psi|^2 (two double-floats a block) for one
-// 64 x 64 operator (basis bit b <-> qubits[b]), n >= 6
-cudaError_t launch_norms64(const float2* psi, int n, const uint32_t* qubits, const float2* kdev, float2* partial,
-                           int* blocks, cudaStream_t st);
+// 64 x 64 operator (basis bit b <-> qubits[b]), n >= 6, times `down`
+cudaError_t launch_norms64(const float2* psi, int n, const uint32_t* qubits, const float2* kdev, float down,
+                           float2* partial, int* blocks, cudaStream_t st);
 // multi-gate pass: up to kMultiGates fused gates (width <= 4, n >= 7 + width,
 // targets ascending, matrix row-major) whose qubits, with the lowest kMultiLow,
 // number at most kMultiBits, applied in order in one pass over the state;

@@ -81,11 +81,9 @@ extern "C" qt_status qt_state_reduced_density_noalloc(const void* state, uint32_
   scr.partial = scratch;
   scr.result = scratch + kPartialDoubles;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  cudaError_t e = launch_rdm(static_cast<const float2*>(state), static_cast<int>(n), static_cast<int>(q), qubits,
-                             scr, st);
   double r[kRdmMaxReals];
-  if (e == cudaSuccess) e = cudaMemcpyAsync(r, scr.result, sizeof(double) << (2 * q), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  const cudaError_t e = read_rdm(static_cast<const float2*>(state), static_cast<int>(n), static_cast<int>(q), qubits,
+                                 scr, st, r);
   if (e != cudaSuccess)
     return set_error(QT_ERR_CUDA, "qt_state_reduced_density_noalloc: %s", cudaGetErrorString(e));
   rdm_unpack(static_cast<int>(q), qubits, r, out);

@@ -141,7 +141,7 @@ struct WideChannel {
       const qt_status s = gram(psi, n, q, qubits, num_ops, K, P, N, st);
       if (s != QT_OK || todo.empty()) return s;
       double n2 = 0.0;
-      return direct(psi, n, q, qubits, K, P, &n2, st);
+      return direct(psi, n, q, qubits, K, P, std::isfinite(*N) ? &n2 : N, st);
     }
     for (uint32_t i = 0; i < num_ops; ++i) todo.push_back(i);
     return direct(psi, n, q, qubits, K, P, N, st);
@@ -168,13 +168,16 @@ struct WideChannel {
     QT_CUDA(launch_kraus_probs(psi, static_cast<int>(n), Q, qubits, nops, res, st), "Kraus probability kernel launch");
     QT_CUDA(cudaMemcpyAsync(rows.data(), res, d2h, cudaMemcpyDeviceToHost, st), "cudaMemcpyAsync(probabilities)");
     QT_CUDA(cudaStreamSynchronize(st), "cudaStreamSynchronize(probabilities)");
-    for (int i = 0; i < nops; ++i) {
-      const double* const r = rows.data() + static_cast<size_t>(i) * slices;
+    auto prob = [&](size_t i) {
       double s = 0.0;
-      for (int k = 0; k + 1 < slices; ++k) s += r[k];
-      if (i == static_cast<int>(num_ops)) *N = s;
-      else if (r[slices - 1] <= s) P[i] = s;
-      else todo.push_back(static_cast<uint32_t>(i));      // its terms cancel (or are NaN)
+      for (int k = 0; k + 1 < slices; ++k) s += rows[i * slices + k];
+      return s;
+    };
+    *N = prob(num_ops);
+    for (uint32_t i = 0; i < num_ops; ++i) {
+      P[i] = prob(i);
+      const double err = rows[static_cast<size_t>(i + 1) * slices - 1];
+      if (!(err <= P[i]) || !std::isfinite(*N)) todo.push_back(i);   // its terms cancel, or leave FP32's range
     }
     return QT_OK;
   }
@@ -202,14 +205,20 @@ struct WideChannel {
       }
       QT_CUDA(cudaMemcpyAsync(kd, ops.data(), sizeof(float2) * G * mat, cudaMemcpyHostToDevice, st),
               "cudaMemcpyAsync(Kraus operators)");
-      QT_CUDA(launch_kraus_norms(psi, static_cast<int>(n), Q, qubits, static_cast<int>(G), kd, scr, st),
-              "Kraus probability kernel launch");
-      QT_CUDA(cudaMemcpyAsync(rows.data(), scr.result, sizeof(double) * (G + 1), cudaMemcpyDeviceToHost, st),
-              "cudaMemcpyAsync(probabilities)");
-      QT_CUDA(cudaStreamSynchronize(st), "cudaStreamSynchronize(probabilities)");
       h2d += sizeof(float2) * G * mat;
-      d2h += sizeof(double) * (G + 1);
-      launches += 2;
+      for (scr.down = 1.f;; scr.down = kRangeDown) {      // again if the sums leave FP32's range
+        QT_CUDA(launch_kraus_norms(psi, static_cast<int>(n), Q, qubits, static_cast<int>(G), kd, scr, st),
+                "Kraus probability kernel launch");
+        QT_CUDA(cudaMemcpyAsync(rows.data(), scr.result, sizeof(double) * (G + 1), cudaMemcpyDeviceToHost, st),
+                "cudaMemcpyAsync(probabilities)");
+        QT_CUDA(cudaStreamSynchronize(st), "cudaStreamSynchronize(probabilities)");
+        d2h += sizeof(double) * (G + 1);
+        launches += 2;
+        const bool finite = std::all_of(rows.begin(), rows.end(), [](double x) { return std::isfinite(x); });
+        if (scr.down != 1.f)
+          for (double& x : rows) x /= scr.down;
+        if (finite || scr.down != 1.f) break;
+      }
       *N = rows[0];
       for (size_t j = 0; j < cnt; ++j) P[todo[g0 + j]] = rows[1 + j];
     }
@@ -1314,12 +1323,9 @@ qt_status qt_state_reduced_density(const void* state, uint32_t n, uint32_t q, co
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   ScratchBufs scr;
   if (!scr.alloc(1, st)) return set_error(QT_ERR_OUT_OF_MEMORY, "qt_state_reduced_density: scratch");
-  QT_CUDA(launch_rdm(static_cast<const float2*>(state), static_cast<int>(n), static_cast<int>(q), qubits, scr.s, st),
-          "qt_state_reduced_density");
   double r[kRdmMaxReals];
-  QT_CUDA(cudaMemcpyAsync(r, scr.s.result, sizeof(double) << (2 * q), cudaMemcpyDeviceToHost, st),
-          "cudaMemcpyAsync");
-  QT_CUDA(cudaStreamSynchronize(st), "cudaStreamSynchronize");
+  QT_CUDA(read_rdm(static_cast<const float2*>(state), static_cast<int>(n), static_cast<int>(q), qubits, scr.s, st, r),
+          "qt_state_reduced_density");
   rdm_unpack(static_cast<int>(q), qubits, r, out);
   return QT_OK;
 }
@@ -1341,12 +1347,9 @@ qt_status qt_state_kraus_probabilities(const void* state, uint32_t n, uint32_t q
   if (q <= kRdmMaxQ) {                     // P_i = tr(K_i^dag K_i rho) from the reduced density
     ScratchBufs scr;
     if (!scr.alloc(1, st)) return set_error(QT_ERR_OUT_OF_MEMORY, "qt_state_kraus_probabilities: scratch");
-    QT_CUDA(launch_rdm(static_cast<const float2*>(state), static_cast<int>(n), static_cast<int>(q), qubits, scr.s, st),
-            "qt_state_kraus_probabilities");
     double r[kRdmMaxReals], rho[2 * 64];
-    QT_CUDA(cudaMemcpyAsync(r, scr.s.result, sizeof(double) << (2 * q), cudaMemcpyDeviceToHost, st),
-            "cudaMemcpyAsync");
-    QT_CUDA(cudaStreamSynchronize(st), "cudaStreamSynchronize");
+    QT_CUDA(read_rdm(static_cast<const float2*>(state), static_cast<int>(n), static_cast<int>(q), qubits, scr.s, st, r),
+            "qt_state_kraus_probabilities");
     rdm_unpack(static_cast<int>(q), qubits, r, rho);
     *N = 0.0;
     for (int b = 0; b < D; ++b) *N += rho[2 * (b * D + b)];
@@ -1428,15 +1431,18 @@ qt_status qt_state_expect_z(const void* state, uint32_t n, uint32_t M, const uin
   for (uint32_t b0 = 0; b0 < G; b0 += batch) {
     const uint32_t nb = std::min(batch, G - b0);
     Scratch sc = scr.s;
-    for (uint32_t b = 0; b < nb; ++b) {
-      const uint32_t g0 = (b0 + b) * kExpGroup;
-      sc.result = scr.extra + per * b;
-      QT_CUDA(launch_expect(static_cast<const float2*>(state), static_cast<int>(n),
-                            static_cast<int>(std::min<uint32_t>(kExpGroup, M - g0)), masks + g0, sc, st),
-              "qt_state_expect_z");
+    for (sc.down = 1.f;; sc.down = kRangeDown) {   // again if the sums leave FP32's range
+      for (uint32_t b = 0; b < nb; ++b) {
+        const uint32_t g0 = (b0 + b) * kExpGroup;
+        sc.result = scr.extra + per * b;
+        QT_CUDA(launch_expect(static_cast<const float2*>(state), static_cast<int>(n),
+                              static_cast<int>(std::min<uint32_t>(kExpGroup, M - g0)), masks + g0, sc, st),
+                "qt_state_expect_z");
+      }
+      QT_CUDA(cudaMemcpyAsync(r.data(), scr.extra, sizeof(double) * per * nb, cudaMemcpyDeviceToHost, st), "cudaMemcpyAsync");
+      QT_CUDA(cudaStreamSynchronize(st), "cudaStreamSynchronize");
+      if (sc.down != 1.f || std::all_of(r.begin(), r.begin() + per * nb, [](double x) { return std::isfinite(x); })) break;
     }
-    QT_CUDA(cudaMemcpyAsync(r.data(), scr.extra, sizeof(double) * per * nb, cudaMemcpyDeviceToHost, st), "cudaMemcpyAsync");
-    QT_CUDA(cudaStreamSynchronize(st), "cudaStreamSynchronize");
     for (uint32_t m = b0 * kExpGroup; m < std::min(M, (b0 + nb) * kExpGroup); ++m) {
       const double* const g = r.data() + per * (m / kExpGroup - b0);
       out[m] = g[1 + m % kExpGroup] / g[0];
