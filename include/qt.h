@@ -319,11 +319,13 @@ typedef struct {
   uint32_t keep_states;        /* 1: keep final states for qt_batch_state */
   uint32_t use_graph;          /* replay the launch sequence as a CUDA graph (needs a stream) */
   uint32_t threads;            /* CTA size of trajectories whose states fit in shared memory
-                                  (n <= 14): 128, 256 or 512 (0 = 512), an upper bound: small
-                                  states take smaller CTAs, several per SM */
+                                  (n <= 14): 128, 256 or 512 (0 = 512), an upper bound: states
+                                  of up to 10 qubits take at most 128, of 11 to 13 at most 256,
+                                  several CTAs per SM.  It also fixes how sums over a state are
+                                  split, so results differ in their last bits between values */
   void* stream;                /* cudaStream_t */
-  uint32_t threads_global;     /* CTA size of trajectories whose states live in global memory
-                                  (n > 14): 128, 256 or 512 (0 = threads) */
+  uint32_t threads_global;     /* the same for trajectories whose states live in global memory
+                                  (n > 14): 128, 256 or 512 (0 = threads); CTAs of at most 256 */
 } qt_batch_params;
 
 /* Run one trajectory of every circuit of the batch (Alg. 2, the same draws
@@ -351,8 +353,9 @@ void qt_batch_destroy(qt_batch* b);
  * costs differ (the first is bound by latency and arithmetic, the second by
  * memory traffic), so each class is tuned on its own spread sample of at
  * most `sample` circuits (0 = 256): every fusion width kmin..kmax (<= 6) at
- * 128, 256 and 512 threads per CTA (warm-up + 2 timed runs).  best receives
- * the fastest width and CTA size of each class (a class absent from the
+ * 128, 256 and 512 threads per CTA (warm-up + 2 timed runs; values that
+ * launch CTAs of the same sizes are timed once and chosen as the largest of
+ * them).  best receives the fastest width and CTA size of each class (a class absent from the
  * batch keeps kmin and 512); table (optional, 2 * (kmax - kmin + 1) * 3
  * doubles) the mean ms per run, [(class * (kmax - kmin + 1) + k - kmin) * 3
  * + {128, 256, 512}], class 0 = shared memory, 1 = global memory. */

@@ -1705,6 +1705,13 @@ static cudaError_t launch_glob_class(uint32_t threads, const bt::Dev& d, uint32_
   return e;
 }
 
+// CTA size of class c where the caller asks for `threads`: the largest that
+// its kernel is built for (k_batch_smem, k_batch_glob)
+static uint32_t class_threads(int c, uint32_t threads) {
+  static constexpr uint32_t most[bt::kClasses] = {bt::kGlobThreads, 512, 256, 256, 128};
+  return std::min(threads, most[c]);
+}
+
 // One run's persistent launches, with tables, outputs and arena as d holds
 // them: the work counters are zeroed on s, then every class launches, the
 // first one present on s and the others on side streams forked from and
@@ -1733,10 +1740,10 @@ static cudaError_t launch_classes(qt_batch* b, const bt::Dev& d, uint32_t thread
     dc.wmat = b->wmat[c];
     if (c == 0) {
       dc.lthreads = threads_glob;
-      r = launch_glob_class(std::min<uint32_t>(threads_glob, bt::kGlobThreads), dc, b->top_n[c], st);
+      r = launch_glob_class(class_threads(c, threads_glob), dc, b->top_n[c], st);
     } else {
       dc.lthreads = threads;
-      const uint32_t tb = std::min(threads, c == 1 ? 512u : (c < 4 ? 256u : 128u));
+      const uint32_t tb = class_threads(c, threads);
       const size_t smem = smem_class_bytes(b->top_n[c], dc.wmat);
       const uint32_t amps = 1u << b->top_n[c];
       r = tb == 512   ? launch_smem_class(bt::k_batch_smem<512, 1>, tb, smem, dc, amps, st)
@@ -2022,22 +2029,34 @@ qt_status qt_batch_autotune(uint32_t num, const qt_circuit* const* circuits, uin
       s = qt_batch_create(ns, const_cast<const qt_fused* const*>(f.data()), &b);
       for (auto* x : f) qt_fused_destroy(x);
       if (s != QT_OK) return s;
-      for (int ti = 0; ti < 3; ++ti) {
-        qt_batch_params p{};
-        p.seed = 0x5eed;
-        p.samples_per_traj = 16;
-        p.threads = kThreadOpts[ti];
-        p.threads_global = kThreadOpts[ti];
-        p.stream = stream;
-        double ms = 0.0;
-        for (int rep = 0; rep < 3 && s == QT_OK; ++rep) {
-          p.first_traj = rep;
-          s = qt_batch_run(b, &p);
-          if (rep > 0) ms += b->device_ms;     // the first run is warm-up
+      // sizes that launch the same CTAs are timed once and stand for the largest
+      // of them: the value also fixes how sums are split, which noise is not to pick
+      double timed[3];
+      for (int ti = 2; ti >= 0; --ti) {
+        int same = -1;
+        for (int tj = ti + 1; tj < 3 && same < 0; ++tj) {
+          same = tj;
+          for (int c = 0; c < bt::kClasses; ++c)
+            if (b->count[c] && class_threads(c, kThreadOpts[ti]) != class_threads(c, kThreadOpts[tj])) same = -1;
         }
-        if (s != QT_OK) { qt_batch_destroy(b); return s; }
-        if (table) table[(cls * nk + (k - kmin)) * 3 + ti] = ms / 2.0;
-        if (ms < best_ms) {
+        double ms = 0.0;
+        if (same < 0) {
+          qt_batch_params p{};
+          p.seed = 0x5eed;
+          p.samples_per_traj = 16;
+          p.threads = kThreadOpts[ti];
+          p.threads_global = kThreadOpts[ti];
+          p.stream = stream;
+          for (int rep = 0; rep < 3 && s == QT_OK; ++rep) {
+            p.first_traj = rep;
+            s = qt_batch_run(b, &p);
+            if (rep > 0) ms += b->device_ms;     // the first run is warm-up
+          }
+          if (s != QT_OK) { qt_batch_destroy(b); return s; }
+        }
+        timed[ti] = same < 0 ? ms / 2.0 : timed[same];
+        if (table) table[(cls * nk + (k - kmin)) * 3 + ti] = timed[ti];
+        if (same < 0 && ms < best_ms) {
           best_ms = ms;
           if (cls == 0) { best->k_shared = k; best->threads_shared = kThreadOpts[ti]; }
           else { best->k_global = k; best->threads_global = kThreadOpts[ti]; }

@@ -145,3 +145,21 @@ def test_timeout_flag_ends_a_run(child, flushes, share, keep):
     fake.fake_set(b"")
     run(2)
     """)
+
+
+@pytest.mark.parametrize("sizes,distinct", [((8, 9, 10), 1), ((9, 11, 13), 2), ((9, 14), 3), ((15, 16), 2)])
+def test_autotuner_times_each_launch_once(child, sizes, distinct):
+    """Values of `threads` that launch the same CTAs are one choice, the largest of them: equal times
+    are not left to noise, which would pick how sums are split."""
+    child(f"""
+    cs = [qt.Circuit.from_synth(qs.chain_circuit(n, 3, n, dep1=1e-2)) for n in {sizes}]
+    best, table = qt.autotune_batch(cs, kmin=2, kmax=3)
+    cls = "global" if {sizes}[0] > 14 else "shared"
+    rows = [[table[(cls, k, t)] for t in (128, 256, 512)] for k in (2, 3)]
+    assert all(t > 0 for r in rows for t in r)
+    one = [x[2] for x in launches("k_batch")]
+    # 2 widths, {distinct} values, 3 runs of a launch for each class present
+    classes = len(set(14 if n == 14 else 13 if n == 13 else 12 if n > 10 else 10 for n in {sizes} if n <= 14)) or 1
+    assert len(one) == 2 * {distinct} * 3 * classes, (len(one), classes)
+    assert best["threads_" + cls] == 512            # every run takes 1 ms here: the first that was timed
+    """)
