@@ -40,6 +40,8 @@
 // n = 13: 0.92 -> 0.22, 0.52 -> 0.19, 0.39 -> 0.21.
 #include <cuda_runtime.h>
 
+#include <cstddef>
+
 #include "kernels.h"
 
 namespace qt {
@@ -68,6 +70,13 @@ struct alignas(16) Args {
   uint64_t swz;               // slot = l ^ nibble (l >> 4) & 15 (lanes differ: no table in the constant bank)
   int ng, bits, C;            // gates; tile bits; contiguous low bits of a row
 };
+// matrix entries come through 8- and 16-byte loads of the constant bank
+template <int CAP>
+constexpr bool kAligned = offsetof(Args<CAP>, ce) % 16 == 0 && offsetof(Args<CAP>, f) % 16 == 0 &&
+                          offsetof(Args<CAP>, poff) % 16 == 0 && offsetof(Args<CAP>, g) % 16 == 0 &&
+                          offsetof(Args<CAP>, swz) % 8 == 0 && sizeof(Args<CAP>) % 16 == 0;
+static_assert(sizeof(Gate) % 16 == 0 && kAligned<512> && kAligned<1024> && kAligned<kMultiEntries>);
+static_assert(sizeof(Args<kMultiEntries>) <= 32764);   // what a launch's parameters may hold
 
 __device__ __forceinline__ float2* slot(float2* sm, uint32_t bytes) {
   return reinterpret_cast<float2*>(reinterpret_cast<char*>(sm) + bytes);
