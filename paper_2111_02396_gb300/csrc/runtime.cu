@@ -294,10 +294,7 @@ struct Controller {
   }
   ~Controller() {
     if (pinned) cudaFreeHost(pinned);
-    if (err_host) {
-      cudaStreamSynchronize(R.st);          // a copy into it may be in flight on an error return
-      cudaFreeHost(err_host);
-    }
+    if (err_st) cudaStreamDestroy(err_st);
     if (err_ev) cudaEventDestroy(err_ev);
     for (auto e : ev) cudaEventDestroy(e);
   }
@@ -348,15 +345,16 @@ struct Controller {
   }
 
   // The error flag comes back with the results of every stage-2 read (whose
-  // choice would rest on a wrong state), and behind every fourth trajectory,
-  // where the host looks at the copy four trajectories later and so keeps
-  // planning ahead (16 of 17 qubits: 21.1 ms without, 21.9 with a look behind
-  // each).  Once the flag is set, waits give up at their first try.
+  // choice would rest on a wrong state), and every fourth trajectory the host
+  // reads it, on a stream of its own, when the fourth before is complete, and
+  // so keeps planning ahead (16 of 17 qubits: 21.1 ms without, 21.9 with a look
+  // behind each; a pinned word to copy to costs a run 0.2 ms).  Once the flag is
+  // set, waits give up at their first try.
   static constexpr uint32_t kErrEvery = 4;
   uint32_t finished = 0;                    // trajectories
   bool tc_used = false;
-  int* err_host = nullptr;
-  cudaEvent_t err_ev = nullptr;             // recorded behind the last copy into err_host
+  cudaStream_t err_st = nullptr;
+  cudaEvent_t err_ev = nullptr;             // recorded behind every fourth trajectory
 
   qt_status device_error(int e) const {
     if (tc_used && e) return set_error(QT_ERR_TIMEOUT, "tensor-core kernel: a bounded wait ran out (code %d)", e);
@@ -371,15 +369,17 @@ struct Controller {
   }
   qt_status pass_device_error() {           // behind a trajectory
     if (!tc_used || ++finished % kErrEvery) return QT_OK;
-    if (err_host) {
-      QT_CUDA(cudaEventSynchronize(err_ev), "cudaEventSynchronize(err)");
-      const qt_status s = device_error(*err_host);
-      if (s != QT_OK) return s;
-    } else {
+    if (!err_ev) {
       QT_CUDA(cudaEventCreateWithFlags(&err_ev, cudaEventDisableTiming), "cudaEventCreate");
-      QT_CUDA(cudaMallocHost(&err_host, sizeof(int)), "cudaMallocHost");
+    } else {
+      if (!err_st) QT_CUDA(cudaStreamCreateWithFlags(&err_st, cudaStreamNonBlocking), "cudaStreamCreate(err)");
+      int e = 0;
+      QT_CUDA(cudaEventSynchronize(err_ev), "cudaEventSynchronize(err)");
+      QT_CUDA(cudaMemcpyAsync(&e, R.scr.flag, sizeof(int), cudaMemcpyDeviceToHost, err_st), "cudaMemcpyAsync(err)");
+      QT_CUDA(cudaStreamSynchronize(err_st), "cudaStreamSynchronize(err)");
+      const qt_status s = device_error(e);
+      if (s != QT_OK) return s;
     }
-    QT_CUDA(cudaMemcpyAsync(err_host, R.scr.flag, sizeof(int), cudaMemcpyDeviceToHost, R.st), "cudaMemcpyAsync(err)");
     QT_CUDA(cudaEventRecord(err_ev, R.st), "cudaEventRecord(err)");
     return QT_OK;
   }
