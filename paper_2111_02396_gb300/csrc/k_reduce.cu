@@ -802,35 +802,33 @@ __device__ __forceinline__ void df_mul_acc(float2& acc, float xh, float xl, floa
 
 // block (x, i): 256 of the terms (eight b, entry a, row j) of operator i,
 // Re(k_ja sum_b rho[a][b] conj(k_jb)), summed into out[i * gridDim.x + x]; the
-// last block of an operator puts E_i there
+// last D^2 / 256 blocks of an operator put 256 terms each of E_i^2 there
 template <int Q>
 __global__ void __launch_bounds__(256) k_kraus_trace(const float4* rho, const float2* __restrict__ ops, double* out) {
   constexpr int D = 1 << Q;
   __shared__ float2 s_sum[8];
   cudaGridDependencySynchronize();
-  if (blockIdx.x == gridDim.x - 1) {
+  constexpr int TERMS = D * D * D / 8 / 256;             // blocks of P_i
+  if (blockIdx.x >= TERMS) {
     __shared__ double s_part[8];
     const float2* const K = ops + static_cast<size_t>(blockIdx.y) * D * D;
-    double s = 0.0;                                        // products of four factors would leave FP32's range
-    for (int e = threadIdx.x; e < D * D; e += 256) {
-      const int x = e % D, y = e / D;
-      float gr = 0.f, gi = 0.f;
+    const int e = (blockIdx.x - TERMS) * 256 + threadIdx.x, x = e % D, y = e / D;
+    float gr = 0.f, gi = 0.f;
 #pragma unroll 8
-      for (int r = 0; r < D; ++r) {
-        const float2 u = __ldg(K + r * D + x), v = __ldg(K + r * D + y);
-        gr = fmaf(u.x, v.x, fmaf(u.y, v.y, gr));
-        gi = fmaf(u.x, v.y, fmaf(-u.y, v.x, gi));
-      }
-      const double g = gr, h = gi;
-      s += (g * g + h * h) * (static_cast<double>(rho[x * (D + 1)].x) * static_cast<double>(rho[y * (D + 1)].x));
+    for (int r = 0; r < D; ++r) {
+      const float2 u = __ldg(K + r * D + x), v = __ldg(K + r * D + y);
+      gr = fmaf(u.x, v.x, fmaf(u.y, v.y, gr));
+      gi = fmaf(u.x, v.y, fmaf(-u.y, v.x, gi));
     }
+    const double g = gr, h = gi;                         // products of four factors would leave FP32's range
+    double s = (g * g + h * h) * (static_cast<double>(rho[x * (D + 1)].x) * static_cast<double>(rho[y * (D + 1)].x));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = s;
     __syncthreads();
     if (threadIdx.x == 0) {
       for (int w = 1; w < 8; ++w) s += s_part[w];
-      out[blockIdx.y * gridDim.x + blockIdx.x] = sqrt(s);
+      out[blockIdx.y * gridDim.x + blockIdx.x] = s;
     }
     return;
   }
@@ -862,7 +860,8 @@ __global__ void __launch_bounds__(256) k_kraus_trace(const float4* rho, const fl
   }
 }
 
-int kraus_slices(int q) { return (1 << (3 * q - 3)) / 256 + 1; }
+int kraus_error_slices(int q) { return (1 << (2 * q)) / 256; }
+int kraus_slices(int q) { return (1 << (3 * q - 3)) / 256 + kraus_error_slices(q); }
 
 // the result rows, padded so that the operators after them are 16-byte aligned
 size_t kraus_results(int q, int nops) { return (static_cast<size_t>(nops) * kraus_slices(q) + 1) & ~size_t(1); }

@@ -84,13 +84,15 @@ cudaError_t read_rdm(const float2* psi, int n, int q, const uint32_t* qubits, Sc
 // Channels on 4 or 5 qubits, at least 2^kGramMinLog gather sets: P_i =
 // <psi|K_i^dag K_i|psi> of nops operators.  scratch (kraus_scratch_bytes(q,
 // nops) bytes of device memory, 16-byte aligned) begins with the results,
-// nops x kraus_slices(q) doubles: row i ends with E_i, and the others sum to
-// P_i, which is only good if E_i <= P_i (see k_kraus_trace).  From
+// nops x kraus_slices(q) doubles: the last kraus_error_slices(q) of row i sum
+// to E_i^2 and the others to P_i, which is only good if E_i <= P_i (see
+// k_kraus_trace).  From
 // kraus_results(q, nops) doubles on come the operators as kraus_sort_columns writes them (K
 // row-major (re, im) FP64, basis bit b <-> qubits[b]; 4^q complex64 each)
 constexpr int kGramMinLog = 18;
 inline bool kraus_by_gram(int n, int q) { return q <= 5 && n - q >= kGramMinLog; }
 int kraus_slices(int q);
+int kraus_error_slices(int q);
 size_t kraus_results(int q, int nops);
 size_t kraus_scratch_bytes(int q, int nops);
 void kraus_sort_columns(int q, const uint32_t* qubits, const double* K, float2* out);

@@ -168,15 +168,16 @@ struct WideChannel {
     QT_CUDA(launch_kraus_probs(psi, static_cast<int>(n), Q, qubits, nops, res, st), "Kraus probability kernel launch");
     QT_CUDA(cudaMemcpyAsync(rows.data(), res, d2h, cudaMemcpyDeviceToHost, st), "cudaMemcpyAsync(probabilities)");
     QT_CUDA(cudaStreamSynchronize(st), "cudaStreamSynchronize(probabilities)");
-    auto prob = [&](size_t i) {
+    auto sum = [&](size_t i, int from, int to) {
       double s = 0.0;
-      for (int k = 0; k + 1 < slices; ++k) s += rows[i * slices + k];
+      for (int k = from; k < to; ++k) s += rows[i * slices + k];
       return s;
     };
-    *N = prob(num_ops);
+    const int terms = slices - kraus_error_slices(Q);
+    *N = sum(num_ops, 0, terms);
     for (uint32_t i = 0; i < num_ops; ++i) {
-      P[i] = prob(i);
-      const double err = rows[static_cast<size_t>(i + 1) * slices - 1];
+      P[i] = sum(i, 0, terms);
+      const double err = std::sqrt(sum(i, terms, slices));
       if (!(err <= P[i]) || !std::isfinite(*N)) todo.push_back(i);   // its terms cancel, or leave FP32's range
     }
     return QT_OK;
