@@ -1677,7 +1677,12 @@ static cudaError_t launch_smem_class(K kern, uint32_t threads, size_t smem, cons
 // trajectories enough to even out over the SMs, two below two per SM (240 of
 // 15 to 18 qubits: 17.6 ms with one, 12.1 with two, 14.4 with four, whose
 // smaller states have fewer tiles than the cluster has halves and whose
-// clusters leave SMs over), more where SMs would stay idle.
+// clusters leave SMs over), more where SMs would stay idle: up to four and
+// eight, in ms of at most two / four / eight CTAs (depth 24, k = 3),
+//   4 of 16 to 18 qubits  1.28 2.68 5.03 / 0.84 1.64 2.87 / 0.84 1.11 1.79
+//   4 of 20               20.9 / 11.2 / 6.3
+//   30 of 18              5.52 / 3.17 / 3.58 (19 clusters of eight fit)
+//   30 of 15 to 18        5.48 / 3.17 / 1.99
 static unsigned glob_cluster(uint32_t num, uint32_t top_n) {
   const uint32_t sms = static_cast<uint32_t>(sm_count());
   const unsigned most = std::min(8u, 1u << (top_n - bt::kTileBits - 1));   // at least a tile per half

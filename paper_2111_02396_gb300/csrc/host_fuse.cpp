@@ -10,7 +10,9 @@
 //   (2) the union of their qubits has at most f qubits.
 // Phase 1 only grows a by gates that share at least one qubit with it (the
 // paper's "nearest neighbours"); phase 2 then packs gates that are disjoint,
-// which still saves a full pass over the state per merge.  Channels are
+// which saves a fused gate per merge (a pass over the state where gates have
+// one each; gates of width <= 4 that fit a tile share theirs, k_multi.cu).
+// Channels are
 // fused like gates of their qubits ("slots"): the operator in a slot is
 // chosen per trajectory.  Which candidate a grows by is a choice the paper
 // leaves open: two rules are run (most shared qubits; most later gates
@@ -94,9 +96,10 @@ bool grow(std::vector<Work>& g, size_t a, int kmax, uint64_t all_mask, bool allo
   }
 }
 
-// relative device time of one pass of a fused gate of width w (measured
-// rates of the fused-gate kernels at 30 qubits: 6.5 TB/s up to width 3,
-// 5.9 at width 4, and 4.5 and 3.9 for the tensor-core kernel at widths 5, 6)
+// relative device time of a fused gate of width w in a pass of its own
+// (measured rates of the fused-gate kernels at 30 qubits: 6.5 TB/s up to width
+// 3, 5.9 at width 4, and 4.5 and 3.9 for the tensor-core kernel at widths 5,
+// 6).  Passes that several gates share are not modelled.
 double pass_cost(int w) {
   static const double c[7] = {1.0, 1.0, 1.0, 1.0, 1.1, 1.45, 1.7};
   return c[w < 7 ? w : 6];

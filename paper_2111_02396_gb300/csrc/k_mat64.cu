@@ -44,12 +44,12 @@ struct Args {
 // a quarter-warp that write together differ in m / 2 mod 8
 __device__ __forceinline__ int word(int m, int c) { return m * (kSets / 2) + (c ^ ((m >> 1) & 7)); }
 
-// LOW0: qubit 0 is a target, so a 16-byte word of the state holds the two
-// members of a set that differ in it; otherwise one member of two neighbouring
-// sets
 // x with a zero inserted at bit z
 __host__ __device__ __forceinline__ int skip(int x, int z) { return ((x >> z) << (z + 1)) | (x & ((1 << z) - 1)); }
 
+// LOW0: qubit 0 is a target, so a 16-byte word of the state holds the two
+// members of a set that differ in it; otherwise one member of two neighbouring
+// sets
 template <bool LOW0>
 struct Tile {
   static constexpr int NI = LOW0 ? 6 : 7, LOGJ = LOW0 ? 7 : 6;

@@ -26,16 +26,16 @@
 //     loaded once for all of them.  The FMAs are scalar: they take an entry
 //     from its uniform register however often it is used, where a packed FMA
 //     takes a pair of them only once and otherwise wants it moved to registers
-//     (n = 28, packed and scalar: 2 qubits 58.8 and 51.8 ms, 3 qubits 60.4 and
-//     46.8).  64 threads with 4 sets of 4 qubits need 15% fewer instructions
-//     but leave 8 warps an SM: 51.8 ms for 45.2.
-// Bound by issue (82% of the slots with 4-qubit gates, 59% of them FMAs) rather
+//     (n = 28, packed and scalar: 2 qubits 58.8 and 51.0 ms, 3 qubits 60.4 and
+//     45.7).  64 threads with 4 sets of 4 qubits need 15% fewer instructions
+//     but leave 8 warps an SM: 51.8 ms for 44.6.
+// Bound by issue (85-89% of the slots with 4-qubit gates, 59% of them FMAs) rather
 // than HBM from two gates a pass on.  Grouping pays at every size, so whatever
 // fits is grouped.  Device time of a grid circuit, one pass a gate -> grouped,
 // fused to at most 2, 3 and 4 qubits (in ms; n = 28: 211, 121 and 70 gates in
 // 47, 46 and 33 passes):
 //   n = 28   129 -> 51.0   79.6 -> 45.7   51.4 -> 44.6
-//   n = 20  1.57 -> 0.60   0.97 -> 0.49   0.69 -> 0.49
+//   n = 20  1.57 -> 0.55   0.97 -> 0.46   0.69 -> 0.45
 // and of 200 gates on random qubits, n = 26: 15.4 -> 5.8, 9.3 -> 4.9, 7.1 -> 6.0;
 // n = 13: 0.92 -> 0.22, 0.52 -> 0.19, 0.39 -> 0.21.
 #include <cuda_runtime.h>
