@@ -1349,9 +1349,10 @@ struct DevMem {
   bool alloc(size_t b) {
     if (p) cudaFree(p);
     p = nullptr;
-    bytes = b;
+    bytes = 0;                               // until there is memory: callers keep a buffer that is large enough
     if (b == 0) return true;
     if (cudaMalloc(&p, b) != cudaSuccess) { cudaGetLastError(); p = nullptr; return false; }
+    bytes = b;
     return true;
   }
 };
@@ -1858,9 +1859,12 @@ qt_status qt_batch_run(qt_batch* b, const qt_batch_params* p) {
     int sms = sm_count();
     const uint64_t slot = b->max_n > static_cast<uint32_t>(bt::kSmemNMax) ? (1ull << b->max_n) : 0;
     const uint64_t arena_amps = b->keep ? b->total_amps : slot * sms;
-    if (!b->arena.alloc(sizeof(float2) * arena_amps))
+    if (!b->arena.alloc(sizeof(float2) * arena_amps)) {
+      b->outs.alloc(0);                      // no layout: the next run lays out again
+      b->keep = 0;
       return set_error(QT_ERR_OUT_OF_MEMORY, "qt_batch_run: state arena (%llu amplitudes)",
                        static_cast<unsigned long long>(arena_amps));
+    }
     d.arena = static_cast<float2*>(b->arena.p);
     d.slot_amps = slot;
     d.keep = b->keep;

@@ -69,13 +69,13 @@ struct DevBuf {
       a = g_alloc;
     }
     st = s;
-    bytes = b;
     if (a.alloc) {
       p = a.alloc(b, s, a.ctx);
     } else if (cudaMallocAsync(&p, b, s) != cudaSuccess) {
       cudaGetLastError();
       p = nullptr;
     }
+    bytes = p ? b : 0;
     return p != nullptr;
   }
   void release() {

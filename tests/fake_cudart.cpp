@@ -18,6 +18,8 @@ std::string launches;                       // "name grid block smem" lines
 std::string fail_kernel, set_kernel;
 int* flag = nullptr;                        // the last int cleared on the device
 cudaError_t last_error = cudaSuccess;
+size_t fail_bytes = 0;                      // the next fail_count allocations of that many bytes or more fail
+int fail_count = 0;
 
 cudaError_t launch(const void* kernel, dim3 grid, dim3 block, size_t smem) {
   const std::string& name = kernel_names[kernel];
@@ -28,7 +30,12 @@ cudaError_t launch(const void* kernel, dim3 grid, dim3 block, size_t smem) {
 }
 
 cudaError_t allocate(void** p, size_t n) {
+  if (fail_count > 0 && n >= fail_bytes) {
+    --fail_count;
+    return last_error = cudaErrorMemoryAllocation;
+  }
   *p = std::aligned_alloc(256, (n + 511) & ~static_cast<size_t>(255));
+  if (*p && n < (size_t{1} << 24)) std::memset(*p, 0, n);
   return *p ? cudaSuccess : cudaErrorMemoryAllocation;
 }
 
@@ -43,6 +50,7 @@ extern "C" {
 const char* fake_launches() { return launches.c_str(); }
 void fake_clear() { launches.clear(); }
 void fake_fail(const char* kernel) { fail_kernel = kernel; }
+void fake_fail_alloc(size_t bytes, int count) { fail_bytes = bytes; fail_count = count; }
 // launches of `kernel` set the error flag, the last int that was cleared
 void fake_set(const char* kernel) { set_kernel = kernel; }
 

@@ -19,6 +19,7 @@ import qtsynth as qs
 from paper_2111_02396_gb300.qt import QtError
 fake = ctypes.CDLL(os.environ["LD_PRELOAD"])
 fake.fake_launches.restype = ctypes.c_char_p
+fake.fake_fail_alloc.argtypes = [ctypes.c_size_t, ctypes.c_int]
 qt.load()
 
 def launches(part=""):
@@ -162,4 +163,47 @@ def test_autotuner_times_each_launch_once(child, sizes, distinct):
     classes = len(set(14 if n == 14 else 13 if n == 13 else 12 if n > 10 else 10 for n in {sizes} if n <= 14)) or 1
     assert len(one) == 2 * {distinct} * 3 * classes, (len(one), classes)
     assert best["threads_" + cls] == 512            # every run takes 1 ms here: the first that was timed
+    """)
+
+
+def test_lane_after_an_allocation_failure(child):
+    """The batch lane keeps its buffers between launches; a request that is deferred because they could
+    not grow is launched with buffers of its size."""
+    child("""
+    f = qt.Fused(qt.Circuit.from_synth(qs.chain_circuit(9, 6, 1, dep1=1e-2)), 3)
+    srv = qt.Server(1 << 33, max_slots=1, small_n_max=14)
+    for samples, fails in ((10, 0), (4000, 1), (16000, 2)):
+        fake.fake_clear()
+        fake.fake_fail_alloc(64 * samples * 8, fails)
+        i = srv.submit(f, seed=1, num_traj=64, samples_per_traj=samples)
+        srv.wait(i, timeout_s=60)
+        smp, inf = srv.result(i)
+        assert smp.shape == (64, samples) and not smp.any()
+        assert len(launches("k_batch_smem")) == 1
+    srv.close()
+    """)
+
+
+@pytest.mark.parametrize("keep", [False, True])
+def test_batch_after_an_allocation_failure(child, keep):
+    """A run whose state arena cannot be had launches nothing, and neither does the next one."""
+    child(f"""
+    f = [qt.Fused(qt.Circuit.from_synth(qs.chain_circuit(n, 4, n, dep1=1e-2)), 3) for n in (16, 9)]
+    b = qt.Batch(f)
+    args = dict(seed=1, samples_per_traj=5, keep_states={keep})
+    for first in (None, dict(seed=1, samples_per_traj=4)):
+        if first:
+            b.run(**first)                      # a layout that the next run replaces
+        fake.fake_clear()
+        fake.fake_fail_alloc(1 << 18, 2)
+        for _ in range(2):
+            try:
+                b.run(**args)
+            except QtError as e:
+                assert e.status == qt.qt.QT_ERR_OUT_OF_MEMORY
+            else:
+                raise AssertionError("the run returned")
+        assert not launches("k_batch")
+        b.run(**args)
+        assert len(launches("k_batch")) == 2
     """)
